@@ -51,8 +51,19 @@ enum Op : int32_t {
     OP_BACKWARD = 1,    // y = x * (x2 - rowsum(x * x2)): x = softmax output, x2 = its gradient
     OP_FORWARD_LONG = 2, // OP_FORWARD for plans with rows longer than a stage (two passes)
     OP_BACKWARD_LONG = 3, // OP_BACKWARD for plans with rows longer than half a stage (two passes)
-    OP_FORWARD_GROUP = 4 // OP_FORWARD of rows split over groups of CTAs (one read; see KernelArgs)
+    OP_FORWARD_GROUP = 4, // OP_FORWARD of rows split over groups of CTAs (one read; see KernelArgs)
+    OP_FORWARD_TEAM = 5  // OP_FORWARD for plans with rows that teams of warps share (past kLaneRowBytes)
 };
+
+// Rows of more bytes than this (up to a stage) are shared by a team of 1 to 16
+// warps, in a kernel instance of its own so that the routines of shorter rows
+// do not pay its registers.  One warp per row with three sweeps over shared
+// memory (before) against teams, GB/s over 256 MiB of rows: bf16 4 KiB 5885 ->
+// 6800, 16 KiB 4880 -> 6720, 64 KiB 1970 -> 6700, 113 KiB 1413 -> 6480; fp32
+// 16 KiB 6450 -> 6690, 64 KiB 3050 -> 6750, 113 KiB 2245 -> 6560.  What
+// bounded the old routines: a stage of one 64 KiB row left 3 of 16 warps
+// busy, each on a serial chain of shared loads.
+constexpr int kLaneRowBytes = 2048;
 
 // Rows split over groups of CTAs (OP_FORWARD_GROUP): group g is CTAs
 // [g*K, g*K + K); its rank-0 CTA claims rows and announces them in the

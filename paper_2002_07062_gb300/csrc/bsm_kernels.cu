@@ -17,10 +17,9 @@
 // The maximum and the sum are per vector (a balanced tree), per lane in vector
 // order, then a butterfly (xor) shuffle tree over the group.  By row length in
 // 16-byte vectors: <= 8: T = 8, 1 vector per lane; <= 16: T = 8, 2; <= 32:
-// T = 8, 4; <= 64: T = 16, 4; <= 128: T = 32, 4; fp32 <= 256: T = 32, 8 -- all
-// in registers (at most 32 elements per lane); longer fp32 rows: one warp,
-// exponentials written back in place in shared memory; longer bf16 rows: one
-// warp, three sweeps over shared memory (max, sum, write).  exp(t) is evaluated as 2^(t*log2 e) with
+// T = 8, 4; <= 64: T = 16, 4; <= 128: T = 32, 4 -- all in registers (at most
+// 32 elements per lane); longer rows: a team of 1 to 16 warps, up to 8 vectors
+// per lane in registers (see row_team).  exp(t) is evaluated as 2^(t*log2 e) with
 // the exponent formed by one fused multiply-add, v*log2e - m*log2e, and the
 // power of two from the PTX ex2.approx instruction; y = p * (1/sum).
 //
@@ -40,6 +39,11 @@ namespace {
 constexpr uint64_t kWaitLimitNs = 2000000000ull;   // 2 s
 constexpr uint32_t kClaimAhead = 2;                 // rows a group's rank 0 announces ahead
 constexpr float kLog2e = 1.4426950408889634f;
+
+// Teams of consumer warps that share a row: 8 of 2 warps, 4 of 4, 2 of 8, or
+// all 16 (whose barrier is xwarp).
+constexpr int kTeamBars = 14;
+constexpr int kTeamVecs = 8;        // 16-byte vectors a lane holds in registers
 
 enum : int32_t { KIND_DATA = 0, KIND_SKIP = 1, KIND_DONE = 2, KIND_LONG = 3, KIND_GROUP = 4 };
 
@@ -65,11 +69,14 @@ static_assert(sizeof(StageMeta) == 64, "StageMeta layout");
 struct SmemHeader {
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
-    uint64_t xwarp;                 // long rows: the consumer warps' partials are in
-    uint32_t xarrive[2];            // rows over groups: warps whose partial is in, by row parity
-    StageMeta meta[kMaxStages];
-    float2 partial[2][kConsumerWarps];   // long rows: (max, sum) per warp, two rows deep
+    union {
+        uint64_t xwarp;             // long rows, rows on 16 warps: the warps' partials are in
+        uint32_t xarrive[2];        // rows over groups: warps whose partial is in, by row parity
+    };
+    uint64_t team[kTeamBars];       // rows shared by a team of warps: its partials are in
     int32_t abort_flag;
+    StageMeta meta[kMaxStages];
+    float2 partial[2][kConsumerWarps];   // (max, sum) per warp of a row they share, two rows deep
 };
 static_assert(sizeof(SmemHeader) <= kSmemHeader, "header too large");
 
@@ -157,6 +164,34 @@ __device__ __noinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity,
     return false;
 }
 
+// The same wait without the call and without sleeping: for the short waits of
+// warps that share a row, which they hold in registers across it (a call
+// would spill them).  The clock is read once in 1024 polls.
+__device__ __forceinline__ bool mbar_spin_bounded(uint64_t *bar, uint32_t parity, const volatile int32_t *abort,
+                                                  uint64_t limit_ns)
+{
+    uint64_t t0 = 0;
+    for (uint32_t it = 0; it < (1u << 30); ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_addr(bar)), "r"(parity)
+            : "memory");
+        if (ok)
+            return true;
+        if ((it & 1023u) == 1023u) {
+            const uint64_t t = global_timer_ns();
+            t0 = t0 ? t0 : t;
+            if (*abort || t - t0 > limit_ns)
+                return false;
+        }
+    }
+    return false;
+}
+
 // 1-D bulk copy global -> shared, completion counted (bytes) on `bar`.
 __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
 {
@@ -167,8 +202,8 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
         : "memory");
 }
 
-// Stage reads and in-place writes are explicit shared-space accesses (a
-// 32-bit shared address), so they are issued as shared loads/stores whatever
+// Stage reads are explicit shared-space accesses (a
+// 32-bit shared address), so they are issued as shared loads whatever
 // the compiler can infer about the pointer; volatile keeps them on their side
 // of the barrier waits.
 __device__ __forceinline__ uint4 lds128(const unsigned char *p)
@@ -178,13 +213,6 @@ __device__ __forceinline__ uint4 lds128(const unsigned char *p)
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "r"(smem_addr(p)));
     return v;
-}
-
-__device__ __forceinline__ void sts128(unsigned char *p, uint4 v)
-{
-    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(smem_addr(p)), "r"(v.x), "r"(v.y),
-                 "r"(v.z), "r"(v.w)
-                 : "memory");
 }
 
 // Output stores: plain 128-bit global stores.
@@ -420,6 +448,44 @@ __device__ __forceinline__ void row_in_registers_scalar(const unsigned char *sro
 
 // ------------------------------------------------ fp32 pair arithmetic
 // One instruction, two IEEE operations, each rounded like its scalar form.
+// As 64-bit registers (Pair): a constant pair is made once, not at each use.
+typedef unsigned long long Pair;
+
+__device__ __forceinline__ Pair pair(float lo, float hi)
+{
+    Pair d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+
+__device__ __forceinline__ float2 halves(Pair p)
+{
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(p));
+    return d;
+}
+
+__device__ __forceinline__ Pair pair_fma(Pair a, Pair b, Pair c)
+{
+    Pair d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b)
+{
+    Pair d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+__device__ __forceinline__ Pair pair_mul(Pair a, Pair b)
+{
+    Pair d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
 {
     float2 d;
@@ -645,99 +711,221 @@ __device__ __forceinline__ void row_in_registers_pairs(const unsigned char *srow
     }
 }
 
-// Shared-memory-resident row of any length: one warp, three sweeps (max;
-// exponentials and their sum; exponentials again, scaled, stored).
-template <typename Tag, bool Checked>
-__device__ __forceinline__ void row_in_smem(const unsigned char *srow, unsigned char *yrow, int nvec,
-                                            int row, bool causal, int lane, const Bounds &bd)
+// The additive causal mask on a vector as loaded: x + (-inf) past the
+// diagonal (-inf, or NaN where x is NaN or +inf), x + (-0) = x elsewhere --
+// exact in the element type, so that what follows needs no mask.
+template <typename Tag> __device__ __forceinline__ uint4 mask_vec(uint4 r, int col0, int row);
+template <> __device__ __forceinline__ uint4 mask_vec<F32>(uint4 r, int col0, int row)
+{
+    if (col0 + 3 > row) {
+        r.x = __float_as_uint(__uint_as_float(r.x) + (col0 > row ? -INFINITY : -0.0f));
+        r.y = __float_as_uint(__uint_as_float(r.y) + (col0 + 1 > row ? -INFINITY : -0.0f));
+        r.z = __float_as_uint(__uint_as_float(r.z) + (col0 + 2 > row ? -INFINITY : -0.0f));
+        r.w = __float_as_uint(__uint_as_float(r.w) + (col0 + 3 > row ? -INFINITY : -0.0f));
+    }
+    return r;
+}
+template <> __device__ __forceinline__ uint4 mask_vec<BF16>(uint4 r, int col0, int row)
+{
+    if (col0 + 7 > row) {
+        uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t add = (col0 + 2 * k > row ? 0xFF80u : 0x8000u) |
+                                 (col0 + 2 * k + 1 > row ? 0xFF800000u : 0x80000000u);
+            asm("add.rn.bf16x2 %0, %0, %1;" : "+r"(w[k]) : "r"(add));
+        }
+        r = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    return r;
+}
+
+// Running maximum of a lane's vectors, NaN operands ignored: bf16 on the
+// packed words (exact), two halves; fp32 as a scalar.
+template <typename Tag> struct MaxAcc;
+template <> struct MaxAcc<F32> {
+    float m = -INFINITY;
+    __device__ __forceinline__ void add(uint4 r)
+    {
+        m = fmaxf(m, fmaxf(fmaxf(__uint_as_float(r.x), __uint_as_float(r.y)),
+                           fmaxf(__uint_as_float(r.z), __uint_as_float(r.w))));
+    }
+    __device__ __forceinline__ float get() const { return m; }
+};
+template <> struct MaxAcc<BF16> {
+    uint32_t w = 0xFF80FF80u;
+    __device__ __forceinline__ void add(uint4 r) { w = bmax2(w, bmax2(bmax2(r.x, r.y), bmax2(r.z, r.w))); }
+    __device__ __forceinline__ float get() const
+    {
+        return fmaxf(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+    }
+};
+
+// The exponents' offset for a maximum m: m * log2 e, no lower than the lowest
+// float.  At that floor (m = -inf, or a mask of the type's lowest value in
+// every element seen) v*log2e - offset is -inf or far below 0 and adds 0 (NaN
+// for a NaN), where m * log2 e = -inf would give inf - inf.
+__device__ __forceinline__ float exp_offset(float m) { return fmaxf(m * kLog2e, -3.402823466e38f); }
+
+// Element pair k of a vector as loaded.
+template <typename Tag> __device__ __forceinline__ Pair vec_pair(uint4 r, int k);
+template <> __device__ __forceinline__ Pair vec_pair<F32>(uint4 r, int k)
+{
+    return k == 0 ? pair(__uint_as_float(r.x), __uint_as_float(r.y)) : pair(__uint_as_float(r.z), __uint_as_float(r.w));
+}
+template <> __device__ __forceinline__ Pair vec_pair<BF16>(uint4 r, int k)
+{
+    const uint32_t w = k == 0 ? r.x : k == 1 ? r.y : k == 2 ? r.z : r.w;
+    return pair(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+}
+
+__device__ __forceinline__ Pair pair_ex2(Pair t)
+{
+    const float2 f = halves(t);
+    return pair(ex2(f.x), ex2(f.y));
+}
+
+// acc + the vector's 2^(v*log2e - mL), pair by pair (nm = -mL twice).
+template <typename Tag> __device__ __forceinline__ Pair vec_sum(Pair acc, uint4 r, Pair l2, Pair nm)
+{
+    constexpr int N = Elem<Tag>::kPerVec / 2;
+    Pair p[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        p[k] = pair_ex2(pair_fma(vec_pair<Tag>(r, k), l2, nm));
+#pragma unroll
+    for (int w = 1; w < N; w *= 2)
+#pragma unroll
+        for (int k = 0; k < N; k += 2 * w)
+            p[k] = pair_add(p[k], p[k + w]);
+    return pair_add(acc, p[0]);
+}
+
+// 2^(v*log2e - mL) * inv of one vector, packed.
+template <typename Tag> __device__ __forceinline__ uint4 vec_softmax(uint4 r, Pair l2, Pair nm, Pair inv2)
+{
+    constexpr int N = Elem<Tag>::kPerVec / 2;
+    float2 y[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        y[k] = halves(pair_mul(pair_ex2(pair_fma(vec_pair<Tag>(r, k), l2, nm)), inv2));
+    if constexpr (Elem<Tag>::kSize == 4)
+        return make_uint4(__float_as_uint(y[0].x), __float_as_uint(y[0].y), __float_as_uint(y[1].x),
+                          __float_as_uint(y[1].y));
+    else
+        return make_uint4(pack_bf16x2(y[0].x, y[0].y), pack_bf16x2(y[1].x, y[1].y), pack_bf16x2(y[2].x, y[2].y),
+                          pack_bf16x2(y[N - 1].x, y[N - 1].y));
+}
+
+// Maximum over the warp, in every lane (no operand is NaN: see MaxAcc).
+__device__ __forceinline__ float warp_max(float m)
+{
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(m));
+    return r;
+}
+
+// A row shared by a team of W consumer warps (wi = this warp's index in it;
+// W = 1, 2, 4, 8 or 16): lane l of warp wi owns the vectors wi*32 + l, + 32 W,
+// ..., V of them in registers (V = 6 or 8: more than 4 exist, so only the last two can be
+// missing in some lanes; 8 hold the whole row up to W * 4 KiB), further ones
+// (rows of 64 to 113 KiB on 16 warps) read again from the stage by each
+// sweep.  W and V are compile-time, so that no address outlives its use.  A warp takes its maximum's offset o_w (the rounded
+// m_w log2 e) and s_w, the sum of 2^(v log2 e - o_w); the team's warps
+// exchange (o_w, s_w) once (`part`: the team's slots) behind one bounded
+// barrier; every warp combines them in a fixed tree, S = sum s_w 2^(o_w - O),
+// and writes 2^(v log2 e - O) / S.  Taking the rounded offsets through the
+// exchange makes their rounding cancel in the quotient, as for a row of one
+// warp.  Two exponentials per element, one exchange per row.  All in fp32;
+// which warps share a row depends on its length only.
+//
+// release() is called once the warp needs the stage no more; returns false
+// when the exchange's wait gave up.
+template <typename Tag, bool Checked, int W, int V, typename Release>
+__device__ __forceinline__ bool row_team(const unsigned char *srow, unsigned char *yrow, int nvec, int row,
+                                         bool causal, int wi, int lane, const Bounds &bd, uint64_t *bar,
+                                         uint32_t parity, float2 *part, const volatile int32_t *abort,
+                                         uint64_t limit_ns, Release &&release)
 {
     using E = Elem<Tag>;
     constexpr int EPV = E::kPerVec;
-    float v[EPV];
-    uint4 raw;
-    float m = -INFINITY;
-    for (int vi = lane; vi < nvec; vi += 32) {
-        if (!load_vec<Checked>(srow + 16 * vi, bd, raw))
-            continue;
-        E::unpack(raw, v);
-        if (causal)
-            apply_causal<EPV>(v, vi * EPV, row);
-        m = fmaxf(m, tree_max<EPV>(v));
-    }
-    m = group_max<32>(m);
-    const float mL = m * kLog2e;
-    float s = 0.0f;
-    for (int vi = lane; vi < nvec; vi += 32) {
-        if (!load_vec<Checked>(srow + 16 * vi, bd, raw))
-            continue;
-        E::unpack(raw, v);
-        if (causal)
-            apply_causal<EPV>(v, vi * EPV, row);
-        vec_exp<EPV>(v, mL, causal && vi * EPV > row);
-        s += tree_sum<EPV>(v);
-    }
-    s = group_sum<32>(s);
-    const float inv = __frcp_rn(s);
-    for (int vi = lane; vi < nvec; vi += 32) {
-        if (!load_vec<Checked>(srow + 16 * vi, bd, raw))
-            continue;
-        E::unpack(raw, v);
-        if (causal)
-            apply_causal<EPV>(v, vi * EPV, row);
-        vec_exp<EPV>(v, mL, causal && vi * EPV > row);
+    constexpr int step = W * 32;
+    const int t0 = wi * 32 + lane;
+    const bool tail = W == 16 && V == kTeamVecs && nvec > V * step;
+    auto fetch = [&](int vi, bool in) -> uint4 {
+        uint4 r = E::neg_inf_vec();
+        if (in) {
+            uint4 u;
+            if (load_vec<Checked>(srow + 16 * vi, bd, u))
+                r = u;
+        }
+        return r;
+    };
+    uint4 r[V];
 #pragma unroll
-        for (int e = 0; e < EPV; ++e)
-            v[e] *= inv;
-        store_vec<Checked>(yrow + 16 * vi, bd, E::pack(v));
-    }
-}
-
-// fp32 rows of any length, two exponential-free sweeps: the second sweep
-// writes p = exp(v - m) back over the row in shared memory (same size as x),
-// the third scales it.  One exponential per element.  The proxy fence orders
-// these generic writes before the bulk copy that later refills the stage.
-template <bool Checked>
-__device__ __forceinline__ void row_in_smem_inplace(unsigned char *srow, unsigned char *yrow, int nvec,
-                                                    int row, bool causal, int lane, const Bounds &bd)
-{
-    using E = Elem<F32>;
-    constexpr int EPV = E::kPerVec;
-    float v[EPV];
-    uint4 raw;
-    float m = -INFINITY;
-    for (int vi = lane; vi < nvec; vi += 32) {
-        if (!load_vec<Checked>(srow + 16 * vi, bd, raw))
-            continue;
-        E::unpack(raw, v);
-        if (causal)
-            apply_causal<EPV>(v, vi * EPV, row);
-        m = fmaxf(m, tree_max<EPV>(v));
-    }
-    m = group_max<32>(m);
-    const float mL = m * kLog2e;
-    float s = 0.0f;
-    for (int vi = lane; vi < nvec; vi += 32) {
-        if (!load_vec<Checked>(srow + 16 * vi, bd, raw))
-            continue;
-        E::unpack(raw, v);
-        if (causal)
-            apply_causal<EPV>(v, vi * EPV, row);
-        vec_exp<EPV>(v, mL, causal && vi * EPV > row);
-        s += tree_sum<EPV>(v);
-        sts128(srow + 16 * vi, E::pack(v));
-    }
-    s = group_sum<32>(s);
-    const float inv = __frcp_rn(s);
-    for (int vi = lane; vi < nvec; vi += 32) {
-        if (!load_vec<Checked>(srow + 16 * vi, bd, raw))
-            continue;
-        E::unpack(raw, v);
+    for (int j = 0; j < V; ++j)
+        r[j] = fetch(t0 + j * step, j < V - 2 || t0 + j * step < nvec);
+    if (causal) {
 #pragma unroll
-        for (int e = 0; e < EPV; ++e)
-            v[e] *= inv;
-        store_vec<Checked>(yrow + 16 * vi, bd, E::pack(v));
+        for (int j = 0; j < V; ++j)
+            r[j] = mask_vec<Tag>(r[j], (t0 + j * step) * EPV, row);
     }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    auto fetch_tail = [&](int vi) -> uint4 {
+        const uint4 u = fetch(vi, true);
+        return causal ? mask_vec<Tag>(u, vi * EPV, row) : u;
+    };
+    MaxAcc<Tag> mx;
+#pragma unroll
+    for (int j = 0; j < V; ++j)
+        mx.add(r[j]);
+    if (tail)
+        for (int vi = t0 + V * step; vi < nvec; vi += step)
+            mx.add(fetch_tail(vi));
+    else
+        release();
+    float mL = exp_offset(warp_max(mx.get()));
+    const Pair l2 = pair(kLog2e, kLog2e);
+    Pair nm = pair(-mL, -mL), acc = pair(0.0f, 0.0f);
+#pragma unroll
+    for (int j = 0; j < V; ++j)
+        acc = vec_sum<Tag>(acc, r[j], l2, nm);
+    if (tail)
+        for (int vi = t0 + V * step; vi < nvec; vi += step)
+            acc = vec_sum<Tag>(acc, fetch_tail(vi), l2, nm);
+    const float2 a2 = halves(acc);
+    float s = group_sum<32>(a2.x + a2.y);
+    if (W > 1) {
+        if (lane == 0) {
+            part[wi] = make_float2(mL, s);
+            mbar_arrive(bar);
+        }
+        if (!__all_sync(0xFFFFFFFFu, mbar_spin_bounded(bar, parity, abort, limit_ns)))
+            return false;
+        const int k = lane & 15;
+        const float2 pw = k < W ? part[k] : make_float2(-INFINITY, 0.0f);
+        mL = warp_max(pw.x);
+        nm = pair(-mL, -mL);
+        s = group_sum<16>(pw.y * ex2(pw.x - mL));
+    }
+    const float inv = __frcp_rn(s);
+    const Pair inv2 = pair(inv, inv);
+    // the write unpacks the vectors again: kept unpacked from the sum on, they
+    // would take twice the registers (bf16) and spill
+#pragma unroll
+    for (int j = 0; j < V; ++j)
+        asm volatile("" : "+r"(r[j].x), "+r"(r[j].y), "+r"(r[j].z), "+r"(r[j].w));
+    unsigned char *yp = yrow + 16 * t0;
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        if (j < V - 2 || t0 + j * step < nvec)
+            store_vec<Checked>(yp + 16 * j * step, bd, vec_softmax<Tag>(r[j], l2, nm, inv2));
+    }
+    if (tail) {
+        for (int vi = t0 + V * step; vi < nvec; vi += step)
+            store_vec<Checked>(yrow + 16 * vi, bd, vec_softmax<Tag>(fetch_tail(vi), l2, nm, inv2));
+        release();
+    }
+    return true;
 }
 
 // ------------------------------------------------ backward row routines
@@ -1018,15 +1206,114 @@ __device__ __forceinline__ int rows_in_registers(const unsigned char *sbuf, cons
     return (mt.nrows + G - 1) / G;
 }
 
-// All rows of one stage that belong to this consumer warp.  The routine
+template <int N> struct Int {
+    static constexpr int value = N;
+};
+
+// Warps that share a row: the fewest whose registers hold it.
+__device__ __forceinline__ int team_warps(int nvec)
+{
+    return nvec <= 256 ? 1 : nvec <= 512 ? 2 : nvec <= 1024 ? 4 : nvec <= 2048 ? 8 : 16;
+}
+
+// A consumer warp's view of the exchanges it took part in: bit W (2, 4, 8, 16)
+// is the phase of its team of W (16: xwarp, long rows too), which is also
+// the half of SmemHeader::partial that the next one uses; the bits from
+// kTeamLast on hold the W of the last one.
+constexpr uint32_t kTeamLast = 8;
+
+// Rows of different team sizes share the partials' slots: before the size
+// changes, all consumer warps meet, so that none still reads the other
+// size's.  (Every warp sees the same stages, hence the same changes.)
+__device__ __forceinline__ bool team_switch(SmemHeader &h, uint32_t W, int lane, uint64_t limit_ns, uint32_t &xs)
+{
+    const uint32_t was = xs >> kTeamLast;
+    if (was == W)
+        return true;
+    xs = (xs & 0xFFu) | (W << kTeamLast);
+    if (was == 0)
+        return true;
+    __syncwarp();
+    if (lane == 0)
+        mbar_arrive(&h.xwarp);
+    const bool ok = mbar_spin_bounded(&h.xwarp, (xs >> 4) & 1u, &h.abort_flag, limit_ns);
+    xs ^= 16u;
+    return __all_sync(0xFFFFFFFFu, ok);
+}
+
+// The rows of one stage that teams of W warps share (see row_team), those of
+// this warp, dealt to the teams round robin after the `seen` warps' worth of
+// rows before.  Returns false when a wait gave up; release() is called
+// exactly once otherwise.
+template <typename Tag, bool Checked, int W, int V, typename Release>
+__device__ __forceinline__ bool rows_team(SmemHeader &h, const unsigned char *sbuf, const StageMeta &mt,
+                                          unsigned char *ybase, int row_bytes, int nvec, bool causal, uint32_t seen,
+                                          int warp, int lane, const Bounds &bd, uint64_t limit_ns,
+                                          uint32_t &xs, Release &&release)
+{
+    constexpr int teams = kConsumerWarps / W;
+    const int team = warp / W;
+    uint64_t *bar = W == 16 ? &h.xwarp : &h.team[(W == 8 ? 12 : W == 4 ? 8 : 0) + (W == 1 ? 0 : team)];
+    int r = static_cast<int>((team + teams - (seen / W) % teams) % teams);
+    int q = 0, qstep = 0;
+    if (causal) {
+        q = (mt.row0 + r) % mt.R;
+        qstep = teams % mt.R;
+    }
+    if (r >= mt.nrows)
+        release();
+    for (; r < mt.nrows; r += teams) {
+        const uint32_t par = (xs & W) ? 1u : 0u;
+        const bool last = r + teams >= mt.nrows;
+        if (!row_team<Tag, Checked, W, V>(sbuf + (size_t)r * row_bytes, ybase + (size_t)r * row_bytes, nvec, q, causal,
+                                       warp % W, lane, bd, bar, par, &h.partial[par][team * W], &h.abort_flag,
+                                       limit_ns, [&]() {
+                                           if (last)
+                                               release();
+                                       }))
+            return false;
+        if (W > 1)
+            xs ^= W;
+        q += qstep;
+        if (q >= mt.R)
+            q -= mt.R;
+    }
+    return true;
+}
+
+template <typename Tag, bool Checked, typename Release>
+__device__ __forceinline__ bool consume_stage_team(SmemHeader &h, const unsigned char *sbuf, const StageMeta &mt,
+                                                   unsigned char *y, bool causal, uint32_t seen, int warp, int lane,
+                                                   Bounds bd, uint64_t limit_ns, uint32_t &xs, Release &&release)
+{
+    const int row_bytes = mt.C * Elem<Tag>::kSize;
+    const int nvec = row_bytes >> 4;
+    unsigned char *yb = y + mt.off * Elem<Tag>::kSize;
+    bd.s_lo = sbuf;
+    bd.s_hi = sbuf + (size_t)mt.nrows * row_bytes;
+    const int W = team_warps(nvec);
+    if (W > 1 && !team_switch(h, W, lane, limit_ns, xs))
+        return false;
+    auto go = [&](auto w) {
+        constexpr int w_ = decltype(w)::value;
+        if (nvec <= 6 * 32 * w_)
+            return rows_team<Tag, Checked, w_, 6>(h, sbuf, mt, yb, row_bytes, nvec, causal, seen, warp, lane, bd,
+                                                  limit_ns, xs, release);
+        return rows_team<Tag, Checked, w_, kTeamVecs>(h, sbuf, mt, yb, row_bytes, nvec, causal, seen, warp, lane, bd,
+                                                      limit_ns, xs, release);
+    };
+    return W == 1 ? go(Int<1>{}) : W == 2 ? go(Int<2>{}) : W == 4 ? go(Int<4>{}) : W == 8 ? go(Int<8>{}) : go(Int<16>{});
+}
+
+// All rows of one stage that belong to this consumer warp, for rows that
+// one lane group's registers hold.  The routine
 // depends on the row length only (see the table at the top of the file).
 // Row groups are dealt round robin over the consumer warps starting at warp
 // `first`; the caller advances `first` by the returned group count, so a
 // stage with fewer groups than warps does not always land on the same warps.
 template <typename Tag, bool Checked>
-__device__ __forceinline__ int consume_stage(const unsigned char *sbuf, const StageMeta &mt,
-                                             unsigned char *y, bool causal, int first, int lane,
-                                             Bounds bd)
+__device__ __forceinline__ int consume_stage(const unsigned char *sbuf, const StageMeta &mt, unsigned char *y,
+                                             bool causal, int first, int lane, Bounds bd)
 {
     using E = Elem<Tag>;
     const int row_bytes = mt.C * E::kSize;
@@ -1041,35 +1328,8 @@ __device__ __forceinline__ int consume_stage(const unsigned char *sbuf, const St
     if (nvec <= 32)
         return rows_in_registers<Tag, Checked, 8, 4>(sbuf, mt, ybase, row_bytes, nvec, causal, first, lane, bd);
     if (nvec <= 64)
-        return rows_in_registers<Tag, Checked, 16, 4>(sbuf, mt, ybase, row_bytes, nvec, causal, first, lane,
-                                                      bd);
-    if (nvec <= 128)
-        return rows_in_registers<Tag, Checked, 32, 4>(sbuf, mt, ybase, row_bytes, nvec, causal, first, lane,
-                                                      bd);
-    // one warp per row from here on
-    int q = 0, qstep = 0;
-    if (causal) {
-        q = (mt.row0 + first) % mt.R;
-        qstep = kConsumerWarps % mt.R;
-    }
-    for (int r = first; r < mt.nrows; r += kConsumerWarps) {
-        const unsigned char *srow = sbuf + (size_t)r * row_bytes;
-        unsigned char *yrow = ybase + (size_t)r * row_bytes;
-        if constexpr (E::kSize == 4) {
-            // fp32: rows up to 4 KiB in registers, longer ones in place in the stage
-            if (nvec <= 256)
-                row_in_registers_scalar<Tag, Checked, 32, 8>(srow, yrow, nvec, q, causal, lane, true, bd);
-            else
-                row_in_smem_inplace<Checked>(const_cast<unsigned char *>(srow), yrow, nvec, q, causal, lane,
-                                             bd);
-        } else {
-            row_in_smem<Tag, Checked>(srow, yrow, nvec, q, causal, lane, bd);
-        }
-        q += qstep;
-        if (q >= mt.R)
-            q -= mt.R;
-    }
-    return mt.nrows;
+        return rows_in_registers<Tag, Checked, 16, 4>(sbuf, mt, ybase, row_bytes, nvec, causal, first, lane, bd);
+    return rows_in_registers<Tag, Checked, 32, 4>(sbuf, mt, ybase, row_bytes, nvec, causal, first, lane, bd);
 }
 
 // -------------------------------------------------------------- the schedule
@@ -1228,10 +1488,14 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
     // without long rows do not pay its registers
     constexpr bool kLong = Op == OP_FORWARD_LONG || Op == OP_BACKWARD_LONG;
     constexpr bool kBwd = Op == OP_BACKWARD || Op == OP_BACKWARD_LONG;
+    // likewise the rows that teams of warps share
+    constexpr bool kTeam = Op == OP_FORWARD_TEAM || Op == OP_FORWARD_LONG;
     extern __shared__ __align__(1024) unsigned char smem[];
     SmemHeader &h = *reinterpret_cast<SmemHeader *>(smem);
     unsigned char *stages = smem + kSmemHeader;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (broadcast for the teams: the compiler then knows that a warp's lanes agree)
+    const int warp = kTeam ? __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0) : threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     const int S = a.n_stages;
     const uint64_t wait_limit = a.wait_limit_ns ? a.wait_limit_ns : kWaitLimitNs;
 
@@ -1241,6 +1505,8 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
             mbar_init(&h.empty[s], kConsumerWarps);
         }
         mbar_init(&h.xwarp, kConsumerWarps);
+        for (int t = 0; t < kTeamBars; ++t)
+            mbar_init(&h.team[t], t < 8 ? 2 : t < 12 ? 4 : 8);
         h.abort_flag = 0;
         mbar_init_fence();
     }
@@ -1504,13 +1770,13 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
     // ----------------------------------------------------------- consumers
     const bool causal = (a.flags & BSM_FLAG_CAUSAL) != 0;
     unsigned char *y = static_cast<unsigned char *>(a.y);
-    uint32_t groups_seen = 0;   // row groups dealt so far (the same count in every warp)
+    uint32_t groups_seen = 0;   // warps' worth of rows dealt so far (the same count in every warp)
+    uint32_t xs = 0;            // the exchanges between warps so far (see kTeamLast)
     // long rows: this lane's running (max, sum); the row's final exponent
     // offset and reciprocal; which partial buffer and barrier phase is next
     float m_l = -INFINITY, s_l = 0.0f, long_mL = 0.0f, long_inv = 0.0f;
-    uint32_t long_rows = 0;
     uint32_t long_first_it = 0;  // stage iteration of the current row's first chunk
-    (void)m_l, (void)s_l, (void)long_mL, (void)long_inv, (void)long_rows;
+    (void)m_l, (void)s_l, (void)long_mL, (void)long_inv, (void)xs;
     for (uint32_t it = 0;; ++it) {
         const int s = it % S;
         const uint32_t ph = (it / S) & 1u;
@@ -1571,12 +1837,21 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
                         combine_ms(m_l, s_l, mo, so);
                     }
                 }
-                const int par = long_rows & 1;
+                if constexpr (kTeam) {
+                    if (!team_switch(h, 16, lane, wait_limit, xs)) {
+                        if (lane == 0) {
+                            atomicOr(a.status, BSM_DEV_TIMEOUT);
+                            h.abort_flag = 1;
+                        }
+                        break;
+                    }
+                }
+                const int par = (xs >> 4) & 1;
                 if (lane == 0) {
                     h.partial[par][warp] = make_float2(kBwd ? s_l : m_l, kBwd ? 0.0f : s_l);
                     mbar_arrive(&h.xwarp);
                 }
-                if (!mbar_wait_bounded(&h.xwarp, long_rows & 1u, &h.abort_flag, wait_limit)) {
+                if (!mbar_wait_bounded(&h.xwarp, par, &h.abort_flag, wait_limit)) {
                     if (lane == 0) {
                         atomicOr(a.status, BSM_DEV_TIMEOUT);
                         h.abort_flag = 1;
@@ -1636,16 +1911,34 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
                 }
                 m_l = -INFINITY;
                 s_l = 0.0f;
-                ++long_rows;
+                xs ^= 16u;
             }
             continue;
         }
         if (mt.kind == KIND_DATA) {
             Bounds bd{nullptr, nullptr, y, y + a.total_elems * E::kSize, a.status};
             const int64_t cap = kBwd ? a.stage_bytes / 2 : a.stage_bytes;
+            const int nvec = (mt.C * E::kSize) >> 4;
             if (Checked && (mt.nrows <= 0 || mt.C <= 0 || (int64_t)mt.nrows * mt.C * E::kSize > cap)) {
                 if (lane == 0)
                     check_fail(a.status, 4, static_cast<uint64_t>(mt.nrows), static_cast<uint64_t>(mt.C));
+            } else if (kTeam && nvec > kLaneRowBytes / 16) {
+                const bool ok = consume_stage_team<Tag, Checked>(
+                    h, stages + (size_t)s * a.stage_bytes, mt, y, causal, groups_seen, warp, lane, bd, wait_limit, xs,
+                    [&]() {
+                        __syncwarp();
+                        if (lane == 0)
+                            mbar_arrive(&h.empty[s]);
+                    });
+                if (!ok) {
+                    if (lane == 0) {
+                        atomicOr(a.status, BSM_DEV_TIMEOUT);
+                        h.abort_flag = 1;
+                    }
+                    break;
+                }
+                groups_seen += static_cast<uint32_t>(mt.nrows) * team_warps(nvec);
+                continue;                  // the stage is released
             } else {
                 const int first = static_cast<int>((warp + kConsumerWarps - groups_seen % kConsumerWarps) %
                                                    kConsumerWarps);
@@ -1653,8 +1946,8 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
                     groups_seen += consume_stage_bwd<Tag, Checked>(stages + (size_t)s * a.stage_bytes,
                                                                    a.stage_bytes / 2, mt, y, first, lane, bd);
                 else
-                    groups_seen += consume_stage<Tag, Checked>(stages + (size_t)s * a.stage_bytes, mt, y,
-                                                               causal, first, lane, bd);
+                    groups_seen += consume_stage<Tag, Checked>(stages + (size_t)s * a.stage_bytes, mt, y, causal,
+                                                               first, lane, bd);
             }
         }
         __syncwarp();
@@ -2200,9 +2493,13 @@ int kernel_set_smem_limit(int bytes)
 {
     const void *fns[] = {
         reinterpret_cast<const void *>(softmax_persistent<F32, OP_FORWARD, false>),
+        reinterpret_cast<const void *>(softmax_persistent<F32, OP_FORWARD_TEAM, false>),
         reinterpret_cast<const void *>(softmax_persistent<BF16, OP_FORWARD, false>),
+        reinterpret_cast<const void *>(softmax_persistent<BF16, OP_FORWARD_TEAM, false>),
         reinterpret_cast<const void *>(softmax_persistent<F32, OP_FORWARD, true>),
+        reinterpret_cast<const void *>(softmax_persistent<F32, OP_FORWARD_TEAM, true>),
         reinterpret_cast<const void *>(softmax_persistent<BF16, OP_FORWARD, true>),
+        reinterpret_cast<const void *>(softmax_persistent<BF16, OP_FORWARD_TEAM, true>),
         reinterpret_cast<const void *>(softmax_persistent<F32, OP_BACKWARD, false>),
         reinterpret_cast<const void *>(softmax_persistent<BF16, OP_BACKWARD, false>),
         reinterpret_cast<const void *>(softmax_persistent<F32, OP_BACKWARD, true>),
@@ -2294,6 +2591,11 @@ int launch_softmax(const KernelArgs &a, int dtype, int op, int grid, void *strea
             launch_one<F32, OP_BACKWARD_LONG>(a, grid, smem, st, checked);
         else
             launch_one<BF16, OP_BACKWARD_LONG>(a, grid, smem, st, checked);
+    } else if (op == OP_FORWARD_TEAM) {
+        if (dtype == BSM_F32)
+            launch_one<F32, OP_FORWARD_TEAM>(a, grid, smem, st, checked);
+        else
+            launch_one<BF16, OP_FORWARD_TEAM>(a, grid, smem, st, checked);
     } else if (op == OP_FORWARD_LONG) {
         if (dtype == BSM_F32)
             launch_one<F32, OP_FORWARD_LONG>(a, grid, smem, st, checked);

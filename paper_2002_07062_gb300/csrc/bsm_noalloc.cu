@@ -186,7 +186,7 @@ int softmax_noalloc(const void *x, void *y, int64_t B, int64_t R, int64_t C, int
     a.status = status;
     a.debug = g_na_debug.load(std::memory_order_relaxed);
     a.wait_limit_ns = g_na_wait_ns.load(std::memory_order_relaxed);
-    if (int e = launch_softmax(a, dtype, OP_FORWARD, nd->n_sm, stream, false))
+    if (int e = launch_softmax(a, dtype, row_bytes > kLaneRowBytes ? OP_FORWARD_TEAM : OP_FORWARD, nd->n_sm, stream, false))
         return record_cuda_error(e, "noalloc kernel launch");
     return BSM_OK;
 }
