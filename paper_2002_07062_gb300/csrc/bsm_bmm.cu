@@ -3,13 +3,13 @@
 // matrix product C_s = A_s * Bt_s^T, on the 5th-generation tensor cores.
 //
 // One persistent CTA per SM, 10 warps:
-//   warp 0, lane 0  producer: pulls output tiles (BM x BN of one slice) from
+//   warp 0          producer: pulls output tiles (BM x BN of one slice) from
 //                   the schedule (the slice scheduler's policies), streams the
 //                   tile's A rows and Bt rows, 64 columns of K at a time, into
-//                   a ring of shared-memory stages with 2-D TMA copies
+//                   a ring of shared-memory stages with 3-D TMA copies
 //                   (128-byte swizzle, completion on the stage's mbarrier);
 //   warp 1          owns the tensor memory (allocates two BN-column fp32
-//                   accumulators, frees them at the end); its lane 0 issues
+//                   accumulators, frees them at the end); issues
 //                   tcgen05.mma (M = 128, N = BN, K = 16 per instruction) from
 //                   shared-memory descriptors and commits each stage back to
 //                   the producer and each finished tile to the epilogue;
@@ -20,7 +20,8 @@
 //                   tensor store; two buffers per warp, so the next unit is
 //                   converted while the last one drains.
 // The accumulators are double-buffered so the epilogue of a tile overlaps the
-// MMAs of the next.  Every wait is bounded (2 s of %globaltimer): on expiry
+// MMAs of the next.  Warps 0 and 1 run their loops as a whole, the copies and
+// MMAs under an election (see elect_one).  Every wait is bounded (2 s of %globaltimer): on expiry
 // the CTA records BSM_DEV_TIMEOUT and leaves; the tensor memory is always
 // deallocated before the CTA exits.
 
@@ -87,6 +88,23 @@ __device__ __forceinline__ uint32_t gemm_smid()
     return s;
 }
 
+// True in one lane of the (converged) warp, the same one every time.  The
+// tensor-core and TMA instructions take their operands from uniform
+// registers: issued under this election in a loop that the whole warp runs,
+// they cost a few cycles each; issued by a lane that left the warp (lane == 0
+// around the loop) about 250 (measured: 64 K blocks of a 256 x 256 tile,
+// operands not even loaded, 36 us against 17 us of tensor time).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xFFFFFFFF;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void bar_init(uint64_t *b, uint32_t n)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(b)), "r"(n) : "memory");
@@ -133,6 +151,48 @@ __device__ __noinline__ bool bar_wait(uint64_t *b, uint32_t parity, const volati
     return false;
 }
 
+// The same wait inline and without the suspend hint, the clock read once in
+// 256 tries: for the waits on a stage, of which there is one per K block.
+__device__ __forceinline__ bool bar_spin(uint64_t *b, uint32_t parity, const volatile int32_t *abort)
+{
+    const uint32_t addr = saddr(b);
+    uint64_t t0 = 0;
+    for (uint32_t it = 0; it < (1u << 28); ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(addr), "r"(parity)
+            : "memory");
+        if (ok)
+            return true;
+        if ((it & 255u) == 255u) {
+            const uint64_t t = gtimer();
+            t0 = t0 ? t0 : t;
+            if (*abort || t - t0 > kGemmWaitNs)
+                return false;
+        }
+    }
+    return false;
+}
+
+// A place in the stage ring and the phase it is in, stepped instead of divided
+// out of a running count (a division per K block is a chain of about 150
+// cycles in the one warp that feeds the tensor cores).
+struct RingPos {
+    int s = 0;
+    uint32_t ph = 0;
+    __device__ __forceinline__ void step(int S)
+    {
+        if (++s == S) {
+            s = 0;
+            ph ^= 1u;
+        }
+    }
+};
+
 // 3-D TMA tile load: box at (c0 = column in the K block, c1 = row, c2 = K block).
 __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, int32_t c0, int32_t c1, int32_t c2,
                                             uint64_t *bar)
@@ -146,7 +206,7 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, i
 
 // Tile record of queue entry idx: read from the plan, or computed when the
 // plan keeps tiles in their natural order (slice, row block, column block).
-template <int BN> __device__ __forceinline__ GemmItem tile_at(const GemmArgs &a, int32_t idx)
+template <int BM, int BN> __device__ __forceinline__ GemmItem tile_at(const GemmArgs &a, int32_t idx)
 {
     if (idx < 0 || idx >= a.n_items)
         return GemmItem{-1, 0, 0, 0};
@@ -154,7 +214,7 @@ template <int BN> __device__ __forceinline__ GemmItem tile_at(const GemmArgs &a,
         return a.items[idx];
     const int32_t per = a.tiles_m * a.tiles_n;
     const int32_t s = idx / per, r = idx - s * per;
-    return GemmItem{s, (r / a.tiles_n) * 128, (r % a.tiles_n) * BN, 0};
+    return GemmItem{s, (r / a.tiles_n) * BM, (r % a.tiles_n) * BN, 0};
 }
 
 // Shared-memory matrix descriptor of a K-major operand tile whose rows are
@@ -169,10 +229,10 @@ __device__ __forceinline__ uint64_t smem_desc(const void *tile)
 }
 
 // Instruction descriptor of kind::f16: fp32 accumulator, bf16 A and B, both
-// K-major, N = BN, M = 128.
-template <int BN> __device__ __forceinline__ uint32_t mma_idesc()
+// K-major, N = BN, M = BM.
+template <int BM, int BN> __device__ __forceinline__ uint32_t mma_idesc()
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(BN >> 3) << 17) | (uint32_t(kBM >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(BN >> 3) << 17) | (uint32_t(BM >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
@@ -246,29 +306,30 @@ __device__ __forceinline__ uint32_t bf16x2(float lo, float hi)
 // softmax kernel: static list, whole slices round robin, die queues).
 struct GemmPuller {
     const GemmArgs &a;
+    int32_t unit, n_units;      // the pulling unit: a CTA, or a pair of CTAs
     int32_t k = 0, slice = -1, cur = 0, end = 0, q = 0, die = 0;
     bool first = true;
 
-    __device__ explicit GemmPuller(const GemmArgs &args) : a(args)
+    __device__ GemmPuller(const GemmArgs &args, int32_t unit_, int32_t n_units_) : a(args), unit(unit_), n_units(n_units_)
     {
         if (a.mode == PULL_QUEUE && a.sm_die) {
             const int d = a.sm_die[gemm_smid() & (BSM_MAX_SM - 1)];
             die = (d >= 0 && d < a.n_queues) ? d : 0;
         }
         if (a.mode == PULL_RR_SLICE)
-            slice = static_cast<int32_t>(blockIdx.x) - static_cast<int32_t>(gridDim.x);
+            slice = unit - n_units;
     }
 
     __device__ int32_t next()
     {
         if (a.mode == PULL_STATIC) {
-            const int64_t idx = (int64_t)a.item_begin + blockIdx.x + (int64_t)k * gridDim.x;
+            const int64_t idx = (int64_t)a.item_begin + unit + (int64_t)k * n_units;
             ++k;
             return idx < a.item_end ? static_cast<int32_t>(idx) : -1;
         }
         if (a.mode == PULL_RR_SLICE) {
             while (cur >= end) {
-                slice += gridDim.x;
+                slice += n_units;
                 if (slice >= a.n_slices)
                     return -1;
                 cur = a.slice_first_item[slice];
@@ -277,9 +338,9 @@ struct GemmPuller {
             return cur++;
         }
         if (a.n_queues == 1) {
-            // one queue: CTA i starts with tile i without touching the
-            // counter; later claims are counter + gridDim.x
-            const uint32_t t = first ? blockIdx.x : atomicAdd(&a.heads[0], 1u) + gridDim.x;
+            // one queue: unit i starts with tile i without touching the
+            // counter; later claims are counter + units
+            const uint32_t t = first ? unit : atomicAdd(&a.heads[0], 1u) + static_cast<uint32_t>(n_units);
             first = false;
             return t < static_cast<uint32_t>(a.queue_len[0]) ? a.queue_begin[0] + static_cast<int32_t>(t) : -1;
         }
@@ -294,6 +355,55 @@ struct GemmPuller {
         return -1;
     }
 };
+
+// One epilogue warp's share of a finished accumulator (tensor memory at tbase,
+// 32 lanes): units half, half + kActive / 4, ... of 32 rows x 128 bytes,
+// rounded, written to the warp's next store buffer (128-byte swizzle) and
+// stored by one TMA copy each, at row crow.  nst counts the warp's stores.
+template <int BN, bool kOutBf16, int kActive>
+__device__ __forceinline__ void store_tile(uint32_t tbase, int half, int bufs, unsigned char *mybuf, uint32_t &nst,
+                                           int lane, const CUtensorMap *tmC, int32_t n0, int32_t crow)
+{
+    constexpr int kEs = kOutBf16 ? 2 : 4;
+    constexpr int kUnitCols = 128 / kEs;                  // output columns per store unit
+    constexpr int kUnits = BN / kUnitCols;                // store units per tile row block
+#pragma unroll 1
+    for (int u = half; u < kUnits; u += kActive / 4, ++nst) {
+        uint32_t r[64];
+        tmem_ld32_nowait(tbase + static_cast<uint32_t>(u * kUnitCols), r);
+        if (kOutBf16)
+            tmem_ld32_nowait(tbase + static_cast<uint32_t>(u * kUnitCols + 32), r + 32);
+        tmem_wait_ld();
+        // the buffer about to be rewritten must have been read by its store
+        if (elect_one()) {
+            if (bufs >= 4)
+                asm volatile("cp.async.bulk.wait_group.read 3;" ::: "memory");
+            else if (bufs == 3)
+                asm volatile("cp.async.bulk.wait_group.read 2;" ::: "memory");
+            else if (bufs == 2)
+                asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            else
+                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        }
+        __syncwarp();
+        unsigned char *ub = mybuf + (nst % static_cast<uint32_t>(bufs)) * kEpiBuf;
+        const uint32_t sb = saddr(ub) + static_cast<uint32_t>(lane * 128);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const uint32_t dst = sb + (static_cast<uint32_t>(c ^ (lane & 7)) << 4);
+            if (kOutBf16) {
+                const float *f = reinterpret_cast<const float *>(r + 8 * c);
+                st_shared_v4(dst, bf16x2(f[0], f[1]), bf16x2(f[2], f[3]), bf16x2(f[4], f[5]), bf16x2(f[6], f[7]));
+            } else {
+                st_shared_v4(dst, r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (elect_one())
+            tma_store_2d(tmC, n0 + u * kUnitCols, crow, ub);
+    }
+}
 
 template <int BN, bool kOutBf16>
 __global__ void __launch_bounds__(kGemmThreads, 1)
@@ -314,7 +424,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     const int bufs = a.epi_bufs;                           // store buffers per active warp
     unsigned char *epi = smem + 1024;
     unsigned char *stages = smem + 1024 + kActive * bufs * kEpiBuf;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int S = a.n_stages;
     const int NS = a.K / (kBK * G);                        // stages per tile
 
@@ -323,7 +433,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         // The first claim and the tensor-map fetches are issued before the
         // barriers are set up; the producer streams as soon as they exist,
         // without waiting for the tensor-memory allocation.
-        GemmPuller pull(a);
+        GemmPuller pull(a, static_cast<int32_t>(blockIdx.x), static_cast<int32_t>(gridDim.x));
         int32_t idx = -1;
         if (lane == 0) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
@@ -352,50 +462,61 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         __syncwarp();
         asm volatile("barrier.cta.arrive 1, %0;" ::"r"(kGemmThreads) : "memory");   // barriers ready
         grid_launch_dependents();
-        if (lane == 0) {
-            uint32_t it = 0;
-            bool ok = true;
-            // the next tile is claimed (and its record fetched) while the
-            // current one streams, so the ring never waits on the queue
-            GemmItem item = tile_at<BN>(a, idx);
-            for (;;) {
-                const int32_t nidx = idx >= 0 ? pull.next() : -1;
-                const bool have = idx >= 0 && idx < a.n_items;
-                const bool valid = have && item.slice >= 0 && item.slice < a.B && item.m0 >= 0 &&
-                                   item.m0 + kBM <= a.M && item.n0 >= 0 && item.n0 + BN <= a.N;
-                if (idx >= 0 && !valid)
-                    atomicOr(a.status, BSM_DEV_BOUNDS);     // skip a bad tile, keep going
-                GemmItem nitem{};
-                const int nks = idx < 0 ? 1 : (valid ? NS : 0);
-                for (int kb = 0; kb < nks; ++kb) {
-                    const int s = static_cast<int>(it % S);
-                    const uint32_t ph = (it / S) & 1u;
-                    if (!bar_wait(&h.empty[s], ph ^ 1u, &h.abort_flag)) {
-                        ok = false;
-                        break;
-                    }
-                    ++it;
-                    if (idx < 0) {
+        uint32_t it = 0;
+        RingPos pos;
+        bool ok = true;
+        // the next tile is claimed (and its record fetched) by lane 0 while
+        // the current one streams, so the ring never waits on the queue
+        GemmItem item{};
+        if (lane == 0)
+            item = tile_at<kBM, BN>(a, idx);
+        for (;;) {
+            idx = __shfl_sync(0xffffffffu, idx, 0);
+            const int32_t slice = __shfl_sync(0xffffffffu, item.slice, 0), m0 = __shfl_sync(0xffffffffu, item.m0, 0),
+                          n0 = __shfl_sync(0xffffffffu, item.n0, 0);
+            const bool done = idx < 0;
+            const bool valid = !done && idx < a.n_items && slice >= 0 && slice < a.B && m0 >= 0 && m0 + kBM <= a.M &&
+                               n0 >= 0 && n0 + BN <= a.N;
+            if (!done && !valid && lane == 0)
+                atomicOr(a.status, BSM_DEV_BOUNDS);     // skip a bad tile, keep going
+            int32_t nidx = -1;
+            if (lane == 0 && !done)
+                nidx = pull.next();
+            GemmItem nitem{};
+            const int nks = done ? 1 : (valid ? NS : 0);
+            for (int kb = 0; kb < nks; ++kb) {
+                const int s = pos.s;
+                if (!__all_sync(0xffffffffu, bar_spin(&h.empty[s], pos.ph ^ 1u, &h.abort_flag))) {
+                    ok = false;
+                    break;
+                }
+                ++it;
+                pos.step(S);
+                unsigned char *st = stages + (size_t)s * stage_bytes;
+                if (elect_one()) {
+                    if (done) {
                         h.smeta[s].kind = GK_DONE;
                         bar_arrive(&h.full[s]);
-                        break;
+                    } else {
+                        if (kb == 0)
+                            h.smeta[s] = GemmMeta{slice, m0, n0, GK_DATA};
+                        bar_expect(&h.full[s], stage_bytes);
+                        tma_load_3d(st, &tmA, 0, slice * a.M + m0, kb * G, &h.full[s]);
+                        tma_load_3d(st + G * kABytes, &tmB, 0, slice * a.N + n0, kb * G, &h.full[s]);
                     }
-                    if (kb == 0)
-                        h.smeta[s] = GemmMeta{item.slice, item.m0, item.n0, GK_DATA};
-                    unsigned char *st = stages + (size_t)s * stage_bytes;
-                    bar_expect(&h.full[s], stage_bytes);
-                    tma_load_3d(st, &tmA, 0, item.slice * a.M + item.m0, kb * G, &h.full[s]);
-                    tma_load_3d(st + G * kABytes, &tmB, 0, item.slice * a.N + item.n0, kb * G, &h.full[s]);
-                    if (kb == 0)
-                        nitem = tile_at<BN>(a, nidx);
                 }
-                if (!ok || idx < 0)
-                    break;
-                if (nks == 0)
-                    nitem = tile_at<BN>(a, nidx);
-                idx = nidx;
-                item = nitem;
+                __syncwarp();
+                if (kb == 0 && !done && lane == 0)
+                    nitem = tile_at<kBM, BN>(a, nidx);
             }
+            if (!ok || done)
+                break;
+            if (nks == 0 && lane == 0)
+                nitem = tile_at<kBM, BN>(a, nidx);
+            idx = nidx;
+            item = nitem;
+        }
+        if (lane == 0) {
             if (!ok) {
                 atomicOr(a.status, BSM_DEV_TIMEOUT);
                 h.abort_flag = 1;
@@ -414,6 +535,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 }
             }
         }
+        __syncwarp();
     } else {
         asm volatile("barrier.cta.sync 1, %0;" ::"r"(kGemmThreads) : "memory");          // barriers ready
         if (warp == 1) {
@@ -428,73 +550,74 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         const uint32_t tmem = h.tmem_base;
         if (warp == 1) {
             // ------------------------------------------------------- MMA issuer
-            if (lane == 0) {
-                // no bounded wait may start before the previous kernel is done
-                grid_dependency_wait();
-                const uint32_t idesc = mma_idesc<BN>();
-                uint32_t it = 0, t = 0;
-                bool ok = true;
-                for (;;) {
-                    int s = static_cast<int>(it % S);
-                    uint32_t ph = (it / S) & 1u;
-                    if (!bar_wait(&h.full[s], ph, &h.abort_flag)) {
-                        ok = false;
-                        break;
-                    }
-                    const GemmMeta m = h.smeta[s];
-                    const int buf = static_cast<int>(t & 1u);
-                    const uint32_t tph = (t >> 1) & 1u;
-                    if (!bar_wait(&h.tempty[buf], tph ^ 1u, &h.abort_flag)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
+            // no bounded wait may start before the previous kernel is done
+            grid_dependency_wait();
+            const uint32_t idesc = mma_idesc<kBM, BN>();
+            uint32_t t = 0;
+            RingPos pos;
+            bool ok = true;
+            for (;;) {
+                const int buf = static_cast<int>(t & 1u);
+                const uint32_t tph = (t >> 1) & 1u;
+                if (!__all_sync(0xffffffffu, bar_spin(&h.full[pos.s], pos.ph, &h.abort_flag) &&
+                                                 bar_spin(&h.tempty[buf], tph ^ 1u, &h.abort_flag))) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const GemmMeta m = h.smeta[pos.s];
+                const bool done = __shfl_sync(0xffffffffu, m.kind, 0) == GK_DONE;
+                if (elect_one()) {
                     h.tmeta[buf] = m;
                     __threadfence_block();              // visible before the MMAs (and their commit)
-                    if (m.kind == GK_DONE) {
+                    if (done)
                         bar_arrive(&h.tfull[buf]);
-                        break;
-                    }
-                    const uint32_t d = tmem + static_cast<uint32_t>(buf * BN);
-                    for (int kb = 0; kb < NS; ++kb) {
-                        if (kb > 0) {
-                            s = static_cast<int>(it % S);
-                            ph = (it / S) & 1u;
-                            if (!bar_wait(&h.full[s], ph, &h.abort_flag)) {
-                                ok = false;
-                                break;
-                            }
+                }
+                __syncwarp();
+                if (done)
+                    break;
+                const uint32_t d = tmem + static_cast<uint32_t>(buf * BN);
+                for (int kb = 0; kb < NS; ++kb) {
+                    const int s = pos.s;
+                    if (kb > 0) {
+                        if (!__all_sync(0xffffffffu, bar_spin(&h.full[s], pos.ph, &h.abort_flag))) {
+                            ok = false;
+                            break;
                         }
                         tc_fence_after();
-                        unsigned char *st = stages + (size_t)s * stage_bytes;
+                    }
+                    unsigned char *st = stages + (size_t)s * stage_bytes;
+                    if (elect_one()) {
                         for (int j = 0; j < G; ++j) {
                             const uint64_t ad = smem_desc(st + j * kABytes);
                             const uint64_t bd = smem_desc(st + G * kABytes + j * kBBytes);
-    #pragma unroll
+#pragma unroll
                             for (int k = 0; k < kBK / 16; ++k)
                                 mma_bf16(d, ad + 2 * k, bd + 2 * k, idesc, (kb | j | k) != 0);
                         }
                         mma_commit(&h.empty[s]);        // the stage is free once these are done
-                        ++it;
+                        if (kb == NS - 1)
+                            mma_commit(&h.tfull[buf]);  // the accumulator is ready
                     }
-                    if (!ok)
-                        break;
-                    mma_commit(&h.tfull[buf]);          // the accumulator is ready
-                    ++t;
+                    __syncwarp();
+                    pos.step(S);
                 }
+                if (!ok)
+                    break;
+                ++t;
+            }
+            // every MMA issued has finished before the tensor memory is freed
+            if (elect_one()) {
                 if (!ok) {
                     atomicOr(a.status, BSM_DEV_TIMEOUT);
                     h.abort_flag = 1;
                 }
-                // every MMA issued has finished before the tensor memory is freed
                 mma_commit(&h.drain);
                 bar_wait(&h.drain, 0, nullptr);
             }
+            __syncwarp();
         } else {
             // ------------------------------------------------------- epilogue
-            constexpr int kEs = kOutBf16 ? 2 : 4;
-            constexpr int kUnitCols = 128 / kEs;                  // output columns per store unit
-            constexpr int kUnits = BN / kUnitCols;                // store units per tile row block
             const int ew = warp - 2;
             const int quarter = warp & 3;                         // TMEM lanes this warp may read
             const int half = ew >> 2;                             // which units of the quarter
@@ -523,48 +646,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 const uint32_t tbase =
                     tmem + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(buf * BN);
                 const int32_t crow = m.slice * a.M + m.m0 + quarter * 32;
-    #pragma unroll 1
-                for (int u = half; u < kUnits; u += kActive / 4, ++nst) {
-                    uint32_t r[64];
-                    tmem_ld32_nowait(tbase + static_cast<uint32_t>(u * kUnitCols), r);
-                    if (kOutBf16)
-                        tmem_ld32_nowait(tbase + static_cast<uint32_t>(u * kUnitCols + 32), r + 32);
-                    tmem_wait_ld();
-                    // the buffer about to be rewritten must have been read by its store
-                    if (lane == 0) {
-                        if (bufs >= 4)
-                            asm volatile("cp.async.bulk.wait_group.read 3;" ::: "memory");
-                        else if (bufs == 3)
-                            asm volatile("cp.async.bulk.wait_group.read 2;" ::: "memory");
-                        else
-                            asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-                    }
-                    __syncwarp();
-                    unsigned char *ub = mybuf + (nst % static_cast<uint32_t>(bufs)) * kEpiBuf;
-                    const uint32_t sb = saddr(ub) + static_cast<uint32_t>(lane * 128);
-    #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const uint32_t dst = sb + (static_cast<uint32_t>(c ^ (lane & 7)) << 4);
-                        if (kOutBf16) {
-                            const float *f = reinterpret_cast<const float *>(r + 8 * c);
-                            st_shared_v4(dst, bf16x2(f[0], f[1]), bf16x2(f[2], f[3]), bf16x2(f[4], f[5]),
-                                         bf16x2(f[6], f[7]));
-                        } else {
-                            st_shared_v4(dst, r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
-                        }
-                    }
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0)
-                        tma_store_2d(&tmC, m.n0 + u * kUnitCols, crow, ub);
-                }
+                store_tile<BN, kOutBf16, kActive>(tbase, half, bufs, mybuf, nst, lane, &tmC, m.n0, crow);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0)
                     bar_arrive(&h.tempty[buf]);
             }
             // stores complete before the CTA leaves
-            if (lane == 0)
+            if (elect_one())
                 asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
             __syncwarp();
         }
