@@ -236,7 +236,8 @@ int bsm_softmax_backward_ragged(const void *y, const void *dy, void *dx, int64_t
 /*
  * Batched matrix product, the paper's other batch algorithm (Sec. 6: batch
  * 384 of (512 x 64) x (64 x 512) and of (512 x 512) x (512 x 64)), on the
- * tensor cores, with the output tiles (128 x 64/128/256 of one slice) as the
+ * tensor cores, with the output tiles (128 x 64/128/256 of one slice; 256
+ * rows, on a pair of SMs, where the tensor cores bound the product) as the
  * patches of the same scheduling policies:
  *     C_s[m, n] = sum_k A_s[m, k] * Bt_s[n, k]        (C_s = A_s Bt_s^T)
  *   a   device, B x M x K bf16, row-major (slice s at s*M*K)

@@ -21,7 +21,8 @@
 //                   converted while the last one drains.
 // The accumulators are double-buffered so the epilogue of a tile overlaps the
 // MMAs of the next.  Warps 0 and 1 run their loops as a whole, the copies and
-// MMAs under an election (see elect_one).  Every wait is bounded (2 s of %globaltimer): on expiry
+// MMAs under an election (see elect_one).  Products bound by the tensor cores
+// run on pairs of CTAs instead (bmm_pair, below).  Every wait is bounded (2 s of %globaltimer): on expiry
 // the CTA records BSM_DEV_TIMEOUT and leaves; the tensor memory is always
 // deallocated before the CTA exits.
 
@@ -670,6 +671,403 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
 }
 
+// ------------------------------------------------ CTA pairs
+// A tile of 256 x BN on a pair of CTAs (a cluster of two): one
+// tcgen05.mma.cta_group::2 (M = 256, issued by the pair's first CTA) reads
+// 128 rows of A and BN / 2 rows of Bt from each CTA's shared memory and leaves
+// 128 rows of the product in each CTA's tensor memory.  A stage of one K block
+// then takes 32 KiB per CTA (BN = 256), so six of them fit beside the store
+// buffers where a 128 x 256 tile has three of 48 KiB, and an SM takes 64
+// bytes a cycle from L2 at the full tensor rate instead of 96.  8 x 2048^3,
+// bf16: 122.9 us (1.12 PFLOP/s) before, 104 with the warp-wide issue alone
+// (elect_one), 80.2 (1.71 PFLOP/s) on pairs; the tensor cores' own time is 60.
+//
+// Roles as in bmm_persistent, in both CTAs; what differs:
+//   - the first CTA claims the pair's tiles and posts each to both CTAs' rings
+//     of claim words (sequence number + 1 in the high half), which producer,
+//     MMA issuer and epilogue follow.  A claim runs at most S stages, two
+//     accumulators and two claims ahead of the slowest of them: kPairRing
+//     words are never overwritten unread.
+//   - both producers' copies count on the first CTA's full barrier; a finished
+//     stage or accumulator is committed to both CTAs;
+//   - both epilogues release an accumulator on the first CTA's barrier.
+// The CTAs meet (cluster barrier) after the barriers are set up and before
+// they leave; every other wait is bounded.
+constexpr int kPairBM = 2 * kBM;
+constexpr int kPairRing = 16;
+constexpr uint32_t kPairDone = 0xFFFFFFFFu;
+
+struct PairSmem {
+    uint64_t full[kGemmMaxStages];      // used in the first CTA
+    uint64_t empty[kGemmMaxStages];
+    uint64_t tfull[2];
+    uint64_t tempty[2];                 // used in the first CTA
+    uint64_t drain;
+    unsigned long long ring[kPairRing];
+    uint32_t tmem_base;
+    int32_t abort_flag;
+};
+static_assert(sizeof(PairSmem) <= 1024, "pair header");
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+// Address of `p` (this CTA's shared memory) in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t peer_addr(const void *p, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr(p)), "r"(rank));
+    return r;
+}
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// 3-D TMA tile load whose bytes count on a barrier of either CTA of the pair.
+__device__ __forceinline__ void tma_load_3d_pair(void *dst, const CUtensorMap *map, int32_t c0, int32_t c1,
+                                                 int32_t c2, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, "
+        "{%2, %3, %4}], [%5];" ::"r"(saddr(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                              uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// Arrive once on `bar` in both CTAs when every MMA issued so far is done.
+__device__ __forceinline__ void mma_commit_pair(uint64_t *bar)
+{
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            saddr(bar)),
+        "h"(static_cast<uint16_t>(3))
+        : "memory");
+}
+
+// The pair's tile number `seq` (bounded wait): false on abort or time out.
+__device__ __noinline__ bool ring_wait(const unsigned long long *ring, uint32_t seq, const volatile int32_t *abort,
+                                       uint32_t *tile)
+{
+    const uint32_t addr = saddr(&ring[seq % kPairRing]);
+    uint64_t t0 = 0;
+    for (uint32_t it = 0; it < (1u << 28); ++it) {
+        unsigned long long w;
+        asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(w) : "r"(addr) : "memory");
+        if (static_cast<uint32_t>(w >> 32) == seq + 1) {
+            *tile = static_cast<uint32_t>(w);
+            return true;
+        }
+        if ((it & 15u) == 15u) {
+            const uint64_t t = gtimer();
+            t0 = t0 ? t0 : t;
+            if (*abort || t - t0 > kGemmWaitNs)
+                return false;
+            __nanosleep(64);
+        }
+    }
+    return false;
+}
+
+template <int BN, bool kOutBf16>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+    bmm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+             const __grid_constant__ CUtensorMap tmC, const GemmArgs a)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *smem = smem_raw + ((1024u - (saddr(smem_raw) & 1023u)) & 1023u);
+    PairSmem &h = *reinterpret_cast<PairSmem *>(smem);
+    constexpr uint32_t kABytes = kBM * kBK * 2;
+    constexpr uint32_t kBBytes = BN / 2 * kBK * 2;
+    const int G = a.kbs;
+    const uint32_t stage_bytes = static_cast<uint32_t>(G) * (kABytes + kBBytes);   // per CTA
+    constexpr uint32_t kTmemCols = 2 * BN;
+    constexpr int kActive = epi_active(BN, kOutBf16);
+    const int bufs = a.epi_bufs;
+    unsigned char *epi = smem + 1024;
+    unsigned char *stages = smem + 1024 + kActive * bufs * kEpiBuf;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int S = a.n_stages;
+    const int NS = a.K / (kBK * G);
+    const uint32_t rank = cluster_rank();
+    auto tile_ok = [&](uint32_t idx, GemmItem &item) -> bool {
+        item = tile_at<kPairBM, BN>(a, static_cast<int32_t>(idx));
+        return item.slice >= 0 && item.slice < a.B && item.m0 >= 0 && item.m0 + kPairBM <= a.M && item.n0 >= 0 &&
+               item.n0 + BN <= a.N;
+    };
+
+    if (threadIdx.x == 0) {
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmC)) : "memory");
+        for (int s = 0; s < S; ++s) {
+            bar_init(&h.full[s], 1);
+            bar_init(&h.empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            bar_init(&h.tfull[b], 1);
+            bar_init(&h.tempty[b], 2 * kActive);
+        }
+        bar_init(&h.drain, 1);
+        for (int i = 0; i < kPairRing; ++i)
+            h.ring[i] = 0ull;
+        h.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&h.tmem_base)),
+                     "r"(kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();
+    tc_fence_after();
+    const uint32_t tmem = h.tmem_base;
+    // memory is touched from here on: wait for the previous kernel of the
+    // stream, then let the next one begin its launch
+    grid_dependency_wait();
+    grid_launch_dependents();
+
+    if (warp == 0) {
+        // ------------------------------------------------------- producer
+        const int32_t n_units = static_cast<int32_t>(gridDim.x >> 1);
+        GemmPuller pull(a, static_cast<int32_t>(blockIdx.x >> 1), n_units);
+        const uint32_t ring_peer = peer_addr(h.ring, 1u);
+        // lane 0 of the first CTA posts the pair's tiles, one claim ahead:
+        // the claim's round trip passes while a tile streams
+        int32_t claimed = -1;
+        uint32_t posted = 0;
+        bool post_done = false;
+        auto post = [&]() {
+            if (post_done)
+                return;
+            const uint32_t v = claimed >= 0 ? static_cast<uint32_t>(claimed) : kPairDone;
+            const unsigned long long w = (static_cast<unsigned long long>(posted + 1) << 32) | v;
+            const uint32_t o = (posted % kPairRing) * 8u;
+            asm volatile("st.relaxed.cluster.shared::cta.u64 [%0], %1;" ::"r"(saddr(h.ring) + o), "l"(w) : "memory");
+            asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(ring_peer + o), "l"(w) : "memory");
+            post_done = claimed < 0;
+            ++posted;
+            if (!post_done)
+                claimed = pull.next();
+        };
+        if (rank == 0 && lane == 0) {
+            claimed = pull.next();
+            post();
+        }
+        __syncwarp();
+        uint32_t it = 0;
+        RingPos pos;
+        bool ok = true;
+        for (uint32_t t = 0;; ++t) {
+            if (rank == 0 && lane == 0)
+                post();                                     // tile t + 1
+            __syncwarp();
+            uint32_t idx = 0;
+            if (!__all_sync(0xffffffffu, ring_wait(h.ring, t, &h.abort_flag, &idx))) {
+                ok = false;
+                break;
+            }
+            idx = __shfl_sync(0xffffffffu, idx, 0);
+            if (idx == kPairDone)
+                break;
+            GemmItem item;
+            if (!__all_sync(0xffffffffu, tile_ok(idx, item))) {
+                if (lane == 0)
+                    atomicOr(a.status, BSM_DEV_BOUNDS);     // every role skips it alike
+                continue;
+            }
+            const int32_t slice = __shfl_sync(0xffffffffu, item.slice, 0);
+            const int32_t arow = slice * a.M + __shfl_sync(0xffffffffu, item.m0, 0) + static_cast<int32_t>(rank) * kBM;
+            const int32_t brow =
+                slice * a.N + __shfl_sync(0xffffffffu, item.n0, 0) + static_cast<int32_t>(rank) * (BN / 2);
+            for (int kb = 0; kb < NS; ++kb, ++it, pos.step(S)) {
+                const int s = pos.s;
+                if (!__all_sync(0xffffffffu, bar_spin(&h.empty[s], pos.ph ^ 1u, &h.abort_flag))) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t full = peer_addr(&h.full[s], 0u);
+                unsigned char *st = stages + (size_t)s * stage_bytes;
+                if (elect_one()) {
+                    if (rank == 0)
+                        bar_expect(&h.full[s], 2 * stage_bytes);      // both CTAs' copies
+                    tma_load_3d_pair(st, &tmA, 0, arow, kb * G, full);
+                    tma_load_3d_pair(st + G * kABytes, &tmB, 0, brow, kb * G, full);
+                }
+                __syncwarp();
+            }
+            if (!ok)
+                break;
+        }
+        if (lane == 0) {
+            if (!ok) {
+                atomicOr(a.status, BSM_DEV_TIMEOUT);
+                h.abort_flag = 1;
+                // copies in flight land before the CTA may leave (normally
+                // the MMAs consumed every stage)
+                if (rank == 0)
+                    for (uint32_t j = it > static_cast<uint32_t>(S) ? it - S : 0u; j < it; ++j)
+                        bar_wait(&h.full[j % S], (j / S) & 1u, nullptr);
+            }
+            if (rank == 0 && a.mode == PULL_QUEUE) {
+                __threadfence();
+                const uint32_t prev = atomicAdd(&a.heads[BSM_MAX_DIES], 1u);
+                if (prev == static_cast<uint32_t>(n_units - 1)) {
+                    for (int d = 0; d < BSM_MAX_DIES; ++d)
+                        atomicExch(&a.heads[d], 0u);
+                    atomicExch(&a.heads[BSM_MAX_DIES], 0u);
+                }
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ------------------------------------------------------- MMA issuer
+        if (rank == 0) {
+            const uint32_t idesc = mma_idesc<kPairBM, BN>();
+            uint32_t acc = 0;
+            RingPos pos;
+            bool ok = true;
+            for (uint32_t t = 0; ok; ++t) {
+                uint32_t idx = 0;
+                if (!__all_sync(0xffffffffu, ring_wait(h.ring, t, &h.abort_flag, &idx))) {
+                    ok = false;
+                    break;
+                }
+                idx = __shfl_sync(0xffffffffu, idx, 0);
+                if (idx == kPairDone)
+                    break;
+                GemmItem item;
+                if (!__all_sync(0xffffffffu, tile_ok(idx, item)))
+                    continue;
+                const int buf = static_cast<int>(acc & 1u);
+                if (!__all_sync(0xffffffffu, bar_spin(&h.tempty[buf], ((acc >> 1) & 1u) ^ 1u, &h.abort_flag))) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t d = tmem + static_cast<uint32_t>(buf * BN);
+                for (int kb = 0; kb < NS; ++kb, pos.step(S)) {
+                    const int s = pos.s;
+                    if (!__all_sync(0xffffffffu, bar_spin(&h.full[s], pos.ph, &h.abort_flag))) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    unsigned char *st = stages + (size_t)s * stage_bytes;
+                    if (elect_one()) {
+                        for (int j = 0; j < G; ++j) {
+                            const uint64_t ad = smem_desc(st + j * kABytes);
+                            const uint64_t bd = smem_desc(st + G * kABytes + j * kBBytes);
+#pragma unroll
+                            for (int k = 0; k < kBK / 16; ++k)
+                                mma_bf16_pair(d, ad + 2 * k, bd + 2 * k, idesc, (kb | j | k) != 0);
+                        }
+                        mma_commit_pair(&h.empty[s]);
+                        if (kb == NS - 1)
+                            mma_commit_pair(&h.tfull[buf]);
+                    }
+                    __syncwarp();
+                }
+                ++acc;
+            }
+            // every MMA issued has finished before either CTA may leave
+            if (elect_one()) {
+                if (!ok) {
+                    atomicOr(a.status, BSM_DEV_TIMEOUT);
+                    h.abort_flag = 1;
+                }
+                asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                 saddr(&h.drain))
+                             : "memory");
+                bar_wait(&h.drain, 0, nullptr);
+            }
+        }
+        __syncwarp();
+    } else {
+        // ------------------------------------------------------- epilogue
+        const int ew = warp - 2;
+        const int quarter = warp & 3;
+        const int half = ew >> 2;
+        unsigned char *mybuf = epi + ew * bufs * kEpiBuf;
+        uint32_t nst = 0, acc = 0;
+        const uint32_t tempty[2] = {peer_addr(&h.tempty[0], 0u), peer_addr(&h.tempty[1], 0u)};
+        for (uint32_t t = 0; ew < kActive; ++t) {
+            const int buf = static_cast<int>(acc & 1u);
+            // lane 0 waits; the warp follows its verdict (tcgen05.ld is warp-wide)
+            uint32_t idx = 0;
+            int ok = 0;
+            GemmItem item{};
+            if (lane == 0) {
+                ok = ring_wait(h.ring, t, &h.abort_flag, &idx) ? 1 : 0;
+                if (ok && idx != kPairDone) {
+                    if (!tile_ok(idx, item))
+                        ok = 2;
+                    else if (!bar_wait(&h.tfull[buf], (acc >> 1) & 1u, &h.abort_flag))
+                        ok = 0;
+                }
+                if (!ok) {
+                    atomicOr(a.status, BSM_DEV_TIMEOUT);
+                    h.abort_flag = 1;
+                }
+            }
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            idx = __shfl_sync(0xffffffffu, idx, 0);
+            if (!ok || idx == kPairDone)
+                break;
+            if (ok == 2)
+                continue;
+            const int32_t crow = __shfl_sync(0xffffffffu, item.slice * a.M + item.m0, 0) +
+                                 static_cast<int32_t>(rank) * kBM + quarter * 32;
+            const int32_t n0 = __shfl_sync(0xffffffffu, item.n0, 0);
+            tc_fence_after();
+            store_tile<BN, kOutBf16, kActive>(tmem + (static_cast<uint32_t>(quarter * 32) << 16) +
+                                                  static_cast<uint32_t>(buf * BN),
+                                              half, bufs, mybuf, nst, lane, &tmC, n0, crow);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(tempty[buf])
+                             : "memory");
+            ++acc;
+        }
+        if (elect_one())
+            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        __syncwarp();
+    }
+
+    // every thread gets here (all waits are bounded); neither CTA frees its
+    // tensor memory or leaves while the other may still use it
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(h.tmem_base), "r"(kTmemCols)
+                     : "memory");
+    }
+}
+
 template <int BN, bool kOutBf16>
 int launch_bn(const CUtensorMap &ta, const CUtensorMap &tb, const CUtensorMap &tc, const GemmArgs &a, int grid,
               cudaStream_t st)
@@ -694,9 +1092,36 @@ int launch_bn(const CUtensorMap &ta, const CUtensorMap &tb, const CUtensorMap &t
 #endif
 }
 
+// A grid of CTA pairs (clusters of two).
+template <int BN, bool kOutBf16>
+int launch_pair(const CUtensorMap &ta, const CUtensorMap &tb, const CUtensorMap &tc, const GemmArgs &a, int grid,
+                cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(kGemmThreads);
+    cfg.dynamicSmemBytes = static_cast<size_t>(gemm_fixed_smem(BN, kOutBf16, a.epi_bufs)) +
+                           (size_t)a.n_stages * a.kbs * gemm_pair_stage_bytes(BN);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+#ifdef BSM_NO_PDL
+    cfg.numAttrs = 1;
+#endif
+    return static_cast<int>(cudaLaunchKernelEx(&cfg, bmm_pair<BN, kOutBf16>, ta, tb, tc, a));
+}
+
 }  // namespace
 
 int gemm_stage_bytes(int bn) { return kBM * kBK * 2 + bn * kBK * 2; }
+int gemm_pair_stage_bytes(int bn) { return kBM * kBK * 2 + bn / 2 * kBK * 2; }
 int gemm_threads() { return kGemmThreads; }
 int gemm_fixed_smem(int bn, bool out_bf16, int epi_bufs)
 {
@@ -710,7 +1135,11 @@ int gemm_set_smem_limit(int bytes)
                          reinterpret_cast<const void *>(bmm_persistent<128, false>),
                          reinterpret_cast<const void *>(bmm_persistent<128, true>),
                          reinterpret_cast<const void *>(bmm_persistent<256, false>),
-                         reinterpret_cast<const void *>(bmm_persistent<256, true>)};
+                         reinterpret_cast<const void *>(bmm_persistent<256, true>),
+                         reinterpret_cast<const void *>(bmm_pair<128, false>),
+                         reinterpret_cast<const void *>(bmm_pair<128, true>),
+                         reinterpret_cast<const void *>(bmm_pair<256, false>),
+                         reinterpret_cast<const void *>(bmm_pair<256, true>)};
     for (const void *f : fns)
         if (cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))
             return static_cast<int>(e);
@@ -724,6 +1153,13 @@ int launch_bmm(const void *tmap_a, const void *tmap_b, const void *tmap_c, const
     const CUtensorMap &tb = *static_cast<const CUtensorMap *>(tmap_b);
     const CUtensorMap &tc = *static_cast<const CUtensorMap *>(tmap_c);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (a.pair) {
+        if (bn == 128)
+            return out_bf16 ? launch_pair<128, true>(ta, tb, tc, a, grid, st)
+                            : launch_pair<128, false>(ta, tb, tc, a, grid, st);
+        return out_bf16 ? launch_pair<256, true>(ta, tb, tc, a, grid, st)
+                        : launch_pair<256, false>(ta, tb, tc, a, grid, st);
+    }
     if (bn == 64)
         return out_bf16 ? launch_bn<64, true>(ta, tb, tc, a, grid, st) : launch_bn<64, false>(ta, tb, tc, a, grid, st);
     if (bn == 128)

@@ -101,6 +101,7 @@ struct GemmPlan {
     int device = 0, policy = 0, bn = 0, grid = 0;
     int want_stages = 0, want_bufs = 0, want_kbs = 0;   // caller's choices (0 = automatic)
     bool out_bf16 = false;
+    bool pair = false;                  // tiles of 256 rows on pairs of CTAs
     const void *a = nullptr, *bt = nullptr;
     void *c = nullptr;
     int64_t B = 0, M = 0, N = 0, K = 0;
@@ -172,7 +173,8 @@ int build_plan(GemmPlan *p, const GemmDev &dev)
 {
     TraceRange trace("bsm_bmm_plan_create");
     const int bn = p->bn;
-    const int64_t mt = p->M / 128, nt = p->N / bn;
+    const int bm = p->pair ? 256 : 128;
+    const int64_t mt = p->M / bm, nt = p->N / bn;
     const int64_t n_items = p->B * mt * nt;
     if (n_items > INT32_MAX)
         return BSM_ERR_UNSUPPORTED;
@@ -183,7 +185,7 @@ int build_plan(GemmPlan *p, const GemmDev &dev)
         slice_first[s] = static_cast<int32_t>(k);
         for (int64_t i = 0; i < mt; ++i)
             for (int64_t j = 0; j < nt; ++j)
-                items[k++] = GemmItem{static_cast<int32_t>(s), static_cast<int32_t>(i * 128),
+                items[k++] = GemmItem{static_cast<int32_t>(s), static_cast<int32_t>(i * bm),
                                       static_cast<int32_t>(j * bn), 0};
     }
     slice_first[p->B] = static_cast<int32_t>(k);
@@ -212,8 +214,8 @@ int build_plan(GemmPlan *p, const GemmDev &dev)
             std::vector<int64_t> pb(items.size()), pe(items.size()), cost(items.size());
             for (size_t i = 0; i < items.size(); ++i) {
                 pb[i] = ((int64_t)items[i].slice * p->M + items[i].m0) * p->K * 2;
-                pe[i] = pb[i] + 128 * p->K * 2;
-                cost[i] = pe[i] - pb[i] + (int64_t)bn * p->K * 2 + 128ll * bn * (p->out_bf16 ? 2 : 4);
+                pe[i] = pb[i] + bm * p->K * 2;
+                cost[i] = pe[i] - pb[i] + (int64_t)bn * p->K * 2 + int64_t(bm) * bn * (p->out_bf16 ? 2 : 4);
             }
             int32_t units[BSM_MAX_DIES] = {std::max(1, topo.sm_per_die[0]), std::max(1, topo.sm_per_die[1])};
             bsm_schedule_desc sd{};
@@ -305,22 +307,26 @@ int build_plan(GemmPlan *p, const GemmDev &dev)
     // and fetch several K blocks per copy when the tile has them (longer
     // runs of each operand row per request), keeping two stages or more
     const int64_t kb = p->K / 64;
+    const int block_bytes = p->pair ? gemm_pair_stage_bytes(bn) : gemm_stage_bytes(bn);
     int kbs = p->want_kbs;
     if (!kbs) {
         kbs = 1;
         for (int g : {4, 2})
-            if (kb % g == 0 &&
-                (dev.smem_optin - gemm_fixed_smem(bn, p->out_bf16, 2)) / (g * gemm_stage_bytes(bn)) >= 2) {
+            if (!p->pair && kb % g == 0 &&
+                (dev.smem_optin - gemm_fixed_smem(bn, p->out_bf16, 2)) / (g * block_bytes) >= 2) {
                 kbs = g;
                 break;
             }
     }
     if (kb % kbs)
         return BSM_ERR_UNSUPPORTED;
-    int bufs = p->want_bufs ? p->want_bufs : (kb <= 2 ? 4 : 2);
+    // (a pair's tile has many K blocks: one store buffer per warp and six
+    // stages of one block; two buffers and five stages ran 8 x 2048^3 in 82.9
+    // us against 80.2, two blocks a stage in 81.7)
+    int bufs = p->want_bufs ? p->want_bufs : p->pair ? 1 : (kb <= 2 ? 4 : 2);
     int fit = 0;
     for (;; --bufs) {
-        fit = (dev.smem_optin - gemm_fixed_smem(bn, p->out_bf16, bufs)) / (kbs * gemm_stage_bytes(bn));
+        fit = (dev.smem_optin - gemm_fixed_smem(bn, p->out_bf16, bufs)) / (kbs * block_bytes);
         if (fit >= 2 || bufs <= 2 || p->want_bufs)
             break;
     }
@@ -328,12 +334,13 @@ int build_plan(GemmPlan *p, const GemmDev &dev)
     // extra store buffers (E1, 384 x (512x64)(64x512): 3 stages x 2 buffers
     // 41.60 us against 2 x 4 41.85 us, same box)
     if (!p->want_bufs && !p->want_stages && fit == 2 && bufs > 2) {
-        const int fit2 = (dev.smem_optin - gemm_fixed_smem(bn, p->out_bf16, 2)) / (kbs * gemm_stage_bytes(bn));
+        const int fit2 = (dev.smem_optin - gemm_fixed_smem(bn, p->out_bf16, 2)) / (kbs * block_bytes);
         if (fit2 >= 3) {
             bufs = 2;
             fit = fit2;
         }
     }
+    a.pair = p->pair ? 1 : 0;
     a.epi_bufs = bufs;
     a.kbs = kbs;
     a.identity = use_die ? 0 : 1;
@@ -345,24 +352,25 @@ int build_plan(GemmPlan *p, const GemmDev &dev)
     a.status = dev.status;
     if (a.n_stages < 2)
         return BSM_ERR_UNSUPPORTED;
+    const int unit = p->pair ? 2 : 1;       // CTAs per tile
     switch (p->policy) {
     case BSM_POLICY_WHOLE_GPU:
         a.mode = PULL_STATIC;
         p->whole_begin = slice_first;
-        p->grid = static_cast<int>(std::min<int64_t>(dev.n_sm, mt * nt));
+        p->grid = unit * static_cast<int>(std::min<int64_t>(dev.n_sm / unit, mt * nt));
         break;
     case BSM_POLICY_RR:
         a.mode = PULL_RR_SLICE;
-        p->grid = static_cast<int>(std::min<int64_t>(dev.n_sm, p->B));
+        p->grid = unit * static_cast<int>(std::min<int64_t>(dev.n_sm / unit, p->B));
         break;
     default:
         a.mode = PULL_QUEUE;
-        p->grid = dev.n_sm;
+        p->grid = unit * (dev.n_sm / unit);
         break;
     }
     if (int rc = make_operand_map(&p->ta, p->a, p->B * p->M, p->K, 128, kbs))
         return rc;
-    if (int rc = make_operand_map(&p->tb, p->bt, p->B * p->N, p->K, bn, kbs))
+    if (int rc = make_operand_map(&p->tb, p->bt, p->B * p->N, p->K, p->pair ? bn / 2 : bn, kbs))
         return rc;
     if (int rc = make_map(&p->tc, p->c, p->B * p->M, p->N, 32, !p->out_bf16))
         return rc;
@@ -387,6 +395,30 @@ int run_plan(GemmPlan *p, bsm_stream_t stream)
         err = launch_bmm(&p->ta, &p->tb, &p->tc, p->args, p->bn, p->out_bf16, p->grid, stream);
     }
     return err ? record_cuda_error(err, "bmm kernel launch") : BSM_OK;
+}
+
+// Whether the product runs on tiles of 256 x bn over pairs of CTAs: where the
+// tensor cores rather than HBM bound it, and a CTA has enough of them.  Pairs
+// against single CTAs (us, bf16 out, same box): 8 x 2048^3 80.2 / 104, 64 x
+// 1024^3 115 / 132, 64 x (1024 x 512)(512 x 1024) 56.7 / 73.0, 32 x (1024 x
+// 2048)(2048 x 384) 53.6 / 71.2, 1 x 2048^3 17.2 / 19.0.
+// - Fewer than 120 operations a byte (about 0.4 of the ratio of the two
+//   peaks) are bound by HBM, where a pair only adds its fixed cost: 300 x (256 x
+//   512)(512 x 128) 26.8 / 25.3, 64 x (1024 x 128)(128 x 1024) 45 / 36.7.
+// - Under 1280 of K per SM (tiles x K / SMs) a pair's start, about 1.5 us
+//   longer, is not made up: 19 x (512 x 1024)(1024 x 512) 12.3 / 11.4, 2048 x
+//   2048 x 1024 12.7 / 11.0 -- but a single long tile is: 1024 x 1024 x 4096
+//   24.8 / 28.9.
+// Results do not depend on it (the same order of the K blocks in one
+// accumulator).
+bool use_pair(int n_sm, int64_t B, int64_t M, int64_t N, int64_t K, int bn, bool out_bf16)
+{
+    if (M % 256 || bn < 128)
+        return false;
+    const double flops = 2.0 * double(B) * double(M) * double(N) * double(K);
+    const double bytes = 2.0 * double(B) * double(M + N) * double(K) + (out_bf16 ? 2.0 : 4.0) * double(B) * double(M) * double(N);
+    const double tiles = double(B) * double(M / 128) * double(N / bn);
+    return flops >= 120.0 * bytes && (K >= 4096 || tiles * double(K) >= 1280.0 * n_sm);
 }
 
 int bmm_impl(const void *a, const void *bt, void *c, int64_t B, int64_t M, int64_t N, int64_t K, int out_dtype,
@@ -438,6 +470,9 @@ int bmm_impl(const void *a, const void *bt, void *c, int64_t B, int64_t M, int64
     p->want_kbs = kbs;
     p->bn = N % 256 == 0 ? 256 : (N % 128 == 0 ? 128 : 64);
     p->out_bf16 = out_dtype == BSM_BF16;
+    // (a split chosen by the caller is one of a single CTA's shared memory)
+    p->pair = !n_stages && !epi_bufs && !kbs && dev->n_sm >= 2 &&
+              use_pair(dev->n_sm, B, M, N, K, p->bn, out_dtype == BSM_BF16);
     p->a = a;
     p->bt = bt;
     p->c = c;

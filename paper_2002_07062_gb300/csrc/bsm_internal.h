@@ -133,8 +133,8 @@ struct KernelArgs {
 // Test-only fault injection (bsm_plan_debug).
 constexpr uint32_t KDEBUG_WITHHOLD_STAGE0 = 1u;   // producer never fills stage 0 of its first round
 
-// One output tile of the batched matrix product: rows [m0, m0 + 128) and
-// columns [n0, n0 + BN) of slice `slice`.
+// One output tile of the batched matrix product: rows [m0, m0 + 128) (256 on
+// pairs of CTAs) and columns [n0, n0 + BN) of slice `slice`.
 struct GemmItem {
     int32_t slice, m0, n0, pad;
 };
@@ -159,6 +159,7 @@ struct GemmArgs {
     int32_t kbs;                    // K blocks of 64 per stage (1, 2 or 4)
     int32_t identity;               // items in natural order: computed, not read
     int32_t tiles_m, tiles_n;       // row / column blocks per slice
+    int32_t pair;                   // 1: tiles of 256 rows on pairs of CTAs (grid even)
     uint32_t *status;
 };
 
@@ -169,6 +170,7 @@ int launch_bmm(const void *tmap_a, const void *tmap_b, const void *tmap_c, const
                bool out_bf16, int grid, void *stream);
 int gemm_set_smem_limit(int bytes);
 int gemm_stage_bytes(int bn);
+int gemm_pair_stage_bytes(int bn);   // per CTA of a pair
 // shared memory of one launch besides the stages (header, slack, epilogue
 // store buffers: epi_bufs of 4 KiB per epilogue warp with work)
 int gemm_fixed_smem(int bn, bool out_bf16, int epi_bufs);
