@@ -37,6 +37,7 @@ constexpr int kFetch = 4;
 constexpr int kMaxStages = 8;
 constexpr int kConsumerWarps = 16;
 constexpr int kThreads = (kConsumerWarps + 1) * 32;  // + one producer warp
+constexpr int kGroupThreads = kThreads + 32;          // rows over groups: + one exchange warp
 constexpr int kSmemHeader = 1024;                     // barriers + stage metadata
 // Smallest stage (three fit the shared memory).  Each stage has a fixed cost
 // (wait, metadata, dispatch, release) that larger stages amortise; measured
@@ -75,7 +76,7 @@ constexpr int kLaneRowBytes = 2048;
 // by the last CTA of every launch.
 constexpr int kGroupRing = 16;
 constexpr int kGroupSlots = 4;
-constexpr int kMaxGroup = 128;
+constexpr int kMaxGroup = 32;     // a member reads one partial per lane of a warp
 // A member's part is held in registers while its group exchanges partials:
 // at most kGroupVecs 16-byte vectors per consumer thread, i.e. parts of at
 // most kGroupVecs * 16 * 512 bytes = 64 KiB.

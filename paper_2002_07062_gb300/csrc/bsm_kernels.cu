@@ -69,14 +69,19 @@ static_assert(sizeof(StageMeta) == 64, "StageMeta layout");
 struct SmemHeader {
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
+    uint64_t xwarp;                 // long rows, rows on 16 warps: the warps' partials are in
     union {
-        uint64_t xwarp;             // long rows, rows on 16 warps: the warps' partials are in
-        uint32_t xarrive[2];        // rows over groups: warps whose partial is in, by row parity
+        uint64_t team[kTeamBars];   // rows shared by a team of warps: its partials are in
+        struct {                    // rows over groups:
+            uint64_t xres;          // a row's result is in
+            float2 result[2];       // ... its (offset, sum), two rows deep
+            uint32_t xarrive[2];    // warps whose partial is in, by row parity
+            uint32_t xleft;         // consumer warps that have left
+        };
     };
-    uint64_t team[kTeamBars];       // rows shared by a team of warps: its partials are in
     int32_t abort_flag;
     StageMeta meta[kMaxStages];
-    float2 partial[2][kConsumerWarps];   // (max, sum) per warp of a row they share, two rows deep
+    float2 partial[2][kConsumerWarps];   // (offset, sum) per warp of a row they share, two rows deep
 };
 static_assert(sizeof(SmemHeader) <= kSmemHeader, "header too large");
 
@@ -582,26 +587,6 @@ __device__ __forceinline__ float vec_exp_sum_pairs(float (&v)[EPV], float mL)
         const float2 b = add2(make_float2(v[2], v[6]), make_float2(v[3], v[7]));
         const float2 c = add2(a, b);
         return c.x + c.y;
-    }
-}
-
-// The maximum of a chunk's vectors as loaded: bf16 on the packed words
-// (exact; a NaN operand loses, as with fmaxf), fp32 through tree_max.
-template <typename Tag, int N>
-__device__ __forceinline__ float raw_max(const uint4 (&raw)[N], const float (&v)[N][Elem<Tag>::kPerVec])
-{
-    if constexpr (Elem<Tag>::kSize == 2) {
-        uint32_t mw = 0xFF80FF80u;
-#pragma unroll
-        for (int j = 0; j < N; ++j)
-            mw = bmax2(mw, bmax2(bmax2(raw[j].x, raw[j].y), bmax2(raw[j].z, raw[j].w)));
-        return fmaxf(__uint_as_float(mw << 16), __uint_as_float(mw & 0xFFFF0000u));
-    } else {
-        float m = -INFINITY;
-#pragma unroll
-        for (int j = 0; j < N; ++j)
-            m = fmaxf(m, tree_max<Elem<Tag>::kPerVec>(v[j]));
-        return m;
     }
 }
 
@@ -1961,34 +1946,28 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
 // A row too long for one SM's shared memory is cut into K parts of equal
 // length (whole 16-byte vectors; the last may be shorter or empty), and the K
 // CTAs of a group each stage one part in one stage: every element is read
-// from memory once.  Each CTA takes its part's running (max, rescaled sum)
-// -- threads, then warps in a fixed order -- and publishes it in global
-// memory as two words tagged with the row's sequence number; every member
-// then reads the K partials until all carry the tag, combines them in the
-// same fixed order (a per-lane sum over ranks l, l + 32, ..., then the xor
-// tree), and writes its part of y.  The consumers work one row ahead: they
-// take the next row's partial (from its stage) before finishing the previous
-// row (held in registers), so the exchange overlaps work.  The group's
+// from memory once.  Each CTA takes its part's (offset, sum) -- warps, then
+// the CTA in a fixed tree, the offset the rounded max * log2 e as in row_team
+// -- and publishes it in global memory as two words tagged with the row's
+// sequence number; every member then reads the K partials (one per lane)
+// until all carry the tag, combines them in the same fixed tree, and writes
+// its part of y.  An exchange warp of its own does that, and the consumers
+// work one row ahead: they take the next row's partial (from its stage) before
+// writing the previous row (held in registers), so the exchange overlaps
+// work.  fp32 1 MiB rows (K = 16) ran at 4811 GB/s when every consumer warp
+// polled for itself, with a running maximum rescaled per chunk and the
+// producer's chain of round trips (see there), and run at 5472; bf16 4137 and
+// 5136; without the row between, 4180; with the exchange warp publishing as
+// well (so behind its polling), 4830.  What is left is the stage held through
+// a partial and a write (5400 without any exchange).  The group's
 // rank-0 CTA claims the rows (any policy's puller, with the group as the
 // unit) and announces them to its members through a ring of claim words.
 // The launch is cooperative, so every member of a group is resident and each
 // wait ends; every wait is bounded all the same.
 
-__device__ __forceinline__ void st_release_u64(unsigned long long *p, unsigned long long v)
-{
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned long long v)
 {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p)
-{
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
 }
 
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long *p)
@@ -2002,13 +1981,13 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
 __device__ __noinline__ bool wait_claim(const unsigned long long *p, uint32_t seq, const volatile int32_t *abort,
                                         uint64_t limit_ns, unsigned long long &word)
 {
-    word = ld_acquire_u64(p);
+    word = ld_relaxed_u64(p);
     if (static_cast<uint32_t>(word >> 32) == seq)
         return true;
     const uint64_t t0 = global_timer_ns();
     for (uint32_t it = 0; it < (1u << 26); ++it) {
         __nanosleep(32);
-        word = ld_acquire_u64(p);
+        word = ld_relaxed_u64(p);
         if (static_cast<uint32_t>(word >> 32) == seq)
             return true;
         if ((abort && *abort) || global_timer_ns() - t0 > limit_ns)
@@ -2017,153 +1996,52 @@ __device__ __noinline__ bool wait_claim(const unsigned long long *p, uint32_t se
     return false;
 }
 
-__device__ __forceinline__ unsigned long long pack_ms(float m, float sum)
-{
-    return (static_cast<unsigned long long>(__float_as_uint(sum)) << 32) | __float_as_uint(m);
-}
-
 // A member's part of a group row held in registers: consumer thread t (of
 // the kConsumerWarps * 32) holds the part's 16-byte vectors t, t + 512, ...
 constexpr int kConsumerThreads = kConsumerWarps * 32;
 
+// Vector vi of the part in the stage; -inf past its end.
 template <typename Tag, bool Checked>
-__device__ __forceinline__ void group_load(uint4 (&r)[kGroupVecs], const unsigned char *sbuf, int nvec, int tid,
-                                           const Bounds &bd)
+__device__ __forceinline__ uint4 group_vec(const unsigned char *sbuf, int vi, int nvec, const Bounds &bd)
 {
-    using E = Elem<Tag>;
-#pragma unroll
-    for (int j = 0; j < kGroupVecs; ++j) {
-        const int vi = tid + j * kConsumerThreads;
-        r[j] = E::neg_inf_vec();
-        if (vi < nvec) {
-            uint4 t;
-            if (load_vec<Checked>(sbuf + 16 * vi, bd, t))
-                r[j] = t;
-        }
+    uint4 r = Elem<Tag>::neg_inf_vec();
+    if (vi < nvec) {
+        uint4 t;
+        if (load_vec<Checked>(sbuf + 16 * vi, bd, t))
+            r = t;
     }
+    return r;
 }
 
-// This thread's running (max, sum of exp(v - max)) over its vectors of the
-// part in the stage, in chunks of 16 elements (4 fp32 or 2 bf16 vectors, so
-// the chunk's unpacked values and the held row fit the registers): a chunk's vectors are
-// loaded first (independent loads), then its maximum taken (bf16 without
-// the causal mask: on the packed words) and, when it grows the running one,
-// the sum rescaled; then the chunk's exponentials added in vector order,
-// computed in fp32 pairs (the same bits as one at a time: each pair is two
-// IEEE operations, each vector's sum in tree_sum's order).  While the
-// running maximum is -inf every value seen is -inf (masked) or NaN: it adds
-// 0 (NaN).  `mid` runs halfway through (the
-// caller issues its exchange loads there).
-template <typename Tag, bool Checked, typename Mid>
-__device__ __forceinline__ void group_partial(const unsigned char *sbuf, int nvec, int tid, int col0, int row,
-                                              bool causal, const Bounds &bd, float &m, float &s, Mid &&mid)
+// A member's two exchange words in one access (each word is validated by its
+// own tag, so nothing depends on the two being one).
+__device__ __forceinline__ void st_words(unsigned long long *p, unsigned long long w0, unsigned long long w1)
 {
-    using E = Elem<Tag>;
-    constexpr int EPV = E::kPerVec;
-    constexpr int kGroupChunk = 16 / EPV;
-    m = -INFINITY;
-    s = 0.0f;
-#pragma unroll
-    for (int c = 0; c < kGroupVecs; c += kGroupChunk) {
-        if (c == kGroupVecs / 2)
-            mid();
-        uint4 raw[kGroupChunk];
-#pragma unroll
-        for (int j = 0; j < kGroupChunk; ++j) {
-            const int vi = tid + (c + j) * kConsumerThreads;
-            raw[j] = E::neg_inf_vec();
-            if (vi < nvec) {
-                uint4 t;
-                if (load_vec<Checked>(sbuf + 16 * vi, bd, t))
-                    raw[j] = t;
-            }
-        }
-        float cm = -INFINITY;
-        float v[kGroupChunk][EPV];
-        if (causal) {
-#pragma unroll
-            for (int j = 0; j < kGroupChunk; ++j) {
-                const int col = col0 + (tid + (c + j) * kConsumerThreads) * EPV;
-                E::unpack(raw[j], v[j]);
-                if (col + EPV - 1 > row)
-                    apply_causal<EPV>(v[j], col, row);
-                cm = fmaxf(cm, tree_max<EPV>(v[j]));
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < kGroupChunk; ++j)
-                E::unpack(raw[j], v[j]);
-            cm = raw_max<Tag, kGroupChunk>(raw, v);
-        }
-        if (cm > m) {
-            s *= ex2((m - cm) * kLog2e);
-            m = cm;
-        }
-        const float mL = m * kLog2e;
-#pragma unroll
-        for (int j = 0; j < kGroupChunk; ++j) {
-            const int vi = tid + (c + j) * kConsumerThreads;
-            const int col = col0 + vi * EPV;
-            if (vi < nvec) {
-                if ((causal && col > row) || m == -INFINITY) {
-                    vec_exp<EPV>(v[j], mL, true);
-                    s += tree_sum<EPV>(v[j]);
-                } else {
-                    s += vec_exp_sum_pairs<EPV>(v[j], mL);
-                }
-            }
-        }
-    }
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(w0), "l"(w1) : "memory");
 }
 
-// y = exp(v - M) / S for this thread's vectors of the part (mL = M log2 e),
-// in fp32 pairs where no element is masked.
-template <typename Tag, bool Checked>
-__device__ __forceinline__ void group_write(const uint4 (&r)[kGroupVecs], int nvec, int tid, int col0, int row,
-                                            bool causal, float mL, float inv, unsigned char *ypart, const Bounds &bd)
+__device__ __forceinline__ void ld_words(const unsigned long long *p, unsigned long long &w0, unsigned long long &w1)
 {
-    using E = Elem<Tag>;
-    constexpr int EPV = E::kPerVec;
-#pragma unroll
-    for (int j = 0; j < kGroupVecs; ++j) {
-        const int vi = tid + j * kConsumerThreads;
-        if (vi < nvec) {
-            const int col = col0 + vi * EPV;
-            const bool masked = causal && col > row;
-            float v[EPV];
-            E::unpack(r[j], v);
-            if (causal && !masked && col + EPV - 1 > row)
-                apply_causal<EPV>(v, col, row);
-            if (masked) {
-                vec_exp<EPV>(v, mL, true);
-#pragma unroll
-                for (int e = 0; e < EPV; ++e)
-                    v[e] *= inv;
-            } else {
-                const float2 l2 = make_float2(kLog2e, kLog2e), nm = make_float2(-mL, -mL);
-                const float2 i2 = make_float2(inv, inv);
-#pragma unroll
-                for (int e = 0; e < EPV; e += 2) {
-                    const float2 t = fma2(make_float2(v[e], v[e + 1]), l2, nm);
-                    const float2 y2 = mul2(make_float2(ex2(t.x), ex2(t.y)), i2);
-                    v[e] = y2.x;
-                    v[e + 1] = y2.y;
-                }
-            }
-            store_vec<Checked>(ypart + 16 * vi, bd, E::pack(v));
-        }
-    }
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w0), "=l"(w1) : "l"(p) : "memory");
+}
+
+// The (offset, sum) of up to 32 partials, one per lane (-inf, 0 in the others),
+// in every lane: a fixed tree.
+__device__ __forceinline__ float2 combine_lanes(float2 p)
+{
+    const float o = warp_max(p.x);
+    return make_float2(o, group_sum<32>(p.y * ex2(p.x - o)));
 }
 
 template <typename Tag, bool Checked>
-__global__ void __launch_bounds__(kThreads, 1) softmax_group(const KernelArgs a)
+__global__ void __launch_bounds__(kGroupThreads, 1) softmax_group(const KernelArgs a)
 {
     using E = Elem<Tag>;
     constexpr int EPV = E::kPerVec;
     extern __shared__ __align__(1024) unsigned char smem[];
     SmemHeader &h = *reinterpret_cast<SmemHeader *>(smem);
     unsigned char *stages = smem + kSmemHeader;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int S = a.n_stages;
     const int K = a.group_k;
     const int grp = static_cast<int>(blockIdx.x) / K, rank = static_cast<int>(blockIdx.x) % K;
@@ -2176,7 +2054,8 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_group(const KernelArgs a)
             mbar_init(&h.full[s], 1);
             mbar_init(&h.empty[s], kConsumerWarps);
         }
-        h.xarrive[0] = h.xarrive[1] = 0u;
+        mbar_init(&h.xres, 1);
+        h.xarrive[0] = h.xarrive[1] = h.xleft = 0u;
         h.abort_flag = 0;
         mbar_init_fence();
     }
@@ -2192,27 +2071,54 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_group(const KernelArgs a)
             for (int s = 0; s < kMaxStages; ++s)
                 issued[s] = false;
             bool aborted = false;
-            uint32_t it = 0, posted = 0;
+            uint32_t it = 0;
+            // Rank 0 announces rows up to kClaimAhead + 1 beyond the current
+            // one; the claim after the last one announced is under way.  Every
+            // member reads a row's claim word and record while the copy of the
+            // row before is under way.  (One after the other at each row,
+            // atomic, release store, acquire load, record load and copy were a
+            // chain of about 4 us of round trips, which set the pace: fp32
+            // 768 KiB rows 4780 GB/s against 5440.)  The words carry all that their readers use, so
+            // relaxed accesses do.
+            uint32_t posted = 0, claim = 0xFFFFFFFFu;
             bool post_done = false;
-            for (uint32_t t = 0; !aborted; ++t) {
-                if (rank == 0) {
-                    // announce rows up to kClaimAhead beyond this one
-                    while (!post_done && posted <= t + kClaimAhead) {
-                        int32_t p1[kFetch];
-                        const int n = pull.next_batch(p1, 1);
-                        const uint32_t pos = n > 0 ? static_cast<uint32_t>(p1[0]) : 0xFFFFFFFFu;
-                        st_release_u64(&ring[posted % kGroupRing],
-                                       (static_cast<unsigned long long>(posted + 1) << 32) | pos);
-                        ++posted;
-                        post_done = n == 0;
-                    }
+            auto claim_next = [&]() {
+                int32_t p1[kFetch];
+                claim = pull.next_batch(p1, 1) > 0 ? static_cast<uint32_t>(p1[0]) : 0xFFFFFFFFu;
+            };
+            auto post = [&](uint32_t upto) {
+                while (rank == 0 && !post_done && posted <= upto) {
+                    st_relaxed_u64(&ring[posted % kGroupRing],
+                                   (static_cast<unsigned long long>(posted + 1) << 32) | claim);
+                    ++posted;
+                    post_done = claim == 0xFFFFFFFFu;
+                    if (!post_done)
+                        claim_next();
                 }
+            };
+            uint32_t next_pos = 0xFFFFFFFFu;
+            Item next_item{-1, 0, 0, 0, 0};
+            auto fetch = [&](uint32_t t) -> bool {
                 unsigned long long word = 0;
-                if (!wait_claim(&ring[t % kGroupRing], t + 1, &h.abort_flag, wait_limit, word)) {
+                if (!wait_claim(&ring[t % kGroupRing], t + 1, &h.abort_flag, wait_limit, word))
+                    return false;
+                next_pos = static_cast<uint32_t>(word);
+                if (next_pos < static_cast<uint32_t>(a.n_items))
+                    next_item = a.items[next_pos];
+                return true;
+            };
+            if (rank == 0)
+                claim_next();
+            post(kClaimAhead);
+            aborted = !fetch(0);
+            for (uint32_t t = 0; !aborted; ++t) {
+                if (t > 0 && !fetch(t)) {
                     aborted = true;
                     break;
                 }
-                const uint32_t pos = static_cast<uint32_t>(word);
+                const uint32_t pos = next_pos;
+                const Item item = next_item;
+                post(t + 1 + kClaimAhead);
                 const int s = static_cast<int>(it % S);
                 const uint32_t ph = (it / S) & 1u;
                 if (!mbar_wait_bounded(&h.empty[s], ph ^ 1u, &h.abort_flag, wait_limit)) {
@@ -2230,7 +2136,6 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_group(const KernelArgs a)
                 if ((a.debug & KDEBUG_WITHHOLD_STAGE0) && it == 1)
                     continue;                      // test hook: stage 0 is never filled
                 const bool in = pos < static_cast<uint32_t>(a.n_items);
-                const Item item = in ? a.items[pos] : Item{-1, 0, 0, 0, 0};
                 // this member's part (the same cut in every member)
                 const int64_t part = ((int64_t(item.C) + K - 1) / K + EPV - 1) / EPV * EPV;
                 const int64_t c0 = part * rank;
@@ -2288,183 +2193,193 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_group(const KernelArgs a)
                     mbar_wait_bounded(&h.full[s], issued_phase[s], nullptr, wait_limit);
         }
         __syncwarp();
+    } else if (warp == kConsumerWarps + 1) {
+        // ------------------------------------------------------- exchange
+        // For every row: the group's words read until all are in, combined,
+        // and handed to the consumers through shared memory.  One warp a CTA
+        // polls (16 polling the same few lines held the stores up), and the
+        // consumers never wait on global memory.
+        uint64_t t0 = 0;
+        uint32_t xt = 0;
+        for (uint32_t tries = 0; tries < (1u << 30); ++tries) {
+            const unsigned long long *xs = &xch[2 * static_cast<size_t>(xt & (kGroupSlots - 1)) * K];
+            const uint32_t tag = xt + 1;
+            float2 pw = make_float2(-INFINITY, 0.0f);
+            bool all = true;
+            if (lane < K) {
+                unsigned long long w0, w1;
+                ld_words(&xs[2 * lane], w0, w1);
+                all = static_cast<uint32_t>(w0 >> 32) == tag && static_cast<uint32_t>(w1 >> 32) == tag;
+                pw = make_float2(__uint_as_float(static_cast<uint32_t>(w0)),
+                                 __uint_as_float(static_cast<uint32_t>(w1)));
+            }
+            if (__all_sync(0xFFFFFFFFu, all)) {
+                pw = combine_lanes(pw);
+                if (lane == 0) {
+                    h.result[xt & 1] = pw;
+                    mbar_arrive(&h.xres);
+                }
+                __syncwarp();
+                ++xt;
+                t0 = 0;
+                continue;
+            }
+            // (a consumer that waits for a result gives up by itself; this
+            // warp, idle between rows, only after a long while)
+            const uint32_t left = *const_cast<volatile uint32_t *>(&h.xleft);
+            const uint64_t now = (tries & 63u) == 63u ? global_timer_ns() : 0;
+            t0 = t0 ? t0 : now;
+            if (__any_sync(0xFFFFFFFFu, left == kConsumerWarps || *const_cast<volatile int32_t *>(&h.abort_flag) ||
+                                            (now && now - t0 > 8 * wait_limit)))
+                break;
+            __nanosleep(20);
+        }
     } else {
         // ----------------------------------------------------------- consumers
-        // A member takes a row's partial straight from its stage, then writes
-        // the previous row -- held in registers (thread t of the 512 consumer
-        // threads holds its vectors t, t + 512, ...: at most kGroupVecs), whose
-        // group exchange has had this row's partial to complete -- and then
-        // moves this row from the stage into the registers and releases the
-        // stage.  One stage is held at a time; the others are in flight.
+        // Thread t of the 512 consumer threads owns the part's vectors t, t +
+        // 512, ... (at most kGroupVecs).  A row's partial is taken from its
+        // stage (read twice, for the maximum and for the sum); then the row
+        // before -- held in registers, its exchange under way meanwhile -- is
+        // written, and this row moves from the stage into the registers.  One
+        // stage is held at a time; the others are in flight.
         const bool causal = (a.flags & BSM_FLAG_CAUSAL) != 0;
         unsigned char *y = static_cast<unsigned char *>(a.y);
         const Bounds bdy{nullptr, nullptr, y, y + a.total_elems * E::kSize, a.status};
         const int tid = warp * 32 + lane;
+        const Pair l2 = pair(kLog2e, kLog2e);
         uint32_t xt = 0;            // group rows this CTA took part in (the exchange sequence)
-        uint4 rr[kGroupVecs];       // the row one behind: published, not yet written
-        StageMeta rm{};
-        uint32_t rx = 0;
-        bool rh = false;
-        // the row held in rr: poll its K partials (each two words carrying the
-        // row's tag) until all are in, combine them in rank order, write this
-        // member's part
-        auto finish = [&](unsigned long long pre0, unsigned long long pre1) -> bool {
-            const uint32_t slot = rx & (kGroupSlots - 1);
-            const uint32_t tag = rx + 1;
-            const unsigned long long *xs = &xch[2 * static_cast<size_t>(slot) * K];
-            float mv[kMaxGroup / 32], sv[kMaxGroup / 32];
-            bool in = false;
-            const uint64_t t0 = global_timer_ns();
-            for (uint32_t tries = 0; tries < (1u << 24); ++tries) {
-                bool all = true;
-#pragma unroll
-                for (int j = 0; j < kMaxGroup / 32; ++j) {
-                    const int r2 = lane + 32 * j;
-                    mv[j] = -INFINITY;
-                    sv[j] = 0.0f;
-                    if (r2 < K) {
-                        // the first round of rank `lane` was loaded early
-                        const bool early = tries == 0 && j == 0;
-                        const unsigned long long w0 = early ? pre0 : ld_relaxed_u64(&xs[2 * r2]);
-                        const unsigned long long w1 = early ? pre1 : ld_relaxed_u64(&xs[2 * r2 + 1]);
-                        all = all && static_cast<uint32_t>(w0 >> 32) == tag && static_cast<uint32_t>(w1 >> 32) == tag;
-                        mv[j] = __uint_as_float(static_cast<uint32_t>(w0));
-                        sv[j] = __uint_as_float(static_cast<uint32_t>(w1));
-                    }
-                }
-                if (__all_sync(0xFFFFFFFFu, all)) {
-                    in = true;
-                    break;
-                }
-                const int give_up = (h.abort_flag || global_timer_ns() - t0 > wait_limit) ? 1 : 0;
-                if (__any_sync(0xFFFFFFFFu, give_up))
-                    break;
-                __nanosleep(32);
-            }
-            if (!in) {
+        uint4 rr[kGroupVecs];       // the row one behind: its partial is out, it is not yet written
+        int rvec = 0;               // ... its vectors, and where they go
+        unsigned char *ry = nullptr;
+        // the row held in rr, once its group's result is in; false when that wait gave up
+        auto finish = [&]() -> bool {
+            const uint32_t par = (xt - 1) & 1u;
+            if (!__all_sync(0xFFFFFFFFu, mbar_spin_bounded(&h.xres, par, &h.abort_flag, wait_limit))) {
                 if (lane == 0) {
                     atomicOr(a.status, BSM_DEV_TIMEOUT);
                     h.abort_flag = 1;
                 }
                 return false;
             }
-            float M = mv[0];
+            const float2 t = h.result[par];
+            const float inv = __frcp_rn(t.y);
+            const Pair nm = pair(-t.x, -t.x), inv2 = pair(inv, inv);
+            if (rvec >= (kGroupVecs - 2) * kConsumerThreads) {
+                // (the usual part: only the last two vectors can be missing)
 #pragma unroll
-            for (int j = 1; j < kMaxGroup / 32; ++j)
-                M = fmaxf(M, mv[j]);
-            M = group_max<32>(M);
-            float sum = 0.0f;
+                for (int j = 0; j < kGroupVecs; ++j)
+                    if (j < kGroupVecs - 2 || tid + j * kConsumerThreads < rvec)
+                        store_vec<Checked>(ry + 16 * j * kConsumerThreads, bdy, vec_softmax<Tag>(rr[j], l2, nm, inv2));
+            } else {
 #pragma unroll
-            for (int j = 0; j < kMaxGroup / 32; ++j)
-                if (lane + 32 * j < K)
-                    sum += mv[j] == M ? sv[j] : sv[j] * ex2((mv[j] - M) * kLog2e);
-            sum = group_sum<32>(sum);
-            group_write<Tag, Checked>(rr, (rm.C * E::kSize) >> 4, tid, rm.col0, rm.row0, causal, M * kLog2e,
-                                      __frcp_rn(sum), y + rm.off * E::kSize, bdy);
-            rh = false;
+                for (int j = 0; j < kGroupVecs; ++j)
+                    if (tid + j * kConsumerThreads < rvec)
+                        store_vec<Checked>(ry + 16 * j * kConsumerThreads, bdy, vec_softmax<Tag>(rr[j], l2, nm, inv2));
+            }
             return true;
         };
-        bool failed = false;
-        for (uint32_t it = 0;; ++it) {
-            const int s = static_cast<int>(it % S);
-            const uint32_t ph = (it / S) & 1u;
+        int s = 0;
+        uint32_t ph = 0;            // the ring's stage and phase
+        bool held = false;
+        for (;;) {
             // the whole warp gives up together (the shuffles need all lanes)
             if (!__all_sync(0xFFFFFFFFu, mbar_wait_bounded(&h.full[s], ph, &h.abort_flag, wait_limit))) {
                 if (lane == 0) {
                     atomicOr(a.status, BSM_DEV_TIMEOUT);
                     h.abort_flag = 1;
                 }
-                failed = true;
+                held = false;
                 break;
             }
-            const StageMeta mt = h.meta[s];
-            if (mt.kind == KIND_DONE)
+            const int32_t kind = h.meta[s].kind;
+            if (kind == KIND_DONE)
                 break;
-            if (mt.kind != KIND_GROUP) {
-                __syncwarp();
-                if (lane == 0)
-                    mbar_arrive(&h.empty[s]);
-                continue;
-            }
-            const int nvec = (mt.C * E::kSize) >> 4;
-            const unsigned char *sbuf = stages + static_cast<size_t>(s) * a.stage_bytes;
-            Bounds bs = bdy;
-            bs.s_lo = sbuf;
-            bs.s_hi = sbuf + static_cast<size_t>(mt.C) * E::kSize;
-            // the held row's exchange words of rank `lane`, loaded halfway
-            // through this row's partial and used after it: late enough that
-            // most members have published, early enough that the second half
-            // covers the loads' latency
-            unsigned long long pre0 = 0, pre1 = 0;
-            auto poll = [&]() {
-                if (rh && lane < K) {
-                    const unsigned long long *xs = &xch[2 * static_cast<size_t>(rx & (kGroupSlots - 1)) * K];
-                    pre0 = ld_relaxed_u64(&xs[2 * lane]);
-                    pre1 = ld_relaxed_u64(&xs[2 * lane + 1]);
-                }
-            };
-            // this member's (max, sum) of its part, from the stage
-            float m_l, s_l;
-            group_partial<Tag, Checked>(sbuf, nvec, tid, mt.col0, mt.row0, causal, bs, m_l, s_l, poll);
+            if (kind == KIND_GROUP) {
+                const int C = h.meta[s].C, row = h.meta[s].row0, col0 = h.meta[s].col0;
+                const int nvec = (C * E::kSize) >> 4;
+                const unsigned char *sbuf = stages + static_cast<size_t>(s) * a.stage_bytes;
+                Bounds bs = bdy;
+                bs.s_lo = sbuf;
+                bs.s_hi = sbuf + static_cast<size_t>(C) * E::kSize;
+                auto part = [&](auto full) -> float2 {
+                    // vector j of this thread (only the last two can be missing in a full part)
+                    auto vec = [&](int j) {
+                        const int vi = tid + j * kConsumerThreads;
+                        const uint4 v = group_vec<Tag, Checked>(
+                            sbuf, vi, decltype(full)::value && j < kGroupVecs - 2 ? INT32_MAX : nvec, bs);
+                        return causal ? mask_vec<Tag>(v, col0 + vi * EPV, row) : v;
+                    };
+                    MaxAcc<Tag> mx;
 #pragma unroll
-            for (int o2 = 16; o2 >= 1; o2 >>= 1) {
-                const float mo2 = __shfl_xor_sync(0xFFFFFFFFu, m_l, o2);
-                const float so2 = __shfl_xor_sync(0xFFFFFFFFu, s_l, o2);
-                combine_ms(m_l, s_l, mo2, so2);
-            }
-            // the warps' partials: the last warp to bring its own combines them
-            // (a fixed tree over 16 lanes) and publishes the CTA's; nobody
-            // waits.  (A warp's partial of row t + 2 comes after its finish of
-            // row t, i.e. after row t's publication: two slots by row parity.)
-            const int par = xt & 1;
-            int last = 0;
-            if (lane == 0) {
-                h.partial[par][warp] = make_float2(m_l, s_l);
-                __threadfence_block();
-                last = atomicAdd(&h.xarrive[par], 1u) == static_cast<uint32_t>(kConsumerWarps - 1) ? 1 : 0;
-                if (last) {
-                    __threadfence_block();
-                    h.xarrive[par] = 0u;
-                }
-            }
-            last = __shfl_sync(0xFFFFFFFFu, last, 0);
-            if (last) {
-                __syncwarp();
-                float2 pw = lane < kConsumerWarps ? h.partial[par][lane] : make_float2(-INFINITY, 0.0f);
+                    for (int j = 0; j < kGroupVecs; ++j)
+                        mx.add(vec(j));
+                    const float o = exp_offset(warp_max(mx.get()));
+                    const Pair nm = pair(-o, -o);
+                    Pair acc = pair(0.0f, 0.0f);
 #pragma unroll
-                for (int o2 = kConsumerWarps / 2; o2 >= 1; o2 >>= 1) {
-                    const float mo2 = __shfl_xor_sync(0xFFFFFFFFu, pw.x, o2);
-                    const float so2 = __shfl_xor_sync(0xFFFFFFFFu, pw.y, o2);
-                    combine_ms(pw.x, pw.y, mo2, so2);
-                }
+                    for (int j = 0; j < kGroupVecs; ++j)
+                        acc = vec_sum<Tag>(acc, vec(j), l2, nm);
+                    const float2 a2 = halves(acc);
+                    return make_float2(o, group_sum<32>(a2.x + a2.y));
+                };
+                const bool full = nvec >= (kGroupVecs - 2) * kConsumerThreads;
+                const float2 mine = full ? part(Int<1>{}) : part(Int<0>{});
+                // the last warp to bring its partial combines the warps' (a fixed
+                // tree over 16 lanes) and publishes the CTA's.  (A warp's partial
+                // of row t + 2 comes after it has seen row t's result, i.e. after
+                // row t's publication: two slots by row parity.)
+                const int par = xt & 1;
+                int last = 0;
                 if (lane == 0) {
-                    // two self-validating words (value, row tag): 8-byte stores
-                    // are single-copy atomic, so a reader that sees the tag
-                    // sees the value written with it
-                    const uint32_t slot = xt & (kGroupSlots - 1);
-                    const unsigned long long tag = static_cast<unsigned long long>(xt + 1) << 32;
-                    unsigned long long *w = &xch[2 * (static_cast<size_t>(slot) * K + rank)];
-                    st_relaxed_u64(w, tag | __float_as_uint(pw.x));
-                    st_relaxed_u64(w + 1, tag | __float_as_uint(pw.y));
+                    h.partial[par][warp] = mine;
+                    __threadfence_block();
+                    last = atomicAdd(&h.xarrive[par], 1u) == static_cast<uint32_t>(kConsumerWarps - 1) ? 1 : 0;
+                    if (last) {
+                        __threadfence_block();
+                        h.xarrive[par] = 0u;
+                    }
                 }
+                if (__shfl_sync(0xFFFFFFFFu, last, 0)) {
+                    __syncwarp();
+                    const float2 pw =
+                        combine_lanes(lane < kConsumerWarps ? h.partial[par][lane] : make_float2(-INFINITY, 0.0f));
+                    // two self-validating words (value, row tag): a reader that
+                    // sees the tag sees the value written with it
+                    if (lane == 0) {
+                        const unsigned long long tag = static_cast<unsigned long long>(xt + 1) << 32;
+                        st_words(&xch[2 * (static_cast<size_t>(xt & (kGroupSlots - 1)) * K + rank)],
+                                 tag | __float_as_uint(pw.x), tag | __float_as_uint(pw.y));
+                    }
+                }
+                if (held && !finish()) {
+                    held = false;
+                    break;
+                }
+                // this row into the registers; the stage is free
+#pragma unroll
+                for (int j = 0; j < kGroupVecs; ++j) {
+                    const int vi = tid + j * kConsumerThreads;
+                    const uint4 v = group_vec<Tag, Checked>(sbuf, vi, nvec, bs);
+                    rr[j] = causal ? mask_vec<Tag>(v, col0 + vi * EPV, row) : v;
+                }
+                rvec = nvec;
+                ry = y + h.meta[s].off * E::kSize + 16 * tid;
+                held = true;
+                ++xt;
             }
-            // the previous row: its partials are (nearly) in by now
-            if (rh && !finish(pre0, pre1)) {
-                failed = true;
-                break;
-            }
-            // this row into the registers; the stage is free
-            group_load<Tag, Checked>(rr, sbuf, nvec, tid, bs);
             __syncwarp();
             if (lane == 0)
                 mbar_arrive(&h.empty[s]);
-            rm = mt;
-            rx = xt;
-            rh = true;
-            ++xt;
+            if (++s == S) {
+                s = 0;
+                ph ^= 1u;
+            }
         }
-        if (!failed && rh)
-            finish(0ull, 0ull);
+        if (held)
+            finish();
+        // the exchange warp leaves too
+        if (lane == 0)
+            atomicAdd(&h.xleft, 1u);
         __syncwarp();
     }
     // the last CTA out resets the queue heads, the claim rings and the
@@ -2557,7 +2472,7 @@ void launch_group(const KernelArgs &a, int grid, size_t smem, cudaStream_t st, b
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kGroupThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
