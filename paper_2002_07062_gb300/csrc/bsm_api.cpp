@@ -681,11 +681,9 @@ int plan_create_impl(bsm_plan **out, const bsm_plan_desc *d)
     const bool reg_long = long_rows > n_grp;   // long rows outside the groups
     bool team = false;                         // rows that teams of warps share
     for (const Item &it : items)
-        team = team || int64_t(it.C) * es > kLaneRowBytes;
-    p->kernel_op = d->op == BSM_OP_BACKWARD ? (reg_long ? OP_BACKWARD_LONG : OP_BACKWARD)
-                   : reg_long               ? OP_FORWARD_LONG
-                   : team                   ? OP_FORWARD_TEAM
-                                            : OP_FORWARD;
+        team = team || int64_t(it.C) * es > (d->op == BSM_OP_BACKWARD ? (es == 4 ? kLaneRowBytesBwd<4> : kLaneRowBytesBwd<2>) : kLaneRowBytes);
+    p->kernel_op = d->op == BSM_OP_BACKWARD ? (reg_long ? OP_BACKWARD_LONG : team ? OP_BACKWARD_TEAM : OP_BACKWARD)
+                                            : (reg_long ? OP_FORWARD_LONG : team ? OP_FORWARD_TEAM : OP_FORWARD);
 
     // ---- the schedule
     std::vector<int32_t> queue;      // schedule order of the patches (queue policies)

@@ -53,7 +53,8 @@ enum Op : int32_t {
     OP_FORWARD_LONG = 2, // OP_FORWARD for plans with rows longer than a stage (two passes)
     OP_BACKWARD_LONG = 3, // OP_BACKWARD for plans with rows longer than half a stage (two passes)
     OP_FORWARD_GROUP = 4, // OP_FORWARD of rows split over groups of CTAs (one read; see KernelArgs)
-    OP_FORWARD_TEAM = 5  // OP_FORWARD for plans with rows that teams of warps share (past kLaneRowBytes)
+    OP_FORWARD_TEAM = 5, // OP_FORWARD for plans with rows that teams of warps share (past kLaneRowBytes)
+    OP_BACKWARD_TEAM = 6 // OP_BACKWARD for such plans (past kLaneRowBytesBwd)
 };
 
 // Rows of more bytes than this (up to a stage) are shared by a team of 1 to 16
@@ -65,6 +66,11 @@ enum Op : int32_t {
 // bounded the old routines: a stage of one 64 KiB row left 3 of 16 warps
 // busy, each on a serial chain of shared loads.
 constexpr int kLaneRowBytes = 2048;
+// The backward pass's (y and dy as at most 32 floats a lane).  One
+// warp a row (two sweeps over shared memory) against teams, 512 MiB of y and
+// dy: bf16 16 KiB rows 6550 -> 7055 GB/s, 32 KiB 4640 -> 7050, 56 KiB 3380 ->
+// 6900; fp32 24 KiB 6680 -> 7050, 48 KiB 6370 -> 7000.
+template <int ElemSize> constexpr int kLaneRowBytesBwd = ElemSize == 4 ? 2048 : 1024;
 
 // Rows split over groups of CTAs (OP_FORWARD_GROUP): group g is CTAs
 // [g*K, g*K + K); its rank-0 CTA claims rows and announces them in the

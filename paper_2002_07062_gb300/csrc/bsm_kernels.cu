@@ -786,6 +786,17 @@ template <typename Tag> __device__ __forceinline__ Pair vec_sum(Pair acc, uint4 
     return pair_add(acc, p[0]);
 }
 
+// A vector of the element type from its element pairs.
+template <typename Tag> __device__ __forceinline__ uint4 pack_pairs(const float2 *y)
+{
+    if constexpr (Elem<Tag>::kSize == 4)
+        return make_uint4(__float_as_uint(y[0].x), __float_as_uint(y[0].y), __float_as_uint(y[1].x),
+                          __float_as_uint(y[1].y));
+    else
+        return make_uint4(pack_bf16x2(y[0].x, y[0].y), pack_bf16x2(y[1].x, y[1].y), pack_bf16x2(y[2].x, y[2].y),
+                          pack_bf16x2(y[3].x, y[3].y));
+}
+
 // 2^(v*log2e - mL) * inv of one vector, packed.
 template <typename Tag> __device__ __forceinline__ uint4 vec_softmax(uint4 r, Pair l2, Pair nm, Pair inv2)
 {
@@ -794,12 +805,7 @@ template <typename Tag> __device__ __forceinline__ uint4 vec_softmax(uint4 r, Pa
 #pragma unroll
     for (int k = 0; k < N; ++k)
         y[k] = halves(pair_mul(pair_ex2(pair_fma(vec_pair<Tag>(r, k), l2, nm)), inv2));
-    if constexpr (Elem<Tag>::kSize == 4)
-        return make_uint4(__float_as_uint(y[0].x), __float_as_uint(y[0].y), __float_as_uint(y[1].x),
-                          __float_as_uint(y[1].y));
-    else
-        return make_uint4(pack_bf16x2(y[0].x, y[0].y), pack_bf16x2(y[1].x, y[1].y), pack_bf16x2(y[2].x, y[2].y),
-                          pack_bf16x2(y[N - 1].x, y[N - 1].y));
+    return pack_pairs<Tag>(y);
 }
 
 // Maximum over the warp, in every lane (no operand is NaN: see MaxAcc).
@@ -812,25 +818,24 @@ __device__ __forceinline__ float warp_max(float m)
 
 // A row shared by a team of W consumer warps (wi = this warp's index in it;
 // W = 1, 2, 4, 8 or 16): lane l of warp wi owns the vectors wi*32 + l, + 32 W,
-// ..., V of them in registers (V = 6 or 8: more than 4 exist, so only the last two can be
-// missing in some lanes; 8 hold the whole row up to W * 4 KiB), further ones
-// (rows of 64 to 113 KiB on 16 warps) read again from the stage by each
-// sweep.  W and V are compile-time, so that no address outlives its use.  A warp takes its maximum's offset o_w (the rounded
-// m_w log2 e) and s_w, the sum of 2^(v log2 e - o_w); the team's warps
-// exchange (o_w, s_w) once (`part`: the team's slots) behind one bounded
-// barrier; every warp combines them in a fixed tree, S = sum s_w 2^(o_w - O),
-// and writes 2^(v log2 e - O) / S.  Taking the rounded offsets through the
-// exchange makes their rounding cancel in the quotient, as for a row of one
-// warp.  Two exponentials per element, one exchange per row.  All in fp32;
-// which warps share a row depends on its length only.
+// ..., V of them in registers (the first Full exist in every lane; 8 hold the
+// whole row up to W * 4 KiB), further ones (rows of 64 to 113 KiB on 16 warps)
+// read again from the stage by each sweep.  W and V are compile-time, so that
+// no address outlives its use.  A warp takes its maximum's offset o_w (see
+// exp_offset) and s_w, the sum of 2^(v log2 e - o_w); exchange() turns the pair
+// into the row's: O = max o_w and S = sum s_w 2^(o_w - O), in a fixed tree, the
+// same in every warp; the warp writes 2^(v log2 e - O) / S.  (Exchanging the
+// maxima themselves cost accuracy: the rounding of m log2 e then differs from
+// warp to warp; 1.0e-7 against 7.2e-8 on a ragged fp32 batch.)  Two
+// exponentials per element, one exchange per row.  All in fp32; which warps
+// share a row depends on its length only.
 //
 // release() is called once the warp needs the stage no more; returns false
 // when the exchange's wait gave up.
-template <typename Tag, bool Checked, int W, int V, typename Release>
+template <typename Tag, bool Checked, int W, int V, int Full, typename Exchange, typename Release>
 __device__ __forceinline__ bool row_team(const unsigned char *srow, unsigned char *yrow, int nvec, int row,
-                                         bool causal, int wi, int lane, const Bounds &bd, uint64_t *bar,
-                                         uint32_t parity, float2 *part, const volatile int32_t *abort,
-                                         uint64_t limit_ns, Release &&release)
+                                         bool causal, int col0, int wi, int lane, const Bounds &bd,
+                                         Exchange &&exchange, Release &&release)
 {
     using E = Elem<Tag>;
     constexpr int EPV = E::kPerVec;
@@ -849,15 +854,15 @@ __device__ __forceinline__ bool row_team(const unsigned char *srow, unsigned cha
     uint4 r[V];
 #pragma unroll
     for (int j = 0; j < V; ++j)
-        r[j] = fetch(t0 + j * step, j < V - 2 || t0 + j * step < nvec);
+        r[j] = fetch(t0 + j * step, j < Full || t0 + j * step < nvec);
     if (causal) {
 #pragma unroll
         for (int j = 0; j < V; ++j)
-            r[j] = mask_vec<Tag>(r[j], (t0 + j * step) * EPV, row);
+            r[j] = mask_vec<Tag>(r[j], col0 + (t0 + j * step) * EPV, row);
     }
     auto fetch_tail = [&](int vi) -> uint4 {
         const uint4 u = fetch(vi, true);
-        return causal ? mask_vec<Tag>(u, vi * EPV, row) : u;
+        return causal ? mask_vec<Tag>(u, col0 + vi * EPV, row) : u;
     };
     MaxAcc<Tag> mx;
 #pragma unroll
@@ -868,7 +873,7 @@ __device__ __forceinline__ bool row_team(const unsigned char *srow, unsigned cha
             mx.add(fetch_tail(vi));
     else
         release();
-    float mL = exp_offset(warp_max(mx.get()));
+    const float mL = exp_offset(warp_max(mx.get()));
     const Pair l2 = pair(kLog2e, kLog2e);
     Pair nm = pair(-mL, -mL), acc = pair(0.0f, 0.0f);
 #pragma unroll
@@ -878,20 +883,11 @@ __device__ __forceinline__ bool row_team(const unsigned char *srow, unsigned cha
         for (int vi = t0 + V * step; vi < nvec; vi += step)
             acc = vec_sum<Tag>(acc, fetch_tail(vi), l2, nm);
     const float2 a2 = halves(acc);
-    float s = group_sum<32>(a2.x + a2.y);
-    if (W > 1) {
-        if (lane == 0) {
-            part[wi] = make_float2(mL, s);
-            mbar_arrive(bar);
-        }
-        if (!__all_sync(0xFFFFFFFFu, mbar_spin_bounded(bar, parity, abort, limit_ns)))
-            return false;
-        const int k = lane & 15;
-        const float2 pw = k < W ? part[k] : make_float2(-INFINITY, 0.0f);
-        mL = warp_max(pw.x);
-        nm = pair(-mL, -mL);
-        s = group_sum<16>(pw.y * ex2(pw.x - mL));
-    }
+    float2 os = make_float2(mL, group_sum<32>(a2.x + a2.y));
+    if (!exchange(os))
+        return false;
+    nm = pair(-os.x, -os.x);
+    const float s = os.y;
     const float inv = __frcp_rn(s);
     const Pair inv2 = pair(inv, inv);
     // the write unpacks the vectors again: kept unpacked from the sum on, they
@@ -902,7 +898,7 @@ __device__ __forceinline__ bool row_team(const unsigned char *srow, unsigned cha
     unsigned char *yp = yrow + 16 * t0;
 #pragma unroll
     for (int j = 0; j < V; ++j) {
-        if (j < V - 2 || t0 + j * step < nvec)
+        if (j < Full || t0 + j * step < nvec)
             store_vec<Checked>(yp + 16 * j * step, bd, vec_softmax<Tag>(r[j], l2, nm, inv2));
     }
     if (tail) {
@@ -959,37 +955,87 @@ __device__ __forceinline__ void row_bwd_registers(const unsigned char *sy, const
     }
 }
 
-template <typename Tag, bool Checked>
-__device__ __forceinline__ void row_bwd_smem(const unsigned char *sy, const unsigned char *sdy,
-                                             unsigned char *dxrow, int nvec, int lane, const Bounds &by,
-                                             const Bounds &bdy)
+// A longer row, shared by a team of W warps as in row_team: the vectors wi*32
+// + l, + 32 W, ... of y and of dy, four of each in registers (the last two can
+// be missing in some lanes; the whole row up to W * 2 KiB), further ones (rows
+// of 32 to 56 KiB on 16 warps, of 2 to 3 KiB on one) read again from the
+// stage.  The warps' dot
+// products are exchanged once and added in a fixed tree.
+constexpr int kTeamVecsBwd = 4;
+
+template <typename Tag, bool Checked, int W, int Full, typename Exchange, typename Release>
+__device__ __forceinline__ bool row_team_bwd(const unsigned char *sy, const unsigned char *sdy, unsigned char *dxrow,
+                                             int nvec, int wi, int lane, const Bounds &by, const Bounds &bdy,
+                                             Exchange &&exchange, Release &&release)
 {
-    using E = Elem<Tag>;
-    constexpr int EPV = E::kPerVec;
-    float yv[EPV], dv[EPV], pr[EPV];
-    uint4 ry, rd;
-    float dot = 0.0f;
-    for (int vi = lane; vi < nvec; vi += 32) {
-        if (!load_vec<Checked>(sy + 16 * vi, by, ry) || !load_vec<Checked>(sdy + 16 * vi, bdy, rd))
-            continue;
-        E::unpack(ry, yv);
-        E::unpack(rd, dv);
+    constexpr int V = kTeamVecsBwd, N = Elem<Tag>::kPerVec / 2, step = W * 32;
+    const int t0 = wi * 32 + lane;
+    const bool tail = (W == 1 || W == 16) && nvec > V * step;
+    auto fetch = [&](const unsigned char *src, int vi, bool in, const Bounds &b) -> uint4 {
+        uint4 r = make_uint4(0u, 0u, 0u, 0u);
+        if (in) {
+            uint4 u;
+            if (load_vec<Checked>(src + 16 * vi, b, u))
+                r = u;
+        }
+        return r;
+    };
+    auto add = [&](Pair acc, uint4 a, uint4 b) -> Pair {
 #pragma unroll
-        for (int e = 0; e < EPV; ++e)
-            pr[e] = yv[e] * dv[e];
-        dot += tree_sum<EPV>(pr);
-    }
-    dot = group_sum<32>(dot);
-    for (int vi = lane; vi < nvec; vi += 32) {
-        if (!load_vec<Checked>(sy + 16 * vi, by, ry) || !load_vec<Checked>(sdy + 16 * vi, bdy, rd))
-            continue;
-        E::unpack(ry, yv);
-        E::unpack(rd, dv);
+        for (int k = 0; k < N; ++k)
+            acc = pair_fma(vec_pair<Tag>(a, k), vec_pair<Tag>(b, k), acc);
+        return acc;
+    };
+    uint4 yv[V], dv[V];
 #pragma unroll
-        for (int e = 0; e < EPV; ++e)
-            yv[e] = yv[e] * (dv[e] - dot);
-        store_vec<Checked>(dxrow + 16 * vi, by, E::pack(yv));
+    for (int j = 0; j < V; ++j) {
+        const int vi = t0 + j * step;
+        const bool in = j < Full || vi < nvec;
+        yv[j] = fetch(sy, vi, in, by);
+        dv[j] = fetch(sdy, vi, in, bdy);
     }
+    Pair acc = pair(0.0f, 0.0f), acc2 = acc;
+#pragma unroll
+    for (int j = 0; j < V; j += 2) {
+        acc = add(acc, yv[j], dv[j]);
+        acc2 = add(acc2, yv[j + 1], dv[j + 1]);
+    }
+    if (tail) {
+        for (int vi = t0 + V * step; vi < nvec; vi += step)
+            acc = add(acc, fetch(sy, vi, true, by), fetch(sdy, vi, true, bdy));
+    } else {
+        release();
+    }
+    const float2 a2 = halves(pair_add(acc, acc2));
+    float dot = group_sum<32>(a2.x + a2.y);
+    if (!exchange(dot))
+        return false;
+    const Pair nd = pair(-dot, -dot);
+    auto dx = [&](uint4 a, uint4 b) -> uint4 {
+        float2 o[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            o[k] = halves(pair_mul(vec_pair<Tag>(a, k), pair_add(vec_pair<Tag>(b, k), nd)));
+        return pack_pairs<Tag>(o);
+    };
+    // (unpacked again for the write, as in row_team)
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        asm volatile("" : "+r"(yv[j].x), "+r"(yv[j].y), "+r"(yv[j].z), "+r"(yv[j].w));
+        asm volatile("" : "+r"(dv[j].x), "+r"(dv[j].y), "+r"(dv[j].z), "+r"(dv[j].w));
+    }
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        const int vi = t0 + j * step;
+        if (j < Full || vi < nvec)
+            store_vec<Checked>(dxrow + 16 * vi, by, dx(yv[j], dv[j]));
+    }
+    if (tail) {
+        for (int vi = t0 + V * step; vi < nvec; vi += step)
+            store_vec<Checked>(dxrow + 16 * vi, by, dx(fetch(sy, vi, true, by), fetch(sdy, vi, true, bdy)));
+        release();
+    }
+    return true;
 }
 
 // Backward rows of a stage, dealt like consume_stage's: groups of G = 32/T
@@ -1032,16 +1078,11 @@ __device__ __forceinline__ int consume_stage_bwd(const unsigned char *sbuf, int 
     if (nvec <= 32)
         return rows_bwd_registers<Tag, Checked, 16, 2>(sbuf, half, mt, ybase, row_bytes, nvec, first, lane, by,
                                                        bdy);
-    if (nvec <= 64)
+    if (VMAX == 2 || nvec <= 64)
         return rows_bwd_registers<Tag, Checked, 32, 2>(sbuf, half, mt, ybase, row_bytes, nvec, first, lane, by,
                                                        bdy);
-    if (VMAX >= 4 && nvec <= 128)
-        return rows_bwd_registers<Tag, Checked, 32, (VMAX >= 4 ? 4 : 2)>(sbuf, half, mt, ybase, row_bytes, nvec,
-                                                                         first, lane, by, bdy);
-    for (int r = first; r < mt.nrows; r += kConsumerWarps)
-        row_bwd_smem<Tag, Checked>(sbuf + (size_t)r * row_bytes, sbuf + half + (size_t)r * row_bytes,
-                                   ybase + (size_t)r * row_bytes, nvec, lane, by, bdy);
-    return mt.nrows;
+    // fp32 (bf16 rows of more than 64 vectors go to teams)
+    return rows_bwd_registers<Tag, Checked, 32, VMAX>(sbuf, half, mt, ybase, row_bytes, nvec, first, lane, by, bdy);
 }
 
 // ------------------------------------------------------------ long rows
@@ -1201,6 +1242,17 @@ __device__ __forceinline__ int team_warps(int nvec)
     return nvec <= 256 ? 1 : nvec <= 512 ? 2 : nvec <= 1024 ? 4 : nvec <= 2048 ? 8 : 16;
 }
 
+// Backward: half as many vectors of each of y and dy fit, but a warp by itself
+// takes rows of up to 192 vectors (64 of them read from the stage twice: bf16
+// rows of 2064 bytes 7080 GB/s, on two warps 6634).
+__device__ __forceinline__ int team_warps_bwd(int nvec) { return nvec <= 192 ? 1 : team_warps(2 * nvec); }
+
+// The barrier of a team (teams of one warp use none).
+__device__ __forceinline__ uint64_t *team_bar(SmemHeader &h, int W, int team)
+{
+    return W == 16 ? &h.xwarp : &h.team[(W == 8 ? 12 : W == 4 ? 8 : 0) + (W == 1 ? 0 : team)];
+}
+
 // A consumer warp's view of the exchanges it took part in: bit W (2, 4, 8, 16)
 // is the phase of its team of W (16: xwarp, long rows too), which is also
 // the half of SmemHeader::partial that the next one uses; the bits from
@@ -1238,7 +1290,7 @@ __device__ __forceinline__ bool rows_team(SmemHeader &h, const unsigned char *sb
 {
     constexpr int teams = kConsumerWarps / W;
     const int team = warp / W;
-    uint64_t *bar = W == 16 ? &h.xwarp : &h.team[(W == 8 ? 12 : W == 4 ? 8 : 0) + (W == 1 ? 0 : team)];
+    uint64_t *bar = team_bar(h, W, team);
     int r = static_cast<int>((team + teams - (seen / W) % teams) % teams);
     int q = 0, qstep = 0;
     if (causal) {
@@ -1250,12 +1302,27 @@ __device__ __forceinline__ bool rows_team(SmemHeader &h, const unsigned char *sb
     for (; r < mt.nrows; r += teams) {
         const uint32_t par = (xs & W) ? 1u : 0u;
         const bool last = r + teams >= mt.nrows;
-        if (!row_team<Tag, Checked, W, V>(sbuf + (size_t)r * row_bytes, ybase + (size_t)r * row_bytes, nvec, q, causal,
-                                       warp % W, lane, bd, bar, par, &h.partial[par][team * W], &h.abort_flag,
-                                       limit_ns, [&]() {
-                                           if (last)
-                                               release();
-                                       }))
+        float2 *part = &h.partial[par][team * W];
+        auto exchange = [&](float2 &os) -> bool {
+            if (W == 1)
+                return true;
+            if (lane == 0) {
+                part[warp % W] = os;
+                mbar_arrive(bar);
+            }
+            if (!__all_sync(0xFFFFFFFFu, mbar_spin_bounded(bar, par, &h.abort_flag, limit_ns)))
+                return false;
+            const int k = lane & 15;
+            const float2 pw = k < W ? part[k] : make_float2(-INFINITY, 0.0f);
+            os.x = warp_max(pw.x);
+            os.y = group_sum<16>(pw.y * ex2(pw.x - os.x));
+            return true;
+        };
+        if (!row_team<Tag, Checked, W, V, V - 2>(sbuf + (size_t)r * row_bytes, ybase + (size_t)r * row_bytes, nvec, q,
+                                                 causal, 0, warp % W, lane, bd, exchange, [&]() {
+                                                     if (last)
+                                                         release();
+                                                 }))
             return false;
         if (W > 1)
             xs ^= W;
@@ -1286,6 +1353,73 @@ __device__ __forceinline__ bool consume_stage_team(SmemHeader &h, const unsigned
                                                   limit_ns, xs, release);
         return rows_team<Tag, Checked, w_, kTeamVecs>(h, sbuf, mt, yb, row_bytes, nvec, causal, seen, warp, lane, bd,
                                                       limit_ns, xs, release);
+    };
+    return W == 1 ? go(Int<1>{}) : W == 2 ? go(Int<2>{}) : W == 4 ? go(Int<4>{}) : W == 8 ? go(Int<8>{}) : go(Int<16>{});
+}
+
+// The backward pass's rows of one stage that teams share; as rows_team.
+template <typename Tag, bool Checked, int W, typename Release>
+__device__ __forceinline__ bool rows_team_bwd(SmemHeader &h, const unsigned char *sbuf, int half, const StageMeta &mt,
+                                              unsigned char *ybase, int row_bytes, int nvec, uint32_t seen, int warp,
+                                              int lane, const Bounds &by, const Bounds &bdy, uint64_t limit_ns,
+                                              uint32_t &xs, Release &&release)
+{
+    constexpr int teams = kConsumerWarps / W;
+    const int team = warp / W;
+    uint64_t *bar = team_bar(h, W, team);
+    int r = static_cast<int>((team + teams - (seen / W) % teams) % teams);
+    if (r >= mt.nrows)
+        release();
+    for (; r < mt.nrows; r += teams) {
+        const uint32_t par = (xs & W) ? 1u : 0u;
+        const bool last = r + teams >= mt.nrows;
+        const size_t o = (size_t)r * row_bytes;
+        float2 *part = &h.partial[par][team * W];
+        auto exchange = [&](float &dot) -> bool {
+            if (W == 1)
+                return true;
+            if (lane == 0) {
+                part[warp % W] = make_float2(dot, 0.0f);
+                mbar_arrive(bar);
+            }
+            if (!__all_sync(0xFFFFFFFFu, mbar_spin_bounded(bar, par, &h.abort_flag, limit_ns)))
+                return false;
+            const int k = lane & 15;
+            dot = group_sum<16>(k < W ? part[k].x : 0.0f);
+            return true;
+        };
+        if (!row_team_bwd<Tag, Checked, W, kTeamVecsBwd - 2>(sbuf + o, sbuf + half + o, ybase + o, nvec, warp % W, lane,
+                                                             by, bdy, exchange, [&]() {
+                                                                 if (last)
+                                                                     release();
+                                                             }))
+            return false;
+        if (W > 1)
+            xs ^= W;
+    }
+    return true;
+}
+
+template <typename Tag, bool Checked, typename Release>
+__device__ __forceinline__ bool consume_stage_team_bwd(SmemHeader &h, const unsigned char *sbuf, int half,
+                                                       const StageMeta &mt, unsigned char *y, uint32_t seen, int warp,
+                                                       int lane, Bounds by, uint64_t limit_ns, uint32_t &xs,
+                                                       Release &&release)
+{
+    const int row_bytes = mt.C * Elem<Tag>::kSize;
+    const int nvec = row_bytes >> 4;
+    unsigned char *yb = y + mt.off * Elem<Tag>::kSize;
+    by.s_lo = sbuf;
+    by.s_hi = sbuf + (size_t)mt.nrows * row_bytes;
+    Bounds bdy = by;
+    bdy.s_lo = sbuf + half;
+    bdy.s_hi = sbuf + half + (size_t)mt.nrows * row_bytes;
+    const int W = team_warps_bwd(nvec);
+    if (W > 1 && !team_switch(h, W, lane, limit_ns, xs))
+        return false;
+    auto go = [&](auto w) {
+        return rows_team_bwd<Tag, Checked, decltype(w)::value>(h, sbuf, half, mt, yb, row_bytes, nvec, seen, warp, lane,
+                                                               by, bdy, limit_ns, xs, release);
     };
     return W == 1 ? go(Int<1>{}) : W == 2 ? go(Int<2>{}) : W == 4 ? go(Int<4>{}) : W == 8 ? go(Int<8>{}) : go(Int<16>{});
 }
@@ -1472,9 +1606,10 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
     // the long-row machinery is compiled into its own instance, so plans
     // without long rows do not pay its registers
     constexpr bool kLong = Op == OP_FORWARD_LONG || Op == OP_BACKWARD_LONG;
-    constexpr bool kBwd = Op == OP_BACKWARD || Op == OP_BACKWARD_LONG;
+    constexpr bool kBwd = Op == OP_BACKWARD || Op == OP_BACKWARD_LONG || Op == OP_BACKWARD_TEAM;
     // likewise the rows that teams of warps share
-    constexpr bool kTeam = Op == OP_FORWARD_TEAM || Op == OP_FORWARD_LONG;
+    constexpr bool kTeam = kLong || Op == OP_FORWARD_TEAM || Op == OP_BACKWARD_TEAM;
+    constexpr int kLaneVecs = (kBwd ? kLaneRowBytesBwd<E::kSize> : kLaneRowBytes) / 16;
     extern __shared__ __align__(1024) unsigned char smem[];
     SmemHeader &h = *reinterpret_cast<SmemHeader *>(smem);
     unsigned char *stages = smem + kSmemHeader;
@@ -1907,14 +2042,20 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
             if (Checked && (mt.nrows <= 0 || mt.C <= 0 || (int64_t)mt.nrows * mt.C * E::kSize > cap)) {
                 if (lane == 0)
                     check_fail(a.status, 4, static_cast<uint64_t>(mt.nrows), static_cast<uint64_t>(mt.C));
-            } else if (kTeam && nvec > kLaneRowBytes / 16) {
-                const bool ok = consume_stage_team<Tag, Checked>(
-                    h, stages + (size_t)s * a.stage_bytes, mt, y, causal, groups_seen, warp, lane, bd, wait_limit, xs,
-                    [&]() {
-                        __syncwarp();
-                        if (lane == 0)
-                            mbar_arrive(&h.empty[s]);
-                    });
+            } else if (kTeam && nvec > kLaneVecs) {
+                auto release = [&]() {
+                    __syncwarp();
+                    if (lane == 0)
+                        mbar_arrive(&h.empty[s]);
+                };
+                bool ok;
+                if constexpr (kBwd)
+                    ok = consume_stage_team_bwd<Tag, Checked>(h, stages + (size_t)s * a.stage_bytes, a.stage_bytes / 2,
+                                                              mt, y, groups_seen, warp, lane, bd, wait_limit, xs,
+                                                              release);
+                else
+                    ok = consume_stage_team<Tag, Checked>(h, stages + (size_t)s * a.stage_bytes, mt, y, causal,
+                                                          groups_seen, warp, lane, bd, wait_limit, xs, release);
                 if (!ok) {
                     if (lane == 0) {
                         atomicOr(a.status, BSM_DEV_TIMEOUT);
@@ -1922,7 +2063,8 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
                     }
                     break;
                 }
-                groups_seen += static_cast<uint32_t>(mt.nrows) * team_warps(nvec);
+                groups_seen +=
+                    static_cast<uint32_t>(mt.nrows) * (kBwd ? team_warps_bwd(nvec) : team_warps(nvec));
                 continue;                  // the stage is released
             } else {
                 const int first = static_cast<int>((warp + kConsumerWarps - groups_seen % kConsumerWarps) %
@@ -1947,7 +2089,7 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
 // length (whole 16-byte vectors; the last may be shorter or empty), and the K
 // CTAs of a group each stage one part in one stage: every element is read
 // from memory once.  Each CTA takes its part's (offset, sum) -- warps, then
-// the CTA in a fixed tree, the offset the rounded max * log2 e as in row_team
+// the CTA in a fixed tree, the offset as in row_team
 // -- and publishes it in global memory as two words tagged with the row's
 // sequence number; every member then reads the K partials (one per lane)
 // until all carry the tag, combines them in the same fixed tree, and writes
@@ -2416,9 +2558,13 @@ int kernel_set_smem_limit(int bytes)
         reinterpret_cast<const void *>(softmax_persistent<BF16, OP_FORWARD, true>),
         reinterpret_cast<const void *>(softmax_persistent<BF16, OP_FORWARD_TEAM, true>),
         reinterpret_cast<const void *>(softmax_persistent<F32, OP_BACKWARD, false>),
+        reinterpret_cast<const void *>(softmax_persistent<F32, OP_BACKWARD_TEAM, false>),
         reinterpret_cast<const void *>(softmax_persistent<BF16, OP_BACKWARD, false>),
+        reinterpret_cast<const void *>(softmax_persistent<BF16, OP_BACKWARD_TEAM, false>),
         reinterpret_cast<const void *>(softmax_persistent<F32, OP_BACKWARD, true>),
+        reinterpret_cast<const void *>(softmax_persistent<F32, OP_BACKWARD_TEAM, true>),
         reinterpret_cast<const void *>(softmax_persistent<BF16, OP_BACKWARD, true>),
+        reinterpret_cast<const void *>(softmax_persistent<BF16, OP_BACKWARD_TEAM, true>),
         reinterpret_cast<const void *>(softmax_persistent<F32, OP_FORWARD_LONG, false>),
         reinterpret_cast<const void *>(softmax_persistent<BF16, OP_FORWARD_LONG, false>),
         reinterpret_cast<const void *>(softmax_persistent<F32, OP_FORWARD_LONG, true>),
@@ -2501,6 +2647,11 @@ int launch_softmax(const KernelArgs &a, int dtype, int op, int grid, void *strea
             launch_one<F32, OP_BACKWARD>(a, grid, smem, st, checked);
         else
             launch_one<BF16, OP_BACKWARD>(a, grid, smem, st, checked);
+    } else if (op == OP_BACKWARD_TEAM) {
+        if (dtype == BSM_F32)
+            launch_one<F32, OP_BACKWARD_TEAM>(a, grid, smem, st, checked);
+        else
+            launch_one<BF16, OP_BACKWARD_TEAM>(a, grid, smem, st, checked);
     } else if (op == OP_BACKWARD_LONG) {
         if (dtype == BSM_F32)
             launch_one<F32, OP_BACKWARD_LONG>(a, grid, smem, st, checked);

@@ -122,3 +122,57 @@ def test_withheld_stage_times_out_on_team_rows():
     assert bsm.bsm_device_status() == 0
     check_all_against_oracle(w, to_host(y))
     p.close()
+
+
+# backward: 16-byte vectors of y (and of dy) around every switch; 3616 fill half a stage
+BWD_EDGES = [65, 96, 97, 128, 129, 192, 193, 256, 257, 400, 512, 513, 800, 1024, 1025, 1600, 2048, 2049, 3615, 3616]
+
+
+@pytest.mark.parametrize("nvec", BWD_EDGES)
+@pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
+def test_backward_row_lengths_at_the_edges(nvec, dtype):
+    import torch
+    from test_backward_gpu import _check, _inputs
+    C = nvec * (4 if dtype == workload.F32 else 8)
+    w = workload.uniform("team bwd", dtype, 3, 37, C, 3.0, 0x7EE0 + nvec).materialize()
+    y, dy = _inputs(w)
+    yd, dyd = to_device(y), to_device(dy)
+    outs = []
+    for p in POLICIES:
+        dx = torch.full_like(yd, float("nan"))
+        bsm.bsm_softmax_backward(yd, dyd, dx, w.nslices, 37, C, dtype, p)
+        outs.append(dx)
+    bsm.bsm_softmax_backward(yd, dyd, dyd, w.nslices, 37, C, dtype, bsm.POLICY_DYNAMIC)   # in place
+    torch.cuda.synchronize()
+    assert bsm.bsm_device_status() == 0
+    for o in outs[1:] + [dyd]:
+        assert torch.equal(bits(o), bits(outs[0]))
+    _check(w, y, dy, to_host(outs[0]))
+
+
+@pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
+def test_backward_team_sizes_mixed_in_one_batch(dtype):
+    import torch
+    from test_backward_gpu import _check, _inputs
+    per = 4 if dtype == workload.F32 else 8
+    rng = np.random.default_rng(0x7EF0 + dtype)
+    nvec = rng.choice(BWD_EDGES + [8, 40], 200)
+    nvec[rng.choice(200, 4, replace=False)] = 5000           # and rows longer than half a stage
+    rows = rng.integers(1, 6, 200).astype(np.int32)
+    cols = (nvec * per).astype(np.int32)
+    sizes = rows.astype(np.int64) * cols
+    off = np.concatenate([[0], np.cumsum(sizes)[:-1]]).astype(np.int64)
+    w = workload.Workload("team bwd mix", dtype, rows, cols, off, 0, 0x7EF1, 3.0)
+    w.materialize()
+    y, dy = _inputs(w)
+    yd, dyd = to_device(y), to_device(dy)
+    outs = []
+    for p in POLICIES:
+        dx = torch.full_like(yd, float("nan"))
+        bsm.bsm_softmax_backward_ragged(yd, dyd, dx, w.offsets, w.rows, w.cols, dtype, p)
+        outs.append(dx)
+    torch.cuda.synchronize()
+    assert bsm.bsm_device_status() == 0
+    for o in outs[1:]:
+        assert torch.equal(bits(o), bits(outs[0]))
+    _check(w, y, dy, to_host(outs[0]))
