@@ -746,11 +746,13 @@ template <> struct MaxAcc<BF16> {
     }
 };
 
-// The exponents' offset for a maximum m: m * log2 e, no lower than the lowest
-// float.  At that floor (m = -inf, or a mask of the type's lowest value in
-// every element seen) v*log2e - offset is -inf or far below 0 and adds 0 (NaN
-// for a NaN), where m * log2 e = -inf would give inf - inf.
-__device__ __forceinline__ float exp_offset(float m) { return fmaxf(m * kLog2e, -3.402823466e38f); }
+// The exponents' offset for a maximum m: m * log2 e rounded down to a whole
+// number, no lower than the lowest float.  Whole: then sums taken with
+// different offsets are brought together by powers of two, without rounding.
+// No lower than the lowest float: there (m = -inf, or a mask of the type's
+// lowest value in every element seen) v*log2e - offset is -inf or far below 0
+// and adds 0 (NaN for a NaN), where m * log2 e = -inf would give inf - inf.
+__device__ __forceinline__ float exp_offset(float m) { return fmaxf(floorf(m * kLog2e), -3.402823466e38f); }
 
 // Element pair k of a vector as loaded.
 template <typename Tag> __device__ __forceinline__ Pair vec_pair(uint4 r, int k);
