@@ -136,16 +136,16 @@ def lib():
     sig = {
         "bsm_softmax": ([vp, vp, i64, i64, i64, ctypes.c_int, ctypes.c_int, vp], ctypes.c_int),
         "bsm_softmax_ex": ([vp, vp, i64, i64, i64, ctypes.c_int, ctypes.c_int, u32, vp], ctypes.c_int),
-        "bsm_softmax_ragged": ([vp, vp, i64, c_i64p, c_i32p, c_i32p, ctypes.c_int, ctypes.c_int, u32,
-                                vp], ctypes.c_int),
+        # (host arrays as addresses: a typed pointer object costs about 2 us a call to make)
+        "bsm_softmax_ragged": ([vp, vp, i64, vp, vp, vp, ctypes.c_int, ctypes.c_int, u32, vp], ctypes.c_int),
         "bsm_softmax_noalloc": ([vp, vp, i64, i64, i64, ctypes.c_int, u32, vp], ctypes.c_int),
         "bsm_softmax_host": ([vp, vp, i64, i64, i64, ctypes.c_int, ctypes.c_int, u32, vp], ctypes.c_int),
         "bsm_bmm": ([vp, vp, vp, i64, i64, i64, i64, ctypes.c_int, ctypes.c_int, vp], ctypes.c_int),
         "bsm_bmm_ex": ([vp, vp, vp, i64, i64, i64, i64, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                         ctypes.c_int, ctypes.c_int, vp], ctypes.c_int),
         "bsm_softmax_backward": ([vp, vp, vp, i64, i64, i64, ctypes.c_int, ctypes.c_int, vp], ctypes.c_int),
-        "bsm_softmax_backward_ragged": ([vp, vp, vp, i64, c_i64p, c_i32p, c_i32p, ctypes.c_int,
-                                         ctypes.c_int, vp], ctypes.c_int),
+        "bsm_softmax_backward_ragged": ([vp, vp, vp, i64, vp, vp, vp, ctypes.c_int, ctypes.c_int, vp],
+                                        ctypes.c_int),
         "bsm_plan_desc_init": ([ctypes.POINTER(PlanDesc)], ctypes.c_int),
         "bsm_plan_create": ([ctypes.POINTER(vp), ctypes.POINTER(PlanDesc)], ctypes.c_int),
         "bsm_plan_execute": ([vp, vp], ctypes.c_int),
@@ -171,7 +171,7 @@ def lib():
         "bsm_device_status": ([ctypes.c_int, ctypes.POINTER(u32)], ctypes.c_int),
         "bsm_device_status_clear": ([ctypes.c_int], ctypes.c_int),
         "bsm_max_row_bytes": ([ctypes.c_int], i64),
-        "bsm_ragged_extent": ([i64, c_i64p, c_i32p, c_i32p], i64),
+        "bsm_ragged_extent": ([i64, vp, vp, vp], i64),
         "bsm_status_string": ([ctypes.c_int], ctypes.c_char_p),
         "bsm_version": ([], ctypes.c_int),
         "bsm_device_debug": ([ctypes.c_int, ctypes.POINTER(ctypes.c_uint32)], ctypes.c_int),
@@ -208,6 +208,12 @@ def _dptr(t, nbytes: Optional[int] = None, what: str = "buffer") -> Optional[int
     A tensor must live on a CUDA device, be contiguous and (when nbytes is
     given) hold at least nbytes: the C ABI sees only the address, so these are
     checked here, before any launch."""
+    try:
+        # the usual case: a tensor that passes every check
+        if t.is_cuda and t.is_contiguous() and (nbytes is None or t.nbytes >= nbytes):
+            return t.data_ptr()
+    except AttributeError:
+        pass
     if t is None:
         return None
     if isinstance(t, int):
@@ -233,41 +239,51 @@ def _bmm_bytes(B: int, M: int, N: int, K: int, out_dtype: int):
     return B * M * K * 2, B * N * K * 2, B * M * N * _esize(out_dtype)
 
 
-def _extent(offsets, rows, cols) -> int:
-    """Elements a ragged batch spans (the end of its furthest non-empty slice),
-    computed by the library's host helper: microseconds even on tens of
-    thousands of slices.  offsets/rows/cols: contiguous int64/int32/int32."""
-    n = len(offsets)
-    e = int(lib().bsm_ragged_extent(n, offsets.ctypes.data_as(c_i64p), rows.ctypes.data_as(c_i32p),
-                                    cols.ctypes.data_as(c_i32p)))
+def _extent(n: int, offsets: int, rows: int, cols: int) -> int:
+    """Elements a ragged batch of n slices spans (the end of its furthest
+    non-empty slice), computed by the library's host helper: microseconds even
+    on tens of thousands of slices.  offsets/rows/cols: host addresses of
+    contiguous int64/int32/int32 arrays."""
+    e = lib().bsm_ragged_extent(n, offsets, rows, cols)
     if e < 0:
         raise ValueError("ragged batch: negative offset or column count")
     return e
 
 
+def _ragged(offsets, rows, cols):
+    """The three host arrays of a ragged batch as contiguous arrays (to be kept
+    alive over the call) and their addresses."""
+    off, r, c = _np(offsets, np.int64), _np(rows, np.int32), _np(cols, np.int32)
+    if not (len(off) == len(r) == len(c)):
+        raise ValueError("offsets, rows and cols must have the same length")
+    return (off, r, c), (len(off), off.ctypes.data, r.ctypes.data, c.ctypes.data)
+
+
 def _stream(s) -> Optional[int]:
-    if s is None:
-        return None
-    if isinstance(s, int):
+    if s is None or isinstance(s, int):
         return s
     return int(s.cuda_stream)
 
 
 def _np(a, dt):
+    if type(a) is np.ndarray and a.dtype == dt and a.flags.c_contiguous:
+        return a
     return np.ascontiguousarray(np.asarray(a), dtype=dt)
 
 
 def bsm_softmax(x, y, B: int, R: int, C: int, dtype: int, policy: int, stream=None):
-    n = max(B * R * C, 0) * _esize(dtype)
-    _check(lib().bsm_softmax(_dptr(x, n, "x"), _dptr(y, n, "y"), B, R, C, dtype, policy,
-                             _stream(stream)), "bsm_softmax")
+    n = B * R * C * (4 if dtype == F32 else 2)      # (negative sizes: refused by the library)
+    rc = lib().bsm_softmax(_dptr(x, n, "x"), _dptr(y, n, "y"), B, R, C, dtype, policy, _stream(stream))
+    if rc:
+        _check(rc, "bsm_softmax")
 
 
 def bsm_softmax_ex(x, y, B: int, R: int, C: int, dtype: int, policy: int, flags: int = 0,
                    stream=None):
-    n = max(B * R * C, 0) * _esize(dtype)
-    _check(lib().bsm_softmax_ex(_dptr(x, n, "x"), _dptr(y, n, "y"), B, R, C, dtype, policy, flags,
-                                _stream(stream)), "bsm_softmax_ex")
+    n = B * R * C * (4 if dtype == F32 else 2)      # (negative sizes: refused by the library)
+    rc = lib().bsm_softmax_ex(_dptr(x, n, "x"), _dptr(y, n, "y"), B, R, C, dtype, policy, flags, _stream(stream))
+    if rc:
+        _check(rc, "bsm_softmax_ex")
 
 
 def bsm_softmax_host(x_host, y_host, B: int, R: int, C: int, dtype: int, policy: int,
@@ -286,7 +302,7 @@ def bsm_softmax_host(x_host, y_host, B: int, R: int, C: int, dtype: int, policy:
 
 def bsm_softmax_noalloc(x, y, B: int, R: int, C: int, dtype: int, flags: int = 0, stream=None):
     """The allocation-free entry point (fixed scratch inside the library)."""
-    n = max(B * R * C, 0) * _esize(dtype)
+    n = B * R * C * (4 if dtype == F32 else 2)      # (negative sizes: refused by the library)
     _check(lib().bsm_softmax_noalloc(_dptr(x, n, "x"), _dptr(y, n, "y"), B, R, C, dtype, flags,
                                      _stream(stream)), "bsm_softmax_noalloc")
 
@@ -309,7 +325,7 @@ def bsm_bmm_ex(a, bt, c, B: int, M: int, N: int, K: int, out_dtype: int, policy:
 
 
 def bsm_softmax_backward(y, dy, dx, B: int, R: int, C: int, dtype: int, policy: int, stream=None):
-    n = max(B * R * C, 0) * _esize(dtype)
+    n = B * R * C * (4 if dtype == F32 else 2)      # (negative sizes: refused by the library)
     _check(lib().bsm_softmax_backward(_dptr(y, n, "y"), _dptr(dy, n, "dy"), _dptr(dx, n, "dx"),
                                       B, R, C, dtype, policy, _stream(stream)),
            "bsm_softmax_backward")
@@ -317,31 +333,20 @@ def bsm_softmax_backward(y, dy, dx, B: int, R: int, C: int, dtype: int, policy: 
 
 def bsm_softmax_backward_ragged(y, dy, dx, offsets, rows, cols, dtype: int, policy: int,
                                 stream=None):
-    off = _np(offsets, np.int64)
-    r = _np(rows, np.int32)
-    c = _np(cols, np.int32)
-    if not (len(off) == len(r) == len(c)):
-        raise ValueError("offsets, rows and cols must have the same length")
-    n = _extent(off, r, c) * _esize(dtype)
-    _check(lib().bsm_softmax_backward_ragged(_dptr(y, n, "y"), _dptr(dy, n, "dy"), _dptr(dx, n, "dx"),
-                                             len(off),
-                                             off.ctypes.data_as(c_i64p), r.ctypes.data_as(c_i32p),
-                                             c.ctypes.data_as(c_i32p), dtype, policy,
-                                             _stream(stream)), "bsm_softmax_backward_ragged")
+    keep, where = _ragged(offsets, rows, cols)
+    n = _extent(*where) * _esize(dtype)
+    _check(lib().bsm_softmax_backward_ragged(_dptr(y, n, "y"), _dptr(dy, n, "dy"), _dptr(dx, n, "dx"), *where,
+                                             dtype, policy, _stream(stream)), "bsm_softmax_backward_ragged")
+    del keep
 
 
 def bsm_softmax_ragged(x, y, offsets, rows, cols, dtype: int, policy: int, flags: int = 0,
                        stream=None):
-    off = _np(offsets, np.int64)
-    r = _np(rows, np.int32)
-    c = _np(cols, np.int32)
-    if not (len(off) == len(r) == len(c)):
-        raise ValueError("offsets, rows and cols must have the same length")
-    n = _extent(off, r, c) * _esize(dtype)
-    _check(lib().bsm_softmax_ragged(_dptr(x, n, "x"), _dptr(y, n, "y"), len(off),
-                                    off.ctypes.data_as(c_i64p), r.ctypes.data_as(c_i32p),
-                                    c.ctypes.data_as(c_i32p), dtype, policy, flags,
+    keep, where = _ragged(offsets, rows, cols)
+    n = _extent(*where) * _esize(dtype)
+    _check(lib().bsm_softmax_ragged(_dptr(x, n, "x"), _dptr(y, n, "y"), *where, dtype, policy, flags,
                                     _stream(stream)), "bsm_softmax_ragged")
+    del keep
 
 
 class Plan:
@@ -381,7 +386,7 @@ def bsm_plan_create(x, y, rows, cols, dtype: int, policy: int, offsets=None, fla
     if off is None:
         n = int(np.sum(r.astype(np.int64) * c.astype(np.int64))) * _esize(dtype)
     else:
-        n = _extent(off, r, c) * _esize(dtype)
+        n = _extent(len(off), off.ctypes.data, r.ctypes.data, c.ctypes.data) * _esize(dtype)
     d.x = _dptr(x, n, "x")
     d.y = _dptr(y, n, "y")
     d.num_slices = len(r)
