@@ -52,19 +52,21 @@
  *     (BSM_ERR_INVALID_ARG).
  *   - Row length: a row of up to bsm_max_row_bytes() (half of it for the
  *     backward pass, where y and dy share a stage) is read once from one
- *     shared-memory stage.  Longer rows go through the stages in chunks, in
- *     two passes -- a running maximum and rescaled sum (backward: the dot
- *     product), then the output.  A row of two chunks whose halves fit three
- *     stages (with the batch's shorter rows) stays staged between the passes
- *     and is read once; longer rows are read again, all but their last
- *     chunk.  When a batch has fewer such rows than two per SM, each is cut
- *     into segments spread over the SMs and the execute takes two launches
- *     (segment partials, then combine and write); otherwise each row stays
- *     on one SM within one launch.  Forward rows of 5 to 32 parts of at most
- *     64 KiB, enough of them to fill two thirds of the groups'
+ *     shared-memory stage, by one warp or, past 2 KiB, by a team of up to 16.
+ *     Batches of longer rows, at least two per SM, run over clusters of 2 or 4
+ *     SMs: each takes a part of the row in one of its stages and every element
+ *     is read once (rows of up to 452 KiB, 226 KiB backward).  Other longer
+ *     rows go through the stages in chunks, in two passes -- a running maximum
+ *     and rescaled sum (backward: the dot product), then the output -- and are
+ *     read again, all but their last chunk (a row of two chunks whose halves
+ *     fit three stages stays staged).  When a batch has fewer such rows than
+ *     two per SM, each is cut into segments spread over the SMs and the execute
+ *     takes two launches (segment partials, then combine and write); otherwise
+ *     each row stays on one SM within one launch.  Forward rows of 5 to 32
+ *     parts of at most 64 KiB, enough of them to fill two thirds of the groups'
  *     waves, are instead split over groups of K CTAs (K = ceil(row / 64
  *     KiB); n_sm / K groups) in one cooperative launch: each CTA stages one
- *     part, the group exchanges (max, sum) partials through global memory
+ *     part, the group exchanges (offset, sum) partials through global memory
  *     and every element is read once.  Which path a row takes depends on the
  *     rows of the batch and the device, never on the policy: every policy
  *     gives the same bits.

@@ -355,6 +355,51 @@ int choose_groups(const std::vector<SliceView> &slices, int es, int n_sm, int64_
     return 1;
 }
 
+// Rows over clusters of CTAs: batches whose every patch is a whole row longer
+// than a stage (so at least two per SM, too short for the groups).  The
+// smallest cluster whose parts fit two stages; K = 0: none does, or too few
+// clusters are resident at once.  Which batches: by row lengths, their number
+// and the device only, never by the policy.
+struct ClusterChoice {
+    int K = 0, units = 0, n_stages = 0;
+    int64_t stage = 0;
+};
+
+ClusterChoice choose_clusters(const PatchLayout &L, int dtype, bool bwd, int n_sm, int64_t smem_optin)
+{
+    ClusterChoice c;
+    if (L.items.empty() || L.segs.size() != L.items.size() || !L.items1.empty() || !L.items_g.empty())
+        return c;
+    int64_t lmax = 0;
+    for (size_t i = 0; i < L.items.size(); ++i) {
+        if (L.segs[i].part_count != 1)
+            return c;
+        lmax = std::max<int64_t>(lmax, L.items[i].C);
+    }
+    const int64_t avail = smem_optin - kClusterHeader, arrays = bwd ? 2 : 1;
+    const int64_t nv = (lmax * esize(dtype) + 15) / 16;
+    for (int K : {2, 4}) {
+        const int64_t stage = arrays * ((((nv + K - 1) / K) * 16 + 127) & ~int64_t(127));
+        const int n_stages = static_cast<int>(std::min<int64_t>(kMaxStages, avail / stage));
+        if (n_stages < 2)
+            continue;
+        int units = 0;
+        if (cluster_units(dtype, bwd, K, n_sm, static_cast<int>(kClusterHeader + n_stages * stage), &units)) {
+            cudaGetLastError();
+            return c;
+        }
+        units = std::min(units, n_sm / K);
+        if (units * K * 8 < n_sm * 7)          // more than an eighth of the SMs would idle
+            return c;
+        c.K = K;
+        c.units = units;
+        c.n_stages = n_stages;
+        c.stage = stage;
+        return c;
+    }
+    return c;
+}
+
 int cut_patches(const bsm_plan_desc *d, const std::vector<SliceView> &slices, int64_t max_row, int n_sm,
                 int64_t smem_optin, PatchLayout &L)
 {
@@ -659,6 +704,15 @@ int plan_create_impl(bsm_plan **out, const bsm_plan_desc *d)
     std::vector<Item> all(items);
     all.insert(all.end(), items_g.begin(), items_g.end());
 
+    ClusterChoice cl;
+    {
+        int prev = -1;
+        cudaGetDevice(&prev);
+        cudaSetDevice(device);
+        cl = choose_clusters(lay, d->dtype, d->op == BSM_OP_BACKWARD, c->n_sm, c->smem_optin);
+        if (prev >= 0)
+            cudaSetDevice(prev);
+    }
     bsm_plan *p = new bsm_plan();
     p->device = device;
     p->policy = d->policy;
@@ -684,6 +738,8 @@ int plan_create_impl(bsm_plan **out, const bsm_plan_desc *d)
         team = team || int64_t(it.C) * es > (d->op == BSM_OP_BACKWARD ? (es == 4 ? kLaneRowBytesBwd<4> : kLaneRowBytesBwd<2>) : kLaneRowBytes);
     p->kernel_op = d->op == BSM_OP_BACKWARD ? (reg_long ? OP_BACKWARD_LONG : team ? OP_BACKWARD_TEAM : OP_BACKWARD)
                                             : (reg_long ? OP_FORWARD_LONG : team ? OP_FORWARD_TEAM : OP_FORWARD);
+    if (cl.K)
+        p->kernel_op = d->op == BSM_OP_BACKWARD ? OP_BACKWARD_CLUSTER : OP_FORWARD_CLUSTER;
 
     // ---- the schedule
     std::vector<int32_t> queue;      // schedule order of the patches (queue policies)
@@ -1000,6 +1056,17 @@ int plan_create_impl(bsm_plan **out, const bsm_plan_desc *d)
         p->grid_g = lay.group_k * lay.n_groups;
     }
 
+    if (cl.K) {
+        // (stats report the layout's stages, which the patches were cut for)
+        a.stage_bytes = static_cast<int32_t>(cl.stage);
+        a.n_stages = cl.n_stages;
+        a.group_k = cl.K;
+        a.n_groups = cl.units;
+        if (a.n_queues > 1)
+            a.steal = 1;                       // as for the groups: every queue must be drained
+    }
+    const int cta = cl.K ? cl.K : 1;           // CTAs per pulling unit, and units
+    const int units = cl.K ? cl.units : c->n_sm;
     const int32_t other_launches = (n_reg > 0 ? (n1 ? 2 : 1) : 0) + (n_grp > 0 ? 1 : 0);
     switch (d->policy) {
     case BSM_POLICY_WHOLE_GPU:
@@ -1007,7 +1074,7 @@ int plan_create_impl(bsm_plan **out, const bsm_plan_desc *d)
         for (size_t k = 0; k < slices.size(); ++k) {
             const int32_t n = slice_first[k + 1] - slice_first[k];
             if (n > 0)
-                p->whole_gpu.push_back({slice_first[k], slice_first[k + 1], std::min(n, c->n_sm), 0});
+                p->whole_gpu.push_back({slice_first[k], slice_first[k + 1], cta * std::min(n, units), 0});
             const int32_t n1s = slice_first1[k + 1] - slice_first1[k];
             if (n1s > 0)
                 p->whole_gpu.push_back({slice_first1[k], slice_first1[k + 1], std::min(n1s, c->n_sm), 1});
@@ -1022,12 +1089,12 @@ int plan_create_impl(bsm_plan **out, const bsm_plan_desc *d)
         break;
     case BSM_POLICY_RR:
         a.mode = PULL_RR_SLICE;
-        p->grid = static_cast<int>(std::min<int64_t>(c->n_sm, std::max<int64_t>(1, int64_t(slices.size()))));
+        p->grid = cta * static_cast<int>(std::min<int64_t>(units, std::max<int64_t>(1, int64_t(slices.size()))));
         st.launches = other_launches;
         break;
     default:
         a.mode = PULL_QUEUE;
-        p->grid = c->n_sm;
+        p->grid = cta * units;
         st.launches = other_launches;
         break;
     }

@@ -39,6 +39,8 @@ constexpr int kConsumerWarps = 16;
 constexpr int kThreads = (kConsumerWarps + 1) * 32;  // + one producer warp
 constexpr int kGroupThreads = kThreads + 32;          // rows over groups: + one exchange warp
 constexpr int kSmemHeader = 1024;                     // barriers + stage metadata
+constexpr int kClusterHeader = 1536;                  // the same of rows over clusters of CTAs
+constexpr int kMaxCluster = 4;
 // Smallest stage (three fit the shared memory).  Each stage has a fixed cost
 // (wait, metadata, dispatch, release) that larger stages amortise; measured
 // over 32 KiB stages: bf16 +11 % causal 512-wide rows, +16 % 32 x 128 slices;
@@ -54,7 +56,9 @@ enum Op : int32_t {
     OP_BACKWARD_LONG = 3, // OP_BACKWARD for plans with rows longer than half a stage (two passes)
     OP_FORWARD_GROUP = 4, // OP_FORWARD of rows split over groups of CTAs (one read; see KernelArgs)
     OP_FORWARD_TEAM = 5, // OP_FORWARD for plans with rows that teams of warps share (past kLaneRowBytes)
-    OP_BACKWARD_TEAM = 6 // OP_BACKWARD for such plans (past kLaneRowBytesBwd)
+    OP_BACKWARD_TEAM = 6, // OP_BACKWARD for such plans (past kLaneRowBytesBwd)
+    OP_FORWARD_CLUSTER = 7, // rows longer than a stage over clusters of group_k CTAs (one read)
+    OP_BACKWARD_CLUSTER = 8
 };
 
 // Rows of more bytes than this (up to a stage) are shared by a team of 1 to 16
@@ -131,7 +135,7 @@ struct KernelArgs {
     float *partials;            // 2 floats per segment
     int32_t phase;              // 0: segments leave their partials; 1: combine and write
     // rows split over groups of CTAs (OP_FORWARD_GROUP): items are whole rows
-    int32_t group_k;            // CTAs per group (2..kMaxGroup); the grid is n_groups * group_k
+    int32_t group_k;            // CTAs per group (2..kMaxGroup; per cluster, OP_*_CLUSTER); the grid is n_groups * group_k
     int32_t n_groups;
     unsigned long long *ring;   // n_groups x kGroupRing claim words
     unsigned long long *xch;    // n_groups x kGroupSlots x group_k x 2 tagged words: max, sum
@@ -185,6 +189,9 @@ int gemm_fixed_smem(int bn, bool out_bf16, int epi_bufs);
 // Launch the persistent softmax kernel (bsm_kernels.cu).  Returns a
 // cudaError_t value (0 = success).
 int launch_softmax(const KernelArgs &a, int dtype, int op, int grid, void *stream, bool checked);
+// How many clusters of K CTAs of the cluster kernel run at once (smem bytes of
+// dynamic shared memory each CTA).  Returns a cudaError_t value.
+int cluster_units(int dtype, bool bwd, int K, int n_sm, int smem, int *units);
 // Raise the dynamic shared-memory limit of both kernel instances.
 int kernel_set_smem_limit(int bytes);
 

@@ -982,11 +982,13 @@ __device__ __forceinline__ bool row_team_bwd(const unsigned char *sy, const unsi
         }
         return r;
     };
+    // (a vector's products first, as a tree: the running sum is rounded once a vector)
     auto add = [&](Pair acc, uint4 a, uint4 b) -> Pair {
-#pragma unroll
-        for (int k = 0; k < N; ++k)
-            acc = pair_fma(vec_pair<Tag>(a, k), vec_pair<Tag>(b, k), acc);
-        return acc;
+        Pair t = pair_fma(vec_pair<Tag>(a, 1), vec_pair<Tag>(b, 1), pair_mul(vec_pair<Tag>(a, 0), vec_pair<Tag>(b, 0)));
+        if constexpr (N == 4)
+            t = pair_add(t, pair_fma(vec_pair<Tag>(a, 3), vec_pair<Tag>(b, 3),
+                                     pair_mul(vec_pair<Tag>(a, 2), vec_pair<Tag>(b, 2))));
+        return pair_add(acc, t);
     };
     uint4 yv[V], dv[V];
 #pragma unroll
@@ -2546,6 +2548,399 @@ __global__ void __launch_bounds__(kGroupThreads, 1) softmax_group(const KernelAr
     }
 }
 
+// ------------------------------------------------ rows over clusters of CTAs
+// Batches of rows too long for one stage, enough of them to fill the SMs: a
+// cluster of K = 2 or 4 CTAs shares a row, a part of it in one stage of each
+// (the parts of a row of 64 to 113 KiB are what a team of 16 warps takes
+// alone), so every element is read once.  The row routines are the teams',
+// W = 16; the exchange goes over the cluster: every warp sends its (offset, sum)
+// (backward: its dot product) to all K CTAs' shared memory with an
+// asynchronous store that counts on the receiver's barrier, and every warp of
+// the cluster combines the 16 K of them in the same fixed tree.  The first
+// CTA claims the rows (any policy's puller, with the cluster as the unit) and
+// posts them to the others' rings of claim words.
+//
+// What bounded these rows: one CTA streamed a row twice, its second read from
+// L2 while the first of the next row waited for a stage.  GB/s over 256 MiB,
+// one CTA a row -> clusters: forward fp32 128 KiB rows 5463 -> 6495, 256 KiB
+// (K = 4, 36 clusters: 144 SMs) 5056 -> 6532; bf16 128 KiB 4592 -> 6356, 224 KiB
+// 4620 -> 6313, 256 KiB 4407 -> 6373; backward (512 MiB of y and dy) fp32 64 KiB
+// 6182 -> 6950, 128 KiB (K = 4) 5887 -> 6981, bf16 5916 -> 6845.
+struct ClusterMeta {
+    int64_t off;
+    int32_t C, row0, col0, kind;
+};
+
+constexpr int kClusterRing = 16;
+
+struct ClusterSmem {
+    uint64_t full[kMaxStages];
+    uint64_t empty[kMaxStages];
+    uint64_t xbar[2];                   // a row's partials are in, by row parity
+    unsigned long long ring[kClusterRing];
+    ClusterMeta meta[kMaxStages];
+    float2 part[2][kMaxCluster * kConsumerWarps];
+    int32_t abort_flag;
+};
+static_assert(sizeof(ClusterSmem) <= kClusterHeader, "cluster header too large");
+
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
+    return r;
+}
+
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Wait (without sleeping, bounded) for a phase that other CTAs of the cluster
+// complete.
+__device__ __forceinline__ bool cluster_spin_bounded(uint64_t *bar, uint32_t parity, const volatile int32_t *abort,
+                                                     uint64_t limit_ns)
+{
+    uint64_t t0 = 0;
+    for (uint32_t it = 0; it < (1u << 30); ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_addr(bar)), "r"(parity)
+            : "memory");
+        if (ok)
+            return true;
+        if ((it & 1023u) == 1023u) {
+            const uint64_t t = global_timer_ns();
+            t0 = t0 ? t0 : t;
+            if (*abort || t - t0 > limit_ns)
+                return false;
+        }
+    }
+    return false;
+}
+
+template <typename Tag, bool Bwd, bool Checked>
+__global__ void __launch_bounds__(kThreads, 1) softmax_cluster(const KernelArgs a)
+{
+    using E = Elem<Tag>;
+    constexpr int EPV = E::kPerVec, kArrays = Bwd ? 2 : 1;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    ClusterSmem &h = *reinterpret_cast<ClusterSmem *>(smem);
+    unsigned char *stages = smem + kClusterHeader;
+    const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int S = a.n_stages, K = a.group_k, half = a.stage_bytes / 2;
+    const int unit = static_cast<int>(blockIdx.x) / K, n_units = static_cast<int>(gridDim.x) / K;
+    const int rank = static_cast<int>(blockIdx.x) % K;          // = the CTA's rank in its cluster
+    const uint64_t wait_limit = a.wait_limit_ns ? a.wait_limit_ns : kWaitLimitNs;
+    // this CTA's part of a row of C elements: whole vectors
+    auto part_of = [&](int32_t C, int64_t &c0, int64_t &cn, int64_t &bytes) {
+        const int64_t nv = (int64_t(C) * E::kSize) >> 4, pv = (nv + K - 1) / K;
+        const int64_t v0 = pv * rank, vn = nv - v0 < 0 ? 0 : (nv - v0 < pv ? nv - v0 : pv);
+        c0 = v0 * EPV;
+        cn = vn * EPV;
+        bytes = pv * 16;                                        // the longest part
+    };
+    auto item_ok = [&](const Item &it, int64_t part_bytes) {
+        return it.off >= 0 && it.C > 0 && it.nrows == 1 && it.R > 0 && it.row0 >= 0 && it.row0 < it.R &&
+               it.off + it.C <= a.total_elems && ((it.off * E::kSize) & 15) == 0 &&
+               ((int64_t(it.C) * E::kSize) & 15) == 0 && part_bytes <= (Bwd ? half : a.stage_bytes);
+    };
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&h.full[s], 1);
+            mbar_init(&h.empty[s], kConsumerWarps);
+        }
+        mbar_init(&h.xbar[0], 1);
+        mbar_init(&h.xbar[1], 1);
+        for (int i = 0; i < kClusterRing; ++i)
+            h.ring[i] = 0ull;
+        h.abort_flag = 0;
+        mbar_init_fence();
+    }
+    __syncthreads();
+    cluster_barrier();
+    // the cluster's likely first row into L2 (a hint, as prefetch_first_batch)
+    if (warp == kConsumerWarps && lane == 0 && a.mode == PULL_QUEUE) {
+        const int q = unit % (a.n_queues > 0 ? a.n_queues : 1), k = unit / (a.n_queues > 0 ? a.n_queues : 1);
+        const int64_t idx = int64_t(a.queue_begin[q]) + k;
+        if (k < a.queue_len[q] && idx >= 0 && idx < a.n_items) {
+            const Item it = a.items[idx];
+            int64_t c0, cn, pb;
+            part_of(it.C, c0, cn, pb);
+            if (item_ok(it, pb) && cn > 0) {
+                prefetch_l2(static_cast<const unsigned char *>(a.x) + (it.off + c0) * E::kSize,
+                            static_cast<uint32_t>(cn * E::kSize));
+                if (Bwd)
+                    prefetch_l2(static_cast<const unsigned char *>(a.x2) + (it.off + c0) * E::kSize,
+                                static_cast<uint32_t>(cn * E::kSize));
+            }
+        }
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    if (warp == kConsumerWarps) {
+        // ------------------------------------------------------- producer
+        if (lane == 0) {
+            Puller pull(a, unit, n_units);
+            bool aborted = false, post_done = false;
+            uint32_t posted = 0, claim = 0xFFFFFFFFu;
+            auto claim_next = [&]() {
+                int32_t p1[kFetch];
+                claim = pull.next_batch(p1, 1) > 0 ? static_cast<uint32_t>(p1[0]) : 0xFFFFFFFFu;
+            };
+            // rows are announced two ahead, the claim after them under way; a
+            // word carries all that its reader uses.  No word is overwritten
+            // unread: a producer is at most S stages and one row ahead of the
+            // slowest.
+            auto post = [&](uint32_t upto) {
+                while (rank == 0 && !post_done && posted <= upto) {
+                    const unsigned long long w = (static_cast<unsigned long long>(posted + 1) << 32) | claim;
+                    for (int r = 0; r < K; ++r)
+                        asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(
+                                         cluster_addr(&h.ring[posted % kClusterRing], r)),
+                                     "l"(w)
+                                     : "memory");
+                    ++posted;
+                    post_done = claim == 0xFFFFFFFFu;
+                    if (!post_done)
+                        claim_next();
+                }
+            };
+            auto ring_word = [&](uint32_t t, uint32_t &pos) -> bool {
+                const uint32_t addr = smem_addr(&h.ring[t % kClusterRing]);
+                uint64_t t0 = 0;
+                for (uint32_t it = 0; it < (1u << 28); ++it) {
+                    unsigned long long w;
+                    asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(w) : "r"(addr) : "memory");
+                    if (static_cast<uint32_t>(w >> 32) == t + 1) {
+                        pos = static_cast<uint32_t>(w);
+                        return true;
+                    }
+                    if ((it & 15u) == 15u) {
+                        const uint64_t now = global_timer_ns();
+                        t0 = t0 ? t0 : now;
+                        if (h.abort_flag || now - t0 > wait_limit)
+                            return false;
+                        __nanosleep(64);
+                    }
+                }
+                return false;
+            };
+            if (rank == 0)
+                claim_next();
+            post(1);
+            int s = 0;
+            uint32_t ph = 0;
+            uint32_t n_issued = 0;              // copies: stages issued so far
+            bool first = true;
+            for (uint32_t t = 0; !aborted; ++t) {
+                uint32_t pos = 0;
+                if (!ring_word(t, pos)) {
+                    aborted = true;
+                    break;
+                }
+                const bool in = pos < static_cast<uint32_t>(a.n_items);
+                Item item{-1, 0, 0, 0, 0};
+                if (in)
+                    item = a.items[pos];        // on its way while the stage is waited for
+                post(t + 2);
+                if (!mbar_wait_bounded(&h.empty[s], ph ^ 1u, &h.abort_flag, wait_limit)) {
+                    aborted = true;
+                    break;
+                }
+                ClusterMeta &mt = h.meta[s];
+                uint64_t *full = &h.full[s];
+                unsigned char *dst = stages + static_cast<size_t>(s) * a.stage_bytes;
+                if (++s == S) {
+                    s = 0;
+                    ph ^= 1u;
+                }
+                if (pos == 0xFFFFFFFFu) {
+                    mt.kind = KIND_DONE;
+                    mbar_arrive(full);
+                    break;
+                }
+                if ((a.debug & KDEBUG_WITHHOLD_STAGE0) && first) {
+                    first = false;
+                    continue;                      // test hook: the first stage is never filled
+                }
+                first = false;
+                int64_t c0, cn, pb;
+                part_of(item.C, c0, cn, pb);
+                if (!in || !item_ok(item, pb)) {
+                    // every CTA of the cluster sees the same record and skips the row alike
+                    atomicOr(a.status, BSM_DEV_BOUNDS);
+                    mt.kind = KIND_SKIP;
+                    mbar_arrive(full);
+                    continue;
+                }
+                mt.off = item.off + c0;
+                mt.C = static_cast<int32_t>(cn);
+                mt.row0 = item.row0;
+                mt.col0 = static_cast<int32_t>(c0);
+                mt.kind = KIND_DATA;
+                if (cn == 0) {
+                    mbar_arrive(full);
+                    continue;
+                }
+                const uint32_t bytes = static_cast<uint32_t>(cn * E::kSize);
+                const unsigned char *src = static_cast<const unsigned char *>(a.x) + (item.off + c0) * E::kSize;
+                const unsigned char *src2 = Bwd ? static_cast<const unsigned char *>(a.x2) + (item.off + c0) * E::kSize
+                                                : nullptr;
+                if (Checked) {
+                    const unsigned char *x0 = static_cast<const unsigned char *>(a.x);
+                    const unsigned char *g0 = static_cast<const unsigned char *>(a.x2);
+                    const int64_t all = a.total_elems * E::kSize;
+                    if (src < x0 || src + bytes > x0 + all || (reinterpret_cast<uintptr_t>(src) & 15) ||
+                        (Bwd && (src2 < g0 || src2 + bytes > g0 + all || (reinterpret_cast<uintptr_t>(src2) & 15))) ||
+                        (smem_addr(dst) & 15) || (half & 15) || bytes > static_cast<uint32_t>(Bwd ? half : a.stage_bytes) ||
+                        dst + a.stage_bytes > smem + kClusterHeader + static_cast<size_t>(S) * a.stage_bytes) {
+                        check_fail(a.status, 3, pos, bytes);
+                        mt.kind = KIND_SKIP;       // the cluster's other CTAs time out
+                        mbar_arrive(full);
+                        continue;
+                    }
+                }
+                mbar_arrive_expect_tx(full, kArrays * bytes);
+                bulk_load(dst, src, bytes, full);
+                if (Bwd)
+                    bulk_load(dst + half, src2, bytes, full);
+                ++n_issued;
+            }
+            if (aborted) {
+                atomicOr(a.status, BSM_DEV_TIMEOUT);
+                h.abort_flag = 1;
+                // the copies in flight land before the CTA may leave (normally
+                // the consumers waited for them): at most the S newest stages
+                for (uint32_t j = 0; j < static_cast<uint32_t>(S) && j < n_issued; ++j) {
+                    s = s == 0 ? S - 1 : s - 1;
+                    if (s == S - 1)
+                        ph ^= 1u;
+                    mbar_wait_bounded(&h.full[s], ph, nullptr, wait_limit);
+                }
+            }
+            if (rank == 0 && a.mode == PULL_QUEUE) {
+                // the last cluster to finish pulling rewinds the queue heads
+                __threadfence();
+                const uint32_t prev = atomicAdd(&a.heads[BSM_MAX_DIES], 1u);
+                if (prev == static_cast<uint32_t>(n_units - 1)) {
+                    for (int d = 0; d < BSM_MAX_DIES; ++d)
+                        atomicExch(&a.heads[d], 0u);
+                    atomicExch(&a.heads[BSM_MAX_DIES], 0u);
+                }
+            }
+        }
+        __syncwarp();
+    } else {
+        // ----------------------------------------------------------- consumers
+        const bool causal = (a.flags & BSM_FLAG_CAUSAL) != 0;
+        unsigned char *y = static_cast<unsigned char *>(a.y);
+        uint32_t x = 0;             // rows exchanged
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        // this warp's pair to every CTA of the cluster, then all warps' pairs:
+        // one of them per lane (of 64, two).  Barrier and slots alternate by
+        // row: a warp sends row t + 2's after it has row t + 1's pairs, which
+        // every warp sent after it had taken row t's.
+        auto gather = [&](float2 mine, float2 none, float2 &p0, float2 &p1) -> bool {
+            const uint32_t par = x & 1u;
+            if (warp == 0 && lane == 0)
+                mbar_arrive_expect_tx(&h.xbar[par], static_cast<uint32_t>(K * kConsumerWarps * sizeof(float2)));
+            __syncwarp();
+            if (lane < K) {
+                unsigned long long w;
+                asm("mov.b64 %0, {%1, %2};" : "=l"(w) : "f"(mine.x), "f"(mine.y));
+                asm volatile(
+                    "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(
+                        cluster_addr(&h.part[par][rank * kConsumerWarps + warp], lane)),
+                    "l"(w), "r"(cluster_addr(&h.xbar[par], lane))
+                    : "memory");
+            }
+            if (!__all_sync(0xFFFFFFFFu, cluster_spin_bounded(&h.xbar[par], (x >> 1) & 1u, &h.abort_flag, wait_limit)))
+                return false;
+            ++x;
+            p0 = lane < K * kConsumerWarps ? h.part[par][lane] : none;
+            p1 = lane + 32 < K * kConsumerWarps ? h.part[par][lane + 32] : none;
+            return true;
+        };
+        for (;;) {
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(&h.full[s], ph, &h.abort_flag, wait_limit));
+            if (!ok)
+                break;
+            const int32_t kind = h.meta[s].kind;
+            if (kind == KIND_DONE)
+                break;
+            const int s0 = s;
+            auto release = [&]() {
+                __syncwarp();
+                if (lane == 0)
+                    mbar_arrive(&h.empty[s0]);
+            };
+            if (++s == S) {
+                s = 0;
+                ph ^= 1u;
+            }
+            if (kind != KIND_DATA) {
+                release();
+                continue;
+            }
+            const unsigned char *sbuf = stages + static_cast<size_t>(s0) * a.stage_bytes;
+            const int bytes = h.meta[s0].C * E::kSize, nvec = bytes >> 4;
+            unsigned char *yp = y + h.meta[s0].off * E::kSize;
+            const Bounds bd{sbuf, sbuf + bytes, y, y + a.total_elems * E::kSize, a.status};
+            if constexpr (Bwd) {
+                auto exchange = [&](float &dot) -> bool {
+                    float2 p0, p1;
+                    if (!gather(make_float2(dot, 0.0f), make_float2(0.0f, 0.0f), p0, p1))
+                        return false;
+                    dot = group_sum<32>(p0.x + p1.x);
+                    return true;
+                };
+                const Bounds bdy{sbuf + half, sbuf + half + bytes, y, y + a.total_elems * E::kSize, a.status};
+                if (nvec >= 2 * kConsumerWarps * 32)
+                    ok = row_team_bwd<Tag, Checked, 16, kTeamVecsBwd - 2>(sbuf, sbuf + half, yp, nvec, warp, lane, bd, bdy,
+                                                                          exchange, release);
+                else
+                    ok = row_team_bwd<Tag, Checked, 16, 0>(sbuf, sbuf + half, yp, nvec, warp, lane, bd, bdy, exchange,
+                                                           release);
+            } else {
+                const int row = h.meta[s0].row0, col0 = h.meta[s0].col0;
+                auto exchange = [&](float2 &os) -> bool {
+                    float2 p0, p1;
+                    if (!gather(os, make_float2(-INFINITY, 0.0f), p0, p1))
+                        return false;
+                    os.x = warp_max(fmaxf(p0.x, p1.x));
+                    os.y = group_sum<32>(p0.y * ex2(p0.x - os.x) + p1.y * ex2(p1.x - os.x));
+                    return true;
+                };
+                if (nvec >= (kTeamVecs - 2) * kConsumerWarps * 32)
+                    ok = row_team<Tag, Checked, 16, kTeamVecs, kTeamVecs - 2>(sbuf, yp, nvec, row, causal, col0, warp,
+                                                                             lane, bd, exchange, release);
+                else
+                    ok = row_team<Tag, Checked, 16, kTeamVecs, 0>(sbuf, yp, nvec, row, causal, col0, warp, lane, bd,
+                                                                 exchange, release);
+            }
+            if (!ok)
+                break;
+        }
+        if (!ok && lane == 0) {
+            atomicOr(a.status, BSM_DEV_TIMEOUT);
+            h.abort_flag = 1;
+        }
+        __syncwarp();
+    }
+    // no CTA leaves while another of its cluster may still write to it
+    cluster_barrier();
+}
+
 }  // namespace
 
 int kernel_set_smem_limit(int bytes)
@@ -2575,6 +2970,14 @@ int kernel_set_smem_limit(int bytes)
         reinterpret_cast<const void *>(softmax_persistent<BF16, OP_BACKWARD_LONG, false>),
         reinterpret_cast<const void *>(softmax_persistent<F32, OP_BACKWARD_LONG, true>),
         reinterpret_cast<const void *>(softmax_persistent<BF16, OP_BACKWARD_LONG, true>),
+        reinterpret_cast<const void *>(softmax_cluster<F32, false, false>),
+        reinterpret_cast<const void *>(softmax_cluster<F32, false, true>),
+        reinterpret_cast<const void *>(softmax_cluster<F32, true, false>),
+        reinterpret_cast<const void *>(softmax_cluster<F32, true, true>),
+        reinterpret_cast<const void *>(softmax_cluster<BF16, false, false>),
+        reinterpret_cast<const void *>(softmax_cluster<BF16, false, true>),
+        reinterpret_cast<const void *>(softmax_cluster<BF16, true, false>),
+        reinterpret_cast<const void *>(softmax_cluster<BF16, true, true>),
         reinterpret_cast<const void *>(softmax_group<F32, false>),
         reinterpret_cast<const void *>(softmax_group<BF16, false>),
         reinterpret_cast<const void *>(softmax_group<F32, true>),
@@ -2633,12 +3036,64 @@ void launch_group(const KernelArgs &a, int grid, size_t smem, cudaStream_t st, b
     else
         cudaLaunchKernelEx(&cfg, softmax_group<Tag, false>, a);
 }
+// Rows over clusters of CTAs: clusters of a.group_k, with the programmatic
+// overlap of launch_one.
+template <typename Tag, bool Bwd>
+cudaError_t cluster_launch(const KernelArgs *a, int K, int grid, size_t smem, cudaStream_t st, bool checked, int *units)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(K);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = units ? 1 : 2;
+#ifdef BSM_NO_PDL
+    cfg.numAttrs = 1;
+#endif
+    if (units)
+        return cudaOccupancyMaxActiveClusters(units, softmax_cluster<Tag, Bwd, false>, &cfg);
+    if (checked)
+        return cudaLaunchKernelEx(&cfg, softmax_cluster<Tag, Bwd, true>, *a);
+    return cudaLaunchKernelEx(&cfg, softmax_cluster<Tag, Bwd, false>, *a);
+}
+
+cudaError_t cluster_dispatch(const KernelArgs *a, int dtype, bool bwd, int K, int grid, size_t smem, cudaStream_t st,
+                             bool checked, int *units)
+{
+    if (dtype == BSM_F32)
+        return bwd ? cluster_launch<F32, true>(a, K, grid, smem, st, checked, units)
+                   : cluster_launch<F32, false>(a, K, grid, smem, st, checked, units);
+    return bwd ? cluster_launch<BF16, true>(a, K, grid, smem, st, checked, units)
+               : cluster_launch<BF16, false>(a, K, grid, smem, st, checked, units);
+}
 }  // namespace
+
+int cluster_units(int dtype, bool bwd, int K, int n_sm, int smem, int *units)
+{
+    *units = 0;
+    return static_cast<int>(cluster_dispatch(nullptr, dtype, bwd, K, K * (n_sm / K), static_cast<size_t>(smem), nullptr,
+                                             false, units));
+}
 
 int launch_softmax(const KernelArgs &a, int dtype, int op, int grid, void *stream, bool checked)
 {
     const size_t smem = kSmemHeader + (size_t)a.n_stages * a.stage_bytes;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (op == OP_FORWARD_CLUSTER || op == OP_BACKWARD_CLUSTER) {
+        const size_t csmem = kClusterHeader + (size_t)a.n_stages * a.stage_bytes;
+        const cudaError_t e = cluster_dispatch(&a, dtype, op == OP_BACKWARD_CLUSTER, a.group_k, grid, csmem, st, checked,
+                                               nullptr);
+        const cudaError_t l = cudaGetLastError();
+        return static_cast<int>(e ? e : l);
+    }
     if (op == OP_FORWARD_GROUP) {
         if (dtype == BSM_F32)
             launch_group<F32>(a, grid, smem, st, checked);

@@ -1,0 +1,146 @@
+"""Batches of rows longer than a stage that clusters of 2 or 4 CTAs share,
+against the oracle (sampled rows) and bit-identical across policies: the
+lengths at which the cluster grows and parts of unequal length, the causal
+mask across parts, NaN, +inf, all -inf and masks of the type's lowest value,
+the self-checking kernel, a withheld stage and a corrupted record."""
+import numpy as np
+import pytest
+
+from gpu_util import bits, check_rows_against_oracle, run, sample_rows, to_device, to_host
+from paper_2002_07062_gb300 import bsm, workload
+
+pytestmark = pytest.mark.gpu
+
+POLICIES = [bsm.POLICY_DYNAMIC, bsm.POLICY_RR, bsm.POLICY_CBMF, bsm.POLICY_CBMF_LB, bsm.POLICY_WHOLE_GPU]
+# 16-byte vectors per row: just past a stage, odd parts, either side of the
+# largest row of two CTAs, up to the rows that groups take
+FWD = [7233, 8195, 14431, 14433, 16383]
+BWD = [3617, 4099, 7213, 7219, 14401]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def setup():
+    import torch
+    import __graft_entry__ as g
+    g.build()
+    torch.cuda.set_device(0)
+    bsm.bsm_device_status_clear()
+    yield
+    bsm.bsm_cache_clear()
+
+
+def _rows():
+    import torch
+    return 2 * torch.cuda.get_device_properties(0).multi_processor_count + 5
+
+
+@pytest.mark.parametrize("nvec", FWD)
+@pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
+@pytest.mark.parametrize("flags", [0, workload.CAUSAL])
+def test_forward_row_lengths(nvec, dtype, flags):
+    import torch
+    C = nvec * (4 if dtype == workload.F32 else 8)
+    w = workload.uniform("cluster", dtype, 5, (_rows() + 4) // 5, C, 3.0, 0xC10 + nvec + flags, flags).materialize()
+    x = to_device(w.x)
+    ys = [run(w, x, p) for p in POLICIES]
+    bsm.bsm_set_device_checks(True)
+    ys.append(run(w, x, bsm.POLICY_DYNAMIC))
+    torch.cuda.synchronize()
+    bsm.bsm_set_device_checks(False)
+    assert bsm.bsm_device_status() == 0, bsm.bsm_device_debug()
+    for y in ys[1:]:
+        assert torch.equal(bits(y), bits(ys[0]))
+    check_rows_against_oracle(w, to_host(ys[0]), sample_rows(w, 24, nvec))
+    s = ys[0].view(-1, C).double().sum(1)
+    assert float((s - 1).abs().max()) < (1e-5 if dtype == workload.F32 else 0.02)     # every row written
+
+
+@pytest.mark.parametrize("nvec", BWD)
+@pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
+def test_backward_row_lengths(nvec, dtype):
+    import torch
+    from test_backward_gpu import _check
+    C = nvec * (4 if dtype == workload.F32 else 8)
+    R = _rows()
+    t = torch.float32 if dtype == workload.F32 else torch.bfloat16
+    g = torch.Generator(device="cuda").manual_seed(nvec)
+    y = torch.softmax(torch.randn(R, C, generator=g, device="cuda") * 3, -1).to(t)
+    dy = torch.randn(R, C, generator=g, device="cuda").to(t)
+    outs = []
+    for p in POLICIES:
+        dx = torch.full_like(y, float("nan"))
+        bsm.bsm_softmax_backward(y, dy, dx, 1, R, C, dtype, p)
+        outs.append(dx)
+    bsm.bsm_softmax_backward(y, dy, dy2 := dy.clone(), 1, R, C, dtype, bsm.POLICY_DYNAMIC)
+    bsm.bsm_set_device_checks(True)
+    dx = torch.full_like(y, float("nan"))
+    bsm.bsm_softmax_backward(y, dy, dx, 1, R, C, dtype, bsm.POLICY_DYNAMIC)
+    torch.cuda.synchronize()
+    bsm.bsm_set_device_checks(False)
+    assert bsm.bsm_device_status() == 0, bsm.bsm_device_debug()
+    for o in outs[1:] + [dx]:
+        assert torch.equal(bits(o), bits(outs[0]))
+    assert not torch.isnan(outs[0]).any() and not torch.isnan(dy2).any()
+    pick = [0, 1, R // 2, R - 1]
+    w = workload.Workload("cluster bwd", dtype, np.full(4, 1, np.int32), np.full(4, C, np.int32),
+                          np.arange(4, dtype=np.int64) * C, 0, 0, 1.0)
+    _check(w, *(to_host(v[pick].reshape(-1)) for v in (y, dy)), to_host(outs[0][pick].reshape(-1)))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("nvec", [9000, 15000])
+def test_non_finite_and_lowest_value_rows(dtype, nvec):
+    import torch
+    t = torch.float32 if dtype == "f32" else torch.bfloat16
+    C, R = nvec * (4 if dtype == "f32" else 8), _rows()
+    low = torch.finfo(t).min
+    x = torch.randn(R, C, device="cuda").to(t)
+    x[1, C - 1] = float("nan")
+    x[2, 5] = float("inf")
+    x[3, :] = -float("inf")
+    x[3, C // 2] = 1.0
+    x[4, :] = -float("inf")
+    x[5, :] = low
+    x[5, C - 3] = 2.0
+    x[6, 8:] = low
+    y = torch.full_like(x, -1.0)
+    bsm.bsm_softmax(x, y, 1, R, C, bsm.F32 if dtype == "f32" else bsm.BF16, bsm.POLICY_DYNAMIC)
+    torch.cuda.synchronize()
+    assert torch.isnan(y[[1, 2, 4]]).all()
+    assert float(y[3, C // 2]) == 1.0 and int(y[3].count_nonzero()) == 1
+    assert float(y[5, C - 3]) == 1.0 and int(y[5].count_nonzero()) == 1
+    rest = [0] + list(range(6, R))
+    ref = torch.softmax(x[rest].double(), -1)
+    err = (y[rest].double() - ref).abs()
+    assert float(err.max()) <= 2e-6 if dtype == "f32" else bool((err <= ref * 2.0 ** -8 + 1e-30).all())
+
+
+def test_backward_withheld_stage_and_corrupted_record():
+    import time
+    import torch
+    R, C = _rows(), 20000
+    y = torch.softmax(torch.randn(R, C, device="cuda"), -1)
+    dy = torch.randn(R, C, device="cuda")
+    dx = torch.full_like(y, -7.0)
+    p = bsm.bsm_plan_create(y, dx, [R], [C], bsm.F32, bsm.POLICY_DYNAMIC, op=bsm.OP_BACKWARD, x2=dy)
+    bsm.bsm_plan_debug(p, bsm.DEBUG_WITHHOLD_STAGE, 100_000_000)
+    t0 = time.time()
+    p.execute()
+    torch.cuda.synchronize()
+    assert time.time() - t0 < 5.0
+    assert bsm.bsm_device_status() & bsm.DEV_TIMEOUT
+    bsm.bsm_plan_debug(p, bsm.DEBUG_NONE)
+    bsm.bsm_device_status_clear()
+    dx.fill_(-7.0)
+    bsm.bsm_plan_debug(p, bsm.DEBUG_CORRUPT_PATCH, 11)
+    p.execute()
+    torch.cuda.synchronize()
+    assert bsm.bsm_device_status() == bsm.DEV_BOUNDS
+    bsm.bsm_device_status_clear()
+    skipped = (dx == -7.0).all(1).nonzero().flatten().tolist()
+    assert skipped == [11]
+    keep = [r for r in range(R) if r != 11]
+    yd, gd = y[keep].double(), dy[keep].double()
+    ref = yd * (gd - (yd * gd).sum(-1, keepdim=True))
+    assert float((dx[keep].double() - ref).abs().max()) < 1e-7
+    p.close()
