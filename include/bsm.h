@@ -53,10 +53,10 @@
  *   - Row length: a row of up to bsm_max_row_bytes() (half of it for the
  *     backward pass, where y and dy share a stage) is read once from one
  *     shared-memory stage, by one warp or, past 2 KiB, by a team of up to 16.
- *     Batches of longer rows, at least two per SM, run over clusters of 2 or 4
- *     SMs: each takes a part of the row in one of its stages and every element
- *     is read once (rows of up to 452 KiB, 226 KiB backward).  Other longer
- *     rows go through the stages in chunks, in two passes -- a running maximum
+ *     Batches of longer rows, at least two per SM, run over clusters of 2, 4, 8
+ *     or 16 SMs: each takes a part of the row in one of its stages and every
+ *     element is read once (rows of up to 1.7 MiB, 880 KiB backward).  Other
+ *     longer rows go through the stages in chunks, in two passes -- a running maximum
  *     and rescaled sum (backward: the dot product), then the output -- and are
  *     read again, all but their last chunk (a row of two chunks whose halves
  *     fit three stages stays staged).  When a batch has fewer such rows than
@@ -65,9 +65,10 @@
  *     each row stays on one SM within one launch.  Forward rows of 5 to 32
  *     parts of at most 64 KiB, enough of them to fill two thirds of the groups'
  *     waves, are instead split over groups of K CTAs (K = ceil(row / 64
- *     KiB); n_sm / K groups) in one cooperative launch: each CTA stages one
+ *     KiB); n_sm / K groups) in one cooperative launch -- each CTA stages one
  *     part, the group exchanges (offset, sum) partials through global memory
- *     and every element is read once.  Which path a row takes depends on the
+ *     and every element is read once -- or over clusters where those are
+ *     faster.  Which path a row takes depends on the
  *     rows of the batch and the device, never on the policy: every policy
  *     gives the same bits.
  */

@@ -144,6 +144,7 @@ struct bsm_plan {
     bsm::KernelArgs argsg{};         // rows over groups of CTAs (one cooperative launch)
     int64_t n_group = 0;
     int grid_g = 0;
+    int op_g = 0;                    // the kernel that runs them: groups, or clusters
     std::vector<Launch> whole_gpu;   // WHOLE_GPU: one launch per slice
     cudaGraphExec_t whole_graph = nullptr;   // ... captured once as a CUDA graph (or null)
     void *blob = nullptr;            // device tables (patches, slice index, sm_die, heads)
@@ -355,47 +356,60 @@ int choose_groups(const std::vector<SliceView> &slices, int es, int n_sm, int64_
     return 1;
 }
 
-// Rows over clusters of CTAs: batches whose every patch is a whole row longer
-// than a stage (so at least two per SM, too short for the groups).  The
-// smallest cluster whose parts fit two stages; K = 0: none does, or too few
-// clusters are resident at once.  Which batches: by row lengths, their number
-// and the device only, never by the policy.
+// Rows over clusters of CTAs (softmax_cluster), for the records of whole rows
+// `items`: the smallest cluster whose parts fit two stages, unless a table of
+// rows for groups of CTAs (group_k > 0) runs faster there.  By row lengths,
+// their number and the device only, never by the policy.
+//
+// Why the smallest: the larger the cluster, the fewer SMs take part (clusters
+// share a GPC: 76 of 2, 36 of 4, 15 of 8, 7 of 16 are resident at once, 152,
+// 144, 120 and 112 SMs), and a part of 57 to 113 KiB runs like a row of that
+// length.  Against groups, GB/s over 256 MiB: fp32 320 KiB rows (K = 4) 6512 /
+// 5680, 512 KiB (8) 6291 / 5668, 768 KiB (8) 6372 / 5775, 1 MiB (16) 5671 /
+// 5472, 1.5 MiB (16) 5885 / 5185; bf16 384 KiB (4) 6410 / 5360, 512 KiB (8) 5234
+// / 5343, 1 MiB (16) 4710 / 5136 (a bf16 part costs as many exponentials as an
+// fp32 part twice as long: on 112 SMs they bound it).  Against one CTA a row,
+// backward: 256 KiB (8) 5900 / 5344, 384 KiB (8) 6660 / 4700, 768 KiB (16) 6100 /
+// 4150.
 struct ClusterChoice {
     int K = 0, units = 0, n_stages = 0;
     int64_t stage = 0;
 };
 
-ClusterChoice choose_clusters(const PatchLayout &L, int dtype, bool bwd, int n_sm, int64_t smem_optin)
+ClusterChoice choose_clusters(const std::vector<Item> &items, int dtype, bool bwd, int n_sm, int64_t smem_optin,
+                              int group_k)
 {
+    const ClusterChoice none;
     ClusterChoice c;
-    if (L.items.empty() || L.segs.size() != L.items.size() || !L.items1.empty() || !L.items_g.empty())
-        return c;
     int64_t lmax = 0;
-    for (size_t i = 0; i < L.items.size(); ++i) {
-        if (L.segs[i].part_count != 1)
-            return c;
-        lmax = std::max<int64_t>(lmax, L.items[i].C);
-    }
-    const int64_t avail = smem_optin - kClusterHeader, arrays = bwd ? 2 : 1;
-    const int64_t nv = (lmax * esize(dtype) + 15) / 16;
-    for (int K : {2, 4}) {
-        const int64_t stage = arrays * ((((nv + K - 1) / K) * 16 + 127) & ~int64_t(127));
-        const int n_stages = static_cast<int>(std::min<int64_t>(kMaxStages, avail / stage));
-        if (n_stages < 2)
-            continue;
-        int units = 0;
-        if (cluster_units(dtype, bwd, K, n_sm, static_cast<int>(kClusterHeader + n_stages * stage), &units)) {
-            cudaGetLastError();
-            return c;
-        }
-        units = std::min(units, n_sm / K);
-        if (units * K * 8 < n_sm * 7)          // more than an eighth of the SMs would idle
-            return c;
+    for (const Item &it : items)
+        lmax = std::max<int64_t>(lmax, it.C);
+    const int64_t arrays = bwd ? 2 : 1, nv = (lmax * esize(dtype) + 15) / 16;
+    for (int K : {2, 4, 8, 16}) {
         c.K = K;
-        c.units = units;
-        c.n_stages = n_stages;
-        c.stage = stage;
-        return c;
+        c.stage = arrays * ((((nv + K - 1) / K) * 16 + 127) & ~int64_t(127));
+        c.n_stages = static_cast<int>(std::min<int64_t>(kMaxStages, (smem_optin - cluster_header(K)) / c.stage));
+        if (c.n_stages >= 2)
+            break;
+    }
+    if (lmax == 0 || c.n_stages < 2)
+        return none;
+    if (cluster_units(dtype, bwd, c.K, n_sm, static_cast<int>(cluster_header(c.K) + c.n_stages * c.stage), &c.units)) {
+        cudaGetLastError();
+        return none;
+    }
+    c.units = std::min(c.units, n_sm / c.K);
+    if (c.units * c.K * 8 < n_sm * 5)          // three eighths of the SMs would idle: another device's clusters
+        return none;
+    if (group_k > 0) {
+        // the two measured rates (TB/s, all units busy) and the rows' waves
+        const double n = static_cast<double>(items.size()), f32 = dtype == BSM_F32;
+        const double rate = c.K <= 4 ? 6.4 : c.K == 8 ? (f32 ? 6.3 : 5.3) : (f32 ? 5.7 : 4.75);
+        const double at = c.K == 2 ? 76 : c.K == 4 ? 36 : c.K == 8 ? 15 : 7;
+        const double groups = n_sm / group_k;
+        const double g_rate = group_k <= 12 ? (f32 ? 5.65 : 5.35) : (f32 ? 5.2 : 5.0);
+        if (std::ceil(n / c.units) * at / rate > std::ceil(n / groups) * groups / g_rate)
+            return none;
     }
     return c;
 }
@@ -628,7 +642,7 @@ cudaGraphExec_t capture_whole_gpu(const bsm_plan *p)
             KernelArgs &al = l.phase == 2 ? ag : (l.phase ? a1 : a);
             al.item_begin = l.begin;
             al.item_end = l.end;
-            if (launch_softmax(al, p->dtype, l.phase == 2 ? OP_FORWARD_GROUP : p->kernel_op, l.grid, st, false)) {
+            if (launch_softmax(al, p->dtype, l.phase == 2 ? p->op_g : p->kernel_op, l.grid, st, false)) {
                 ok = false;
                 break;
             }
@@ -704,12 +718,19 @@ int plan_create_impl(bsm_plan **out, const bsm_plan_desc *d)
     std::vector<Item> all(items);
     all.insert(all.end(), items_g.begin(), items_g.end());
 
-    ClusterChoice cl;
+    ClusterChoice cl, clg;                     // of the regular rows, of the group rows
     {
         int prev = -1;
         cudaGetDevice(&prev);
         cudaSetDevice(device);
-        cl = choose_clusters(lay, d->dtype, d->op == BSM_OP_BACKWARD, c->n_sm, c->smem_optin);
+        // every patch a whole row longer than a stage (so at least two per SM)
+        bool whole = !lay.items.empty() && lay.segs.size() == lay.items.size() && lay.items1.empty() && lay.items_g.empty();
+        for (size_t i = 0; whole && i < lay.segs.size(); ++i)
+            whole = lay.segs[i].part_count == 1;
+        if (whole)
+            cl = choose_clusters(lay.items, d->dtype, d->op == BSM_OP_BACKWARD, c->n_sm, c->smem_optin, 0);
+        if (!lay.items_g.empty())
+            clg = choose_clusters(lay.items_g, d->dtype, false, c->n_sm, c->smem_optin, lay.group_k);
         if (prev >= 0)
             cudaSetDevice(prev);
     }
@@ -1054,6 +1075,15 @@ int plan_create_impl(bsm_plan **out, const bsm_plan_desc *d)
         ag.ring = reinterpret_cast<unsigned long long *>(b + o_ring);
         ag.xch = reinterpret_cast<unsigned long long *>(b + o_xch);
         p->grid_g = lay.group_k * lay.n_groups;
+        p->op_g = OP_FORWARD_GROUP;
+        if (clg.K) {
+            ag.stage_bytes = static_cast<int32_t>(clg.stage);
+            ag.n_stages = clg.n_stages;
+            ag.group_k = clg.K;
+            ag.n_groups = clg.units;
+            p->grid_g = clg.K * clg.units;
+            p->op_g = OP_FORWARD_CLUSTER;
+        }
     }
 
     if (cl.K) {
@@ -1193,7 +1223,7 @@ int plan_execute_impl(const bsm_plan *p, bsm_stream_t stream)
             KernelArgs &al = l.phase == 2 ? ag : (l.phase ? a1 : a);
             al.item_begin = l.begin;
             al.item_end = l.end;
-            if ((err = launch_softmax(al, p->dtype, l.phase == 2 ? OP_FORWARD_GROUP : p->kernel_op, l.grid, stream,
+            if ((err = launch_softmax(al, p->dtype, l.phase == 2 ? p->op_g : p->kernel_op, l.grid, stream,
                                       checked)))
                 break;
         }
@@ -1203,7 +1233,7 @@ int plan_execute_impl(const bsm_plan *p, bsm_stream_t stream)
         if (!err && p->n_phase1)
             err = launch_softmax(p->args1, p->dtype, p->kernel_op, p->grid, stream, checked);
         if (!err && p->n_group)
-            err = launch_softmax(p->argsg, p->dtype, OP_FORWARD_GROUP, p->grid_g, stream, checked);
+            err = launch_softmax(p->argsg, p->dtype, p->op_g, p->grid_g, stream, checked);
     }
     if (prev >= 0 && prev != p->device)
         cudaSetDevice(prev);
@@ -1403,7 +1433,7 @@ int bsm_plan_device_table(const bsm_plan *plan, int phase, bsm_patch *out, int64
         out[i].row0 = items[i].row0;
         out[i].slice_rows = items[i].R;
         out[i].col0 = segs.empty() ? 0 : segs[i].col0;
-        out[i].part_count = phase == 2 ? -a.group_k : (segs.empty() ? 0 : segs[i].part_count);
+        out[i].part_count = phase == 2 ? -plan->stats.group_k : (segs.empty() ? 0 : segs[i].part_count);
     }
     return BSM_OK;
 }

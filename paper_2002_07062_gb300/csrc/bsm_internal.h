@@ -39,8 +39,11 @@ constexpr int kConsumerWarps = 16;
 constexpr int kThreads = (kConsumerWarps + 1) * 32;  // + one producer warp
 constexpr int kGroupThreads = kThreads + 32;          // rows over groups: + one exchange warp
 constexpr int kSmemHeader = 1024;                     // barriers + stage metadata
-constexpr int kClusterHeader = 1536;                  // the same of rows over clusters of CTAs
-constexpr int kMaxCluster = 4;
+constexpr int kClusterHeader = 512;                   // the same of rows over clusters of CTAs,
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr int cluster_header(int K) { return kClusterHeader + 2 * K * kConsumerWarps * 8; }   // and their partials
 // Smallest stage (three fit the shared memory).  Each stage has a fixed cost
 // (wait, metadata, dispatch, release) that larger stages amortise; measured
 // over 32 KiB stages: bf16 +11 % causal 512-wide rows, +16 % 32 x 128 slices;

@@ -2550,7 +2550,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1) softmax_group(const KernelAr
 
 // ------------------------------------------------ rows over clusters of CTAs
 // Batches of rows too long for one stage, enough of them to fill the SMs: a
-// cluster of K = 2 or 4 CTAs shares a row, a part of it in one stage of each
+// cluster of K = 2, 4, 8 or 16 CTAs shares a row, a part of it in one stage of each
 // (the parts of a row of 64 to 113 KiB are what a team of 16 warps takes
 // alone), so every element is read once.  The row routines are the teams',
 // W = 16; the exchange goes over the cluster: every warp sends its (offset, sum)
@@ -2579,7 +2579,6 @@ struct ClusterSmem {
     uint64_t xbar[2];                   // a row's partials are in, by row parity
     unsigned long long ring[kClusterRing];
     ClusterMeta meta[kMaxStages];
-    float2 part[2][kMaxCluster * kConsumerWarps];
     int32_t abort_flag;
 };
 static_assert(sizeof(ClusterSmem) <= kClusterHeader, "cluster header too large");
@@ -2624,6 +2623,34 @@ __device__ __forceinline__ bool cluster_spin_bounded(uint64_t *bar, uint32_t par
     return false;
 }
 
+// The row's (offset, sum) or dot product from 32 P pairs in shared memory, P a
+// lane: fixed trees, the loads and exponentials of a lane independent of one
+// another (a loop over them cost 12 % on bf16 256 KiB rows).
+template <int P> __device__ __forceinline__ float2 lanes_pairs(const float2 *in, int lane)
+{
+    float2 p[P];
+    float o[P], t[P];
+#pragma unroll
+    for (int j = 0; j < P; ++j) {
+        p[j] = in[lane + 32 * j];
+        o[j] = p[j].x;
+    }
+    const float O = warp_max(tree_max<P>(o));
+#pragma unroll
+    for (int j = 0; j < P; ++j)
+        t[j] = p[j].y * ex2(p[j].x - O);
+    return make_float2(O, group_sum<32>(tree_sum<P>(t)));
+}
+
+template <int P> __device__ __forceinline__ float lanes_dot(const float2 *in, int lane)
+{
+    float t[P];
+#pragma unroll
+    for (int j = 0; j < P; ++j)
+        t[j] = in[lane + 32 * j].x;
+    return group_sum<32>(tree_sum<P>(t));
+}
+
 template <typename Tag, bool Bwd, bool Checked>
 __global__ void __launch_bounds__(kThreads, 1) softmax_cluster(const KernelArgs a)
 {
@@ -2631,7 +2658,8 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_cluster(const KernelArgs 
     constexpr int EPV = E::kPerVec, kArrays = Bwd ? 2 : 1;
     extern __shared__ __align__(1024) unsigned char smem[];
     ClusterSmem &h = *reinterpret_cast<ClusterSmem *>(smem);
-    unsigned char *stages = smem + kClusterHeader;
+    float2 *parts = reinterpret_cast<float2 *>(smem + kClusterHeader);     // [2][K * 16], by row parity
+    unsigned char *stages = smem + cluster_header(a.group_k);
     const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int S = a.n_stages, K = a.group_k, half = a.stage_bytes / 2;
     const int unit = static_cast<int>(blockIdx.x) / K, n_units = static_cast<int>(gridDim.x) / K;
@@ -2801,7 +2829,7 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_cluster(const KernelArgs 
                     if (src < x0 || src + bytes > x0 + all || (reinterpret_cast<uintptr_t>(src) & 15) ||
                         (Bwd && (src2 < g0 || src2 + bytes > g0 + all || (reinterpret_cast<uintptr_t>(src2) & 15))) ||
                         (smem_addr(dst) & 15) || (half & 15) || bytes > static_cast<uint32_t>(Bwd ? half : a.stage_bytes) ||
-                        dst + a.stage_bytes > smem + kClusterHeader + static_cast<size_t>(S) * a.stage_bytes) {
+                        dst + a.stage_bytes > stages + static_cast<size_t>(S) * a.stage_bytes) {
                         check_fail(a.status, 3, pos, bytes);
                         mt.kind = KIND_SKIP;       // the cluster's other CTAs time out
                         mbar_arrive(full);
@@ -2846,29 +2874,31 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_cluster(const KernelArgs 
         int s = 0;
         uint32_t ph = 0;
         bool ok = true;
-        // this warp's pair to every CTA of the cluster, then all warps' pairs:
-        // one of them per lane (of 64, two).  Barrier and slots alternate by
-        // row: a warp sends row t + 2's after it has row t + 1's pairs, which
-        // every warp sent after it had taken row t's.
-        auto gather = [&](float2 mine, float2 none, float2 &p0, float2 &p1) -> bool {
+        // this warp's pair to every CTA of the cluster; true once all the
+        // cluster's are in, at parts_in.  Barrier and slots alternate by row:
+        // a warp sends row t + 2's after it has row t + 1's pairs, which every
+        // warp sent after it had taken row t's.
+        const int n_pairs = K * kConsumerWarps;
+        const float2 *parts_in = nullptr;
+        auto gather = [&](float2 mine) -> bool {
             const uint32_t par = x & 1u;
+            float2 *in = parts + par * n_pairs;
             if (warp == 0 && lane == 0)
-                mbar_arrive_expect_tx(&h.xbar[par], static_cast<uint32_t>(K * kConsumerWarps * sizeof(float2)));
+                mbar_arrive_expect_tx(&h.xbar[par], static_cast<uint32_t>(n_pairs * sizeof(float2)));
             __syncwarp();
             if (lane < K) {
                 unsigned long long w;
                 asm("mov.b64 %0, {%1, %2};" : "=l"(w) : "f"(mine.x), "f"(mine.y));
                 asm volatile(
                     "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(
-                        cluster_addr(&h.part[par][rank * kConsumerWarps + warp], lane)),
+                        cluster_addr(&in[rank * kConsumerWarps + warp], lane)),
                     "l"(w), "r"(cluster_addr(&h.xbar[par], lane))
                     : "memory");
             }
             if (!__all_sync(0xFFFFFFFFu, cluster_spin_bounded(&h.xbar[par], (x >> 1) & 1u, &h.abort_flag, wait_limit)))
                 return false;
             ++x;
-            p0 = lane < K * kConsumerWarps ? h.part[par][lane] : none;
-            p1 = lane + 32 < K * kConsumerWarps ? h.part[par][lane + 32] : none;
+            parts_in = in;
             return true;
         };
         for (;;) {
@@ -2898,10 +2928,12 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_cluster(const KernelArgs 
             const Bounds bd{sbuf, sbuf + bytes, y, y + a.total_elems * E::kSize, a.status};
             if constexpr (Bwd) {
                 auto exchange = [&](float &dot) -> bool {
-                    float2 p0, p1;
-                    if (!gather(make_float2(dot, 0.0f), make_float2(0.0f, 0.0f), p0, p1))
+                    if (!gather(make_float2(dot, 0.0f)))
                         return false;
-                    dot = group_sum<32>(p0.x + p1.x);
+                    dot = K == 2   ? lanes_dot<1>(parts_in, lane)
+                          : K == 4 ? lanes_dot<2>(parts_in, lane)
+                          : K == 8 ? lanes_dot<4>(parts_in, lane)
+                                   : lanes_dot<8>(parts_in, lane);
                     return true;
                 };
                 const Bounds bdy{sbuf + half, sbuf + half + bytes, y, y + a.total_elems * E::kSize, a.status};
@@ -2914,11 +2946,12 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_cluster(const KernelArgs 
             } else {
                 const int row = h.meta[s0].row0, col0 = h.meta[s0].col0;
                 auto exchange = [&](float2 &os) -> bool {
-                    float2 p0, p1;
-                    if (!gather(os, make_float2(-INFINITY, 0.0f), p0, p1))
+                    if (!gather(os))
                         return false;
-                    os.x = warp_max(fmaxf(p0.x, p1.x));
-                    os.y = group_sum<32>(p0.y * ex2(p0.x - os.x) + p1.y * ex2(p1.x - os.x));
+                    os = K == 2   ? lanes_pairs<1>(parts_in, lane)
+                         : K == 4 ? lanes_pairs<2>(parts_in, lane)
+                         : K == 8 ? lanes_pairs<4>(parts_in, lane)
+                                  : lanes_pairs<8>(parts_in, lane);
                     return true;
                 };
                 if (nvec >= (kTeamVecs - 2) * kConsumerWarps * 32)
@@ -3058,8 +3091,15 @@ cudaError_t cluster_launch(const KernelArgs *a, int K, int grid, size_t smem, cu
 #ifdef BSM_NO_PDL
     cfg.numAttrs = 1;
 #endif
-    if (units)
+    if (units) {
+        // clusters of 16 are past the portable size: allowed once, before the
+        // first plan that uses them
+        for (const void *f : {reinterpret_cast<const void *>(softmax_cluster<Tag, Bwd, false>),
+                              reinterpret_cast<const void *>(softmax_cluster<Tag, Bwd, true>)})
+            if (cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1))
+                return e;
         return cudaOccupancyMaxActiveClusters(units, softmax_cluster<Tag, Bwd, false>, &cfg);
+    }
     if (checked)
         return cudaLaunchKernelEx(&cfg, softmax_cluster<Tag, Bwd, true>, *a);
     return cudaLaunchKernelEx(&cfg, softmax_cluster<Tag, Bwd, false>, *a);
@@ -3088,7 +3128,7 @@ int launch_softmax(const KernelArgs &a, int dtype, int op, int grid, void *strea
     const size_t smem = kSmemHeader + (size_t)a.n_stages * a.stage_bytes;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (op == OP_FORWARD_CLUSTER || op == OP_BACKWARD_CLUSTER) {
-        const size_t csmem = kClusterHeader + (size_t)a.n_stages * a.stage_bytes;
+        const size_t csmem = cluster_header(a.group_k) + (size_t)a.n_stages * a.stage_bytes;
         const cudaError_t e = cluster_dispatch(&a, dtype, op == OP_BACKWARD_CLUSTER, a.group_k, grid, csmem, st, checked,
                                                nullptr);
         const cudaError_t l = cudaGetLastError();

@@ -1,4 +1,4 @@
-"""Batches of rows longer than a stage that clusters of 2 or 4 CTAs share,
+"""Batches of rows longer than a stage that clusters of 2 to 16 CTAs share,
 against the oracle (sampled rows) and bit-identical across policies: the
 lengths at which the cluster grows and parts of unequal length, the causal
 mask across parts, NaN, +inf, all -inf and masks of the type's lowest value,
@@ -13,9 +13,10 @@ pytestmark = pytest.mark.gpu
 
 POLICIES = [bsm.POLICY_DYNAMIC, bsm.POLICY_RR, bsm.POLICY_CBMF, bsm.POLICY_CBMF_LB, bsm.POLICY_WHOLE_GPU]
 # 16-byte vectors per row: just past a stage, odd parts, either side of the
-# largest row of two CTAs, up to the rows that groups take
-FWD = [7233, 8195, 14431, 14433, 16383]
-BWD = [3617, 4099, 7213, 7219, 14401]
+# largest row of two CTAs, then rows of 4, 8 and 16 (forward rows of more than
+# 16384 vectors are those that groups take otherwise)
+FWD = [7233, 8195, 14463, 14465, 16383, 28845, 40001, 70003]
+BWD = [3617, 4099, 7231, 7233, 14401, 20003, 29001]
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -29,9 +30,10 @@ def setup():
     bsm.bsm_cache_clear()
 
 
-def _rows():
+def _rows(nvec=0):
     import torch
-    return 2 * torch.cuda.get_device_properties(0).multi_processor_count + 5
+    # (rows for groups: a few waves of them, whichever kernel runs)
+    return 150 if nvec > 16384 else 2 * torch.cuda.get_device_properties(0).multi_processor_count + 5
 
 
 @pytest.mark.parametrize("nvec", FWD)
@@ -40,7 +42,7 @@ def _rows():
 def test_forward_row_lengths(nvec, dtype, flags):
     import torch
     C = nvec * (4 if dtype == workload.F32 else 8)
-    w = workload.uniform("cluster", dtype, 5, (_rows() + 4) // 5, C, 3.0, 0xC10 + nvec + flags, flags).materialize()
+    w = workload.uniform("cluster", dtype, 5, (_rows(nvec) + 4) // 5, C, 3.0, 0xC10 + nvec + flags, flags).materialize()
     x = to_device(w.x)
     ys = [run(w, x, p) for p in POLICIES]
     bsm.bsm_set_device_checks(True)
