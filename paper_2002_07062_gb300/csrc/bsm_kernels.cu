@@ -14,13 +14,14 @@
 //
 // Row routine (the arithmetic, identical under every policy): a row is owned
 // by a group of T lanes; lane l owns the 16-byte vectors l, l + T, l + 2T, ...
-// The maximum and the sum are per vector (a balanced tree), per lane in vector
-// order, then a butterfly (xor) shuffle tree over the group.  By row length in
-// 16-byte vectors: <= 8: T = 8, 1 vector per lane; <= 16: T = 8, 2; <= 32:
-// T = 8, 4; <= 64: T = 16, 4; <= 128: T = 32, 4 -- all in registers (at most
-// 32 elements per lane); longer rows: a team of 1 to 16 warps, up to 8 vectors
-// per lane in registers (see row_team).  exp(t) is evaluated as 2^(t*log2 e) with
-// the exponent formed by one fused multiply-add, v*log2e - m*log2e, and the
+// The maximum is exact; the sum is per vector (a balanced tree), per lane in
+// vector order, then a butterfly (xor) shuffle tree over the group.  By row
+// length in 16-byte vectors: 1: T = 1, 1 vector per lane; 2: T = 1, 2; <= 4:
+// T = 2, 2; <= 8: T = 4, 2; <= 16: T = 8, 2; <= 32: T = 8, 3 or 4; <= 64:
+// T = 16, 3 or 4; <= 128: T = 32, 3 or 4 -- all in registers (see
+// rows_in_lanes); longer rows: a team of 1 to 16 warps, up to 8 vectors per
+// lane in registers (see row_team).  exp(t) is evaluated as 2^(t*log2 e) with
+// the exponent formed by one fused multiply-add, v*log2e - offset, and the
 // power of two from the PTX ex2.approx instruction; y = p * (1/sum).
 //
 // Every wait is bounded (2 s of wall time unless the launch asks for less):
@@ -395,62 +396,6 @@ __device__ __forceinline__ void apply_causal(float (&v)[EPV], int col0, int row)
         v[e] += (col0 + e > row) ? -INFINITY : 0.0f;
 }
 
-// Register-resident fp32 row: T lanes, up to V vectors per lane, scalar
-// arithmetic (fp32 rows move 8 bytes per element: memory, not instruction
-// issue, bounds them).  Under the causal mask a vector is unmasked (all its
-// columns <= row), on the diagonal (masked element by element) or wholly
-// masked (it adds nothing to the max; its p is 0 or NaN, see vec_exp).
-template <typename Tag, bool Checked, int T, int V>
-__device__ __forceinline__ void row_in_registers_scalar(const unsigned char *srow, unsigned char *yrow,
-                                                 int nvec, int row, bool causal, int l, bool valid,
-                                                 const Bounds &bd)
-{
-    using E = Elem<Tag>;
-    constexpr int EPV = E::kPerVec;
-    float v[V][EPV];
-    float m = -INFINITY;
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-        const int vi = j * T + l;
-        const bool masked = causal && vi * EPV > row;
-        uint4 raw;
-        if (valid && vi < nvec && load_vec<Checked>(srow + 16 * vi, bd, raw)) {
-            E::unpack(raw, v[j]);
-            if (!masked) {
-                if (causal && vi * EPV + EPV - 1 > row)
-                    apply_causal<EPV>(v[j], vi * EPV, row);
-                m = fmaxf(m, tree_max<EPV>(v[j]));
-            }
-        } else {
-#pragma unroll
-            for (int e = 0; e < EPV; ++e)
-                v[j][e] = -INFINITY;
-        }
-    }
-    m = group_max<T>(m);
-    const float mL = m * kLog2e;
-    float s = 0.0f;
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-        const int vi = j * T + l;
-        vec_exp<EPV>(v[j], mL, (causal && vi * EPV > row) || vi >= nvec);
-        if (vi < nvec)
-            s += tree_sum<EPV>(v[j]);
-    }
-    s = group_sum<T>(s);
-    const float inv = __frcp_rn(s);
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-        const int vi = j * T + l;
-        if (valid && vi < nvec) {
-#pragma unroll
-            for (int e = 0; e < EPV; ++e)
-                v[j][e] *= inv;
-            store_vec<Checked>(yrow + 16 * vi, bd, E::pack(v[j]));
-        }
-    }
-}
-
 // ------------------------------------------------ fp32 pair arithmetic
 // One instruction, two IEEE operations, each rounded like its scalar form.
 // As 64-bit registers (Pair): a constant pair is made once, not at each use.
@@ -513,57 +458,12 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b)
     return d;
 }
 
-__device__ __forceinline__ float2 mul2(float2 a, float2 b)
-{
-    float2 d;
-    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
-        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
-        "mul.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return d;
-}
-
-// p = 2^(v*log2e - mL) for one vector, in pairs; returns the vector's sum as
-// a pair: ((p0,p1) + (p2,p3)) [+ ((p4,p5) + (p6,p7))].
-template <int EPV>
-__device__ __forceinline__ float2 vec_exp_pairs(float (&v)[EPV], float mL)
-{
-    const float2 l2 = make_float2(kLog2e, kLog2e), nm = make_float2(-mL, -mL);
-#pragma unroll
-    for (int e = 0; e < EPV; e += 2) {
-        const float2 t = fma2(make_float2(v[e], v[e + 1]), l2, nm);
-        v[e] = ex2(t.x);
-        v[e + 1] = ex2(t.y);
-    }
-    const float2 a = add2(make_float2(v[0], v[1]), make_float2(v[2], v[3]));
-    if constexpr (EPV == 4)
-        return a;
-    else
-        return add2(a, add2(make_float2(v[4], v[5]), make_float2(v[6], v[7])));
-}
-
 // Element-wise maximum of two bf16 pairs.
 __device__ __forceinline__ uint32_t bmax2(uint32_t a, uint32_t b)
 {
     uint32_t d;
     asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
     return d;
-}
-
-// True when one of the vector's elements is NaN or +inf (such an element
-// masked by the causal mask still turns its row into NaN: NaN + (-inf) and
-// +inf + (-inf) are NaN); a NaN-propagating maximum over the raw vector.
-template <typename Tag> __device__ __forceinline__ bool vec_poisons(uint4 r);
-template <> __device__ __forceinline__ bool vec_poisons<BF16>(uint4 r)
-{
-    uint32_t w;
-    asm("{\n\t.reg .b32 a, b;\n\tmax.NaN.bf16x2 a, %1, %2;\n\tmax.NaN.bf16x2 b, %3, %4;\n\t"
-        "max.NaN.bf16x2 %0, a, b;\n\t}"
-        : "=r"(w)
-        : "r"(r.x), "r"(r.y), "r"(r.z), "r"(r.w));
-    const float lo = __uint_as_float(w << 16), hi = __uint_as_float(w & 0xFFFF0000u);
-    return !(lo < INFINITY) || !(hi < INFINITY);
 }
 
 // p = 2^(v*log2e - mL) for one vector in fp32 pairs (each pair two IEEE
@@ -587,112 +487,6 @@ __device__ __forceinline__ float vec_exp_sum_pairs(float (&v)[EPV], float mL)
         const float2 b = add2(make_float2(v[2], v[6]), make_float2(v[3], v[7]));
         const float2 c = add2(a, b);
         return c.x + c.y;
-    }
-}
-
-// Register-resident bf16 row (bf16 rows move 4 bytes per element, so
-// instruction issue matters): T lanes, V vectors per lane (vector j of lane l
-// is vector j*T + l of the row).  Arithmetic, the same in both variants and
-// under every policy: m = max over the lane's vectors (balanced tree per
-// vector, vectors in order), butterfly over the lane group; p = 2^(v*log2e
-// - m*log2e) in fp32 pairs; the lane's sum is a pair accumulated vector by
-// vector, then its two halves, then the butterfly; y = p * (1/sum).
-// Full = true: every lane holds V vectors of a valid row and nothing needs a
-// bound (no per-vector predicates).  Under the causal mask each vector is
-// classed for the whole warp: unmasked everywhere (no mask work), masked
-// everywhere (p = 0 without an exponential; a NaN or +inf among its inputs
-// still makes the row NaN), or mixed (the additive -inf mask element by
-// element).  Results do not depend on the class: the mask's sums are exact.
-template <typename Tag, bool Checked, int T, int V, bool Full>
-__device__ __forceinline__ void row_in_registers_pairs(const unsigned char *srow, unsigned char *yrow,
-                                                 int nvec, int row, bool causal, int l, bool valid,
-                                                 const Bounds &bd)
-{
-    using E = Elem<Tag>;
-    constexpr int EPV = E::kPerVec;
-    float v[V][EPV];
-    uint32_t skip = 0;          // bit j: vector j is masked for the whole warp
-    bool poison = false;
-    float m = -INFINITY;
-    uint32_t mw = 0xFF80FF80u;  // running maximum of the unmasked vectors, two bf16 halves
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-        const int vi = j * T + l;
-        const int col0 = vi * EPV;
-        const bool in = Full || (valid && vi < nvec);
-        // the vector's mask class depends on its position only (warp-wide)
-        bool mixed = false;
-        if (causal) {
-            const bool lane_un = !in || col0 + EPV - 1 <= row;
-            const bool lane_mk = !in || col0 > row;
-            if (!__all_sync(0xFFFFFFFFu, lane_un)) {
-                if (__all_sync(0xFFFFFFFFu, lane_mk))
-                    skip |= 1u << j;
-                else
-                    mixed = true;
-            }
-        }
-        uint4 raw = E::neg_inf_vec();
-        if (Full) {
-            raw = lds128(srow + 16 * vi);
-        } else if (in) {
-            uint4 r;
-            if (load_vec<Checked>(srow + 16 * vi, bd, r))
-                raw = r;
-        }
-        if (skip & (1u << j)) {
-            if (in)
-                poison |= vec_poisons<Tag>(raw);
-#pragma unroll
-            for (int e = 0; e < EPV; ++e)
-                v[j][e] = 0.0f;
-            continue;
-        }
-        E::unpack(raw, v[j]);
-        if (mixed) {
-#pragma unroll
-            for (int e = 0; e < EPV; ++e)
-                v[j][e] += (col0 + e > row) ? -INFINITY : 0.0f;
-            m = fmaxf(m, tree_max<EPV>(v[j]));
-        } else {
-            // the maximum of bf16 values is exact in bf16: take it on the
-            // packed words (non-NaN operand wins, as fmaxf), unpack once
-            mw = bmax2(mw, bmax2(bmax2(raw.x, raw.y), bmax2(raw.z, raw.w)));
-        }
-    }
-    m = fmaxf(m, fmaxf(__uint_as_float(mw << 16), __uint_as_float(mw & 0xFFFF0000u)));
-    m = group_max<T>(m);
-    const float mL = m * kLog2e;
-    float2 acc = make_float2(0.0f, 0.0f);
-#pragma unroll
-    for (int j = 0; j < V; ++j)
-        if (!(skip & (1u << j)))
-            acc = add2(acc, vec_exp_pairs<EPV>(v[j], mL));
-    float s = acc.x + acc.y;
-    if (poison)
-        s = __int_as_float(0x7FC00000);
-    s = group_sum<T>(s);
-    const float inv = __frcp_rn(s);
-    const float2 inv2 = make_float2(inv, inv);
-    const float zero_y = 0.0f * inv;   // the output of a masked element (0, or NaN in a NaN row)
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-        const int vi = j * T + l;
-        if (Full || (valid && vi < nvec)) {
-            if (skip & (1u << j)) {
-#pragma unroll
-                for (int e = 0; e < EPV; ++e)
-                    v[j][e] = zero_y;
-            } else {
-#pragma unroll
-                for (int e = 0; e < EPV; e += 2) {
-                    const float2 y2 = mul2(make_float2(v[j][e], v[j][e + 1]), inv2);
-                    v[j][e] = y2.x;
-                    v[j][e + 1] = y2.y;
-                }
-            }
-            store_vec<Checked>(yrow + 16 * vi, bd, E::pack(v[j]));
-        }
     }
 }
 
@@ -752,7 +546,8 @@ template <> struct MaxAcc<BF16> {
 // No lower than the lowest float: there (m = -inf, or a mask of the type's
 // lowest value in every element seen) v*log2e - offset is -inf or far below 0
 // and adds 0 (NaN for a NaN), where m * log2 e = -inf would give inf - inf.
-__device__ __forceinline__ float exp_offset(float m) { return fmaxf(floorf(m * kLog2e), -3.402823466e38f); }
+constexpr float kLowest = -3.402823466e38f;
+__device__ __forceinline__ float exp_offset(float m) { return fmaxf(floorf(m * kLog2e), kLowest); }
 
 // Element pair k of a vector as loaded.
 template <typename Tag> __device__ __forceinline__ Pair vec_pair(uint4 r, int k);
@@ -1196,46 +991,6 @@ __device__ __forceinline__ void long_chunk_bwd(const unsigned char *sbuf, int ha
     }
 }
 
-// The rows of a stage handled by one register routine: groups of T lanes,
-// G = 32/T rows per group of a warp.  Row groups are dealt to the consumer
-// warps round robin, starting at warp `first` (see consume_stage); q tracks
-// each lane group's row inside its slice ((row0 + r) mod R) without a
-// division per row.  Returns the number of row groups of the stage.
-template <typename Tag, bool Checked, int T, int V>
-__device__ __forceinline__ int rows_in_registers(const unsigned char *sbuf, const StageMeta &mt,
-                                                 unsigned char *ybase, int row_bytes, int nvec,
-                                                 bool causal, int first, int lane, const Bounds &bd)
-{
-    constexpr int G = 32 / T;
-    const int g = lane / T, l = lane % T;
-    const int step = G * kConsumerWarps;
-    int q = 0, qstep = 0;
-    if (causal) {
-        q = (mt.row0 + first * G + g) % mt.R;
-        qstep = step % mt.R;
-    }
-    const bool full_rows = nvec == T * V;
-    for (int rb = first * G; rb < mt.nrows; rb += step) {
-        const int r = rb + g;
-        if constexpr (Elem<Tag>::kSize == 4)
-            row_in_registers_scalar<Tag, Checked, T, V>(sbuf + (size_t)r * row_bytes,
-                                                        ybase + (size_t)r * row_bytes, nvec, q, causal, l,
-                                                        r < mt.nrows, bd);
-        else if (full_rows && rb + G <= mt.nrows)   // warp-uniform
-            row_in_registers_pairs<Tag, Checked, T, V, true>(sbuf + (size_t)r * row_bytes,
-                                                             ybase + (size_t)r * row_bytes, nvec, q, causal, l,
-                                                             true, bd);
-        else
-            row_in_registers_pairs<Tag, Checked, T, V, false>(sbuf + (size_t)r * row_bytes,
-                                                              ybase + (size_t)r * row_bytes, nvec, q, causal, l,
-                                                              r < mt.nrows, bd);
-        q += qstep;
-        if (q >= mt.R)
-            q -= mt.R;
-    }
-    return (mt.nrows + G - 1) / G;
-}
-
 template <int N> struct Int {
     static constexpr int value = N;
 };
@@ -1428,12 +1183,97 @@ __device__ __forceinline__ bool consume_stage_team_bwd(SmemHeader &h, const unsi
     return W == 1 ? go(Int<1>{}) : W == 2 ? go(Int<2>{}) : W == 4 ? go(Int<4>{}) : W == 8 ? go(Int<8>{}) : go(Int<16>{});
 }
 
-// All rows of one stage that belong to this consumer warp, for rows that
-// one lane group's registers hold.  The routine
-// depends on the row length only (see the table at the top of the file).
-// Row groups are dealt round robin over the consumer warps starting at warp
-// `first`; the caller advances `first` by the returned group count, so a
-// stage with fewer groups than warps does not always land on the same warps.
+// Rows that one lane group's registers hold: T lanes, V vectors a lane (vector
+// j of lane l is vector j*T + l), of which only the last can be missing
+// ((V-1) * T <= nvec, see consume_stage).  Issue bounds these rows (shared
+// memory and the copies are ahead of it), so a group has no more lanes than
+// two to four vectors a lane leave: fewer steps of the two butterflies a row,
+// and no vector slot that is empty in every lane.  The mask is added to the
+// vectors as loaded, a missing vector is -inf, and nothing else has a bound;
+// rows past the patch repeat its last row and are not stored.  Maximum, offset
+// and 2^(v log2 e - offset) as in row_team; the exponentials stay in registers,
+// one per element.  Up to four vectors the offset is m log2 e itself: there the
+// largest element carries the sum, and 2^0 has no error (rounded down, the
+// error at unit variance is 8 % larger at 4 elements, 1 % at 16; at larger
+// variances and lengths rounding down has the smaller error).
+// GB/s over 256 MiB, bf16, groups of 8, 16 or 32 lanes with a bound on every
+// vector -> this routine: 16 B 828 -> 6728, 64 B 3020 -> 6821, 112 B 4821 ->
+// 6607, 192 B 5308 -> 6300, 256 B 6703 -> 6740, 528 B 4287 -> 6466, 1024 B
+// 6649 -> 6795, 1040 B 4233 -> 6327, 1232 B 4888 -> 6617; fp32: 16 B 888 ->
+// 6840, 64 B 3267 -> 6841, 528 B 5620 -> 6726, 2048 B 6799 -> 6848.
+template <typename Tag, bool Checked, int T, int V>
+__device__ __forceinline__ int rows_in_lanes(const unsigned char *sbuf, const StageMeta &mt, unsigned char *ybase,
+                                             int row_bytes, int nvec, bool causal, int first, int lane,
+                                             const Bounds &bd)
+{
+    using E = Elem<Tag>;
+    constexpr int EPV = E::kPerVec, N = EPV / 2, G = 32 / T, step = G * kConsumerWarps;
+    const int g = lane / T, l = lane % T;
+    const Pair l2 = pair(kLog2e, kLog2e);
+    const bool in_last = (V - 1) * T + l < nvec;
+    int q = 0, qstep = 0;
+    if (causal) {
+        q = (mt.row0 + first * G + g) % mt.R;
+        qstep = step % mt.R;
+    }
+    for (int rb = first * G; rb < mt.nrows; rb += step) {
+        const int r = rb + g;
+        const bool valid = r < mt.nrows;
+        const unsigned char *sp = sbuf + (size_t)(valid ? r : mt.nrows - 1) * row_bytes + 16 * l;
+        uint4 raw[V];
+        MaxAcc<Tag> mx;
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            raw[j] = E::neg_inf_vec();
+            if (j < V - 1 || in_last) {
+                uint4 u;
+                if (load_vec<Checked>(sp + 16 * j * T, bd, u))
+                    raw[j] = causal ? mask_vec<Tag>(u, (j * T + l) * EPV, q) : u;
+            }
+            mx.add(raw[j]);
+        }
+        const float m = group_max<T>(mx.get());
+        const float o = T > 2 ? exp_offset(m) : fmaxf(m * kLog2e, kLowest);
+        const Pair nm = pair(-o, -o);
+        Pair p[V][N], acc = pair(0.0f, 0.0f);
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+#pragma unroll
+            for (int k = 0; k < N; ++k)
+                p[j][k] = pair_ex2(pair_fma(vec_pair<Tag>(raw[j], k), l2, nm));
+            if constexpr (N == 4)
+                acc = pair_add(acc, pair_add(pair_add(p[j][0], p[j][1]), pair_add(p[j][2], p[j][3])));
+            else
+                acc = pair_add(acc, pair_add(p[j][0], p[j][1]));
+        }
+        const float2 a2 = halves(acc);
+        const float inv = __frcp_rn(group_sum<T>(a2.x + a2.y));
+        const Pair inv2 = pair(inv, inv);
+        unsigned char *yp = ybase + (size_t)r * row_bytes + 16 * l;
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+            if (valid && (j < V - 1 || in_last)) {
+                float2 y2[N];
+#pragma unroll
+                for (int k = 0; k < N; ++k)
+                    y2[k] = halves(pair_mul(p[j][k], inv2));
+                store_vec<Checked>(yp + 16 * j * T, bd, pack_pairs<Tag>(y2));
+            }
+        q += qstep;
+        if (q >= mt.R)
+            q -= mt.R;
+    }
+    return (mt.nrows + G - 1) / G;
+}
+
+// All rows of one stage that belong to this consumer warp, for rows that one
+// lane group's registers hold.  The routine depends on the row length only.
+// Two vectors a lane up to 16: 128-byte bf16 rows on 8 lanes of one 5905 GB/s,
+// on 4 of two 6788; 64-byte rows on 4 of one 5918, on 2 of two 6821.  Three
+// instead of four where three hold the row.  Row groups are dealt round robin
+// over the consumer warps starting at warp `first`; the caller advances
+// `first` by the returned group count, so a stage with fewer groups than warps
+// does not always land on the same warps.
 template <typename Tag, bool Checked>
 __device__ __forceinline__ int consume_stage(const unsigned char *sbuf, const StageMeta &mt, unsigned char *y,
                                              bool causal, int first, int lane, Bounds bd)
@@ -1444,15 +1284,22 @@ __device__ __forceinline__ int consume_stage(const unsigned char *sbuf, const St
     unsigned char *ybase = y + mt.off * E::kSize;
     bd.s_lo = sbuf;
     bd.s_hi = sbuf + (size_t)mt.nrows * row_bytes;
+    auto rows = [&](auto t, auto v) {
+        return rows_in_lanes<Tag, Checked, decltype(t)::value, decltype(v)::value>(sbuf, mt, ybase, row_bytes, nvec,
+                                                                                   causal, first, lane, bd);
+    };
     if (nvec <= 8)
-        return rows_in_registers<Tag, Checked, 8, 1>(sbuf, mt, ybase, row_bytes, nvec, causal, first, lane, bd);
-    if (nvec <= 16)
-        return rows_in_registers<Tag, Checked, 8, 2>(sbuf, mt, ybase, row_bytes, nvec, causal, first, lane, bd);
+        return nvec > 4    ? rows(Int<4>{}, Int<2>{})
+               : nvec > 2  ? rows(Int<2>{}, Int<2>{})
+               : nvec == 2 ? rows(Int<1>{}, Int<2>{})
+                           : rows(Int<1>{}, Int<1>{});
     if (nvec <= 32)
-        return rows_in_registers<Tag, Checked, 8, 4>(sbuf, mt, ybase, row_bytes, nvec, causal, first, lane, bd);
+        return nvec > 24   ? rows(Int<8>{}, Int<4>{})
+               : nvec > 16 ? rows(Int<8>{}, Int<3>{})
+                           : rows(Int<8>{}, Int<2>{});
     if (nvec <= 64)
-        return rows_in_registers<Tag, Checked, 16, 4>(sbuf, mt, ybase, row_bytes, nvec, causal, first, lane, bd);
-    return rows_in_registers<Tag, Checked, 32, 4>(sbuf, mt, ybase, row_bytes, nvec, causal, first, lane, bd);
+        return nvec > 48 ? rows(Int<16>{}, Int<4>{}) : rows(Int<16>{}, Int<3>{});
+    return nvec > 96 ? rows(Int<32>{}, Int<4>{}) : rows(Int<32>{}, Int<3>{});
 }
 
 // -------------------------------------------------------------- the schedule
