@@ -706,58 +706,41 @@ __device__ __forceinline__ bool row_team(const unsigned char *srow, unsigned cha
     return true;
 }
 
+template <int N> struct Int {
+    static constexpr int value = N;
+};
+
 // ------------------------------------------------ backward row routines
 // dx = y * (dy - <y, dy>) of one row; y and dy sit in the two halves of the
-// stage.  The dot product: per vector a balanced tree of y*dy, per lane in
-// vector order, then the butterfly over the lane group.
+// stage.
 
-template <typename Tag, bool Checked, int T, int V>
-__device__ __forceinline__ void row_bwd_registers(const unsigned char *sy, const unsigned char *sdy,
-                                                  unsigned char *dxrow, int nvec, int l, bool valid,
-                                                  const Bounds &by, const Bounds &bdy)
+// The products of one vector of y and of dy, added to a running pair (as a
+// tree first: the running sum is rounded once a vector).
+template <typename Tag> __device__ __forceinline__ Pair add_products(Pair acc, uint4 a, uint4 b)
 {
-    using E = Elem<Tag>;
-    constexpr int EPV = E::kPerVec;
-    float yv[V][EPV], dv[V][EPV];
-    float dot = 0.0f;
+    Pair t = pair_fma(vec_pair<Tag>(a, 1), vec_pair<Tag>(b, 1), pair_mul(vec_pair<Tag>(a, 0), vec_pair<Tag>(b, 0)));
+    if constexpr (Elem<Tag>::kPerVec == 8)
+        t = pair_add(t, pair_fma(vec_pair<Tag>(a, 3), vec_pair<Tag>(b, 3),
+                                 pair_mul(vec_pair<Tag>(a, 2), vec_pair<Tag>(b, 2))));
+    return pair_add(acc, t);
+}
+
+// y * (dy - dot) of one vector (nd = -dot, twice).
+template <typename Tag> __device__ __forceinline__ uint4 vec_dx(uint4 a, uint4 b, Pair nd)
+{
+    constexpr int N = Elem<Tag>::kPerVec / 2;
+    float2 o[N];
 #pragma unroll
-    for (int j = 0; j < V; ++j) {
-        const int vi = j * T + l;
-        uint4 ry, rd;
-        if (valid && vi < nvec && load_vec<Checked>(sy + 16 * vi, by, ry) &&
-            load_vec<Checked>(sdy + 16 * vi, bdy, rd)) {
-            E::unpack(ry, yv[j]);
-            E::unpack(rd, dv[j]);
-            float pr[EPV];
-#pragma unroll
-            for (int e = 0; e < EPV; ++e)
-                pr[e] = yv[j][e] * dv[j][e];
-            dot += tree_sum<EPV>(pr);
-        } else {
-#pragma unroll
-            for (int e = 0; e < EPV; ++e)
-                yv[j][e] = dv[j][e] = 0.0f;
-        }
-    }
-    dot = group_sum<T>(dot);
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-        const int vi = j * T + l;
-        if (valid && vi < nvec) {
-#pragma unroll
-            for (int e = 0; e < EPV; ++e)
-                yv[j][e] = yv[j][e] * (dv[j][e] - dot);
-            store_vec<Checked>(dxrow + 16 * vi, by, E::pack(yv[j]));
-        }
-    }
+    for (int k = 0; k < N; ++k)
+        o[k] = halves(pair_mul(vec_pair<Tag>(a, k), pair_add(vec_pair<Tag>(b, k), nd)));
+    return pack_pairs<Tag>(o);
 }
 
 // A longer row, shared by a team of W warps as in row_team: the vectors wi*32
 // + l, + 32 W, ... of y and of dy, four of each in registers (the last two can
 // be missing in some lanes; the whole row up to W * 2 KiB), further ones (rows
 // of 32 to 56 KiB on 16 warps, of 2 to 3 KiB on one) read again from the
-// stage.  The warps' dot
-// products are exchanged once and added in a fixed tree.
+// stage.  The warps' dot products are exchanged once and added in a fixed tree.
 constexpr int kTeamVecsBwd = 4;
 
 template <typename Tag, bool Checked, int W, int Full, typename Exchange, typename Release>
@@ -765,7 +748,7 @@ __device__ __forceinline__ bool row_team_bwd(const unsigned char *sy, const unsi
                                              int nvec, int wi, int lane, const Bounds &by, const Bounds &bdy,
                                              Exchange &&exchange, Release &&release)
 {
-    constexpr int V = kTeamVecsBwd, N = Elem<Tag>::kPerVec / 2, step = W * 32;
+    constexpr int V = kTeamVecsBwd, step = W * 32;
     const int t0 = wi * 32 + lane;
     const bool tail = (W == 1 || W == 16) && nvec > V * step;
     auto fetch = [&](const unsigned char *src, int vi, bool in, const Bounds &b) -> uint4 {
@@ -776,14 +759,6 @@ __device__ __forceinline__ bool row_team_bwd(const unsigned char *sy, const unsi
                 r = u;
         }
         return r;
-    };
-    // (a vector's products first, as a tree: the running sum is rounded once a vector)
-    auto add = [&](Pair acc, uint4 a, uint4 b) -> Pair {
-        Pair t = pair_fma(vec_pair<Tag>(a, 1), vec_pair<Tag>(b, 1), pair_mul(vec_pair<Tag>(a, 0), vec_pair<Tag>(b, 0)));
-        if constexpr (N == 4)
-            t = pair_add(t, pair_fma(vec_pair<Tag>(a, 3), vec_pair<Tag>(b, 3),
-                                     pair_mul(vec_pair<Tag>(a, 2), vec_pair<Tag>(b, 2))));
-        return pair_add(acc, t);
     };
     uint4 yv[V], dv[V];
 #pragma unroll
@@ -796,12 +771,12 @@ __device__ __forceinline__ bool row_team_bwd(const unsigned char *sy, const unsi
     Pair acc = pair(0.0f, 0.0f), acc2 = acc;
 #pragma unroll
     for (int j = 0; j < V; j += 2) {
-        acc = add(acc, yv[j], dv[j]);
-        acc2 = add(acc2, yv[j + 1], dv[j + 1]);
+        acc = add_products<Tag>(acc, yv[j], dv[j]);
+        acc2 = add_products<Tag>(acc2, yv[j + 1], dv[j + 1]);
     }
     if (tail) {
         for (int vi = t0 + V * step; vi < nvec; vi += step)
-            acc = add(acc, fetch(sy, vi, true, by), fetch(sdy, vi, true, bdy));
+            acc = add_products<Tag>(acc, fetch(sy, vi, true, by), fetch(sdy, vi, true, bdy));
     } else {
         release();
     }
@@ -810,13 +785,6 @@ __device__ __forceinline__ bool row_team_bwd(const unsigned char *sy, const unsi
     if (!exchange(dot))
         return false;
     const Pair nd = pair(-dot, -dot);
-    auto dx = [&](uint4 a, uint4 b) -> uint4 {
-        float2 o[N];
-#pragma unroll
-        for (int k = 0; k < N; ++k)
-            o[k] = halves(pair_mul(vec_pair<Tag>(a, k), pair_add(vec_pair<Tag>(b, k), nd)));
-        return pack_pairs<Tag>(o);
-    };
     // (unpacked again for the write, as in row_team)
 #pragma unroll
     for (int j = 0; j < V; ++j) {
@@ -827,29 +795,65 @@ __device__ __forceinline__ bool row_team_bwd(const unsigned char *sy, const unsi
     for (int j = 0; j < V; ++j) {
         const int vi = t0 + j * step;
         if (j < Full || vi < nvec)
-            store_vec<Checked>(dxrow + 16 * vi, by, dx(yv[j], dv[j]));
+            store_vec<Checked>(dxrow + 16 * vi, by, vec_dx<Tag>(yv[j], dv[j], nd));
     }
     if (tail) {
         for (int vi = t0 + V * step; vi < nvec; vi += step)
-            store_vec<Checked>(dxrow + 16 * vi, by, dx(fetch(sy, vi, true, by), fetch(sdy, vi, true, bdy)));
+            store_vec<Checked>(dxrow + 16 * vi, by, vec_dx<Tag>(fetch(sy, vi, true, by), fetch(sdy, vi, true, bdy), nd));
         release();
     }
     return true;
 }
 
-// Backward rows of a stage, dealt like consume_stage's: groups of G = 32/T
-// rows round robin over the consumer warps from warp `first`.
+// Backward rows that one lane group's registers hold, as rows_in_lanes: T
+// lanes, V vectors of y and of dy a lane, of which only the last can be
+// missing (0: it adds nothing), no other bound.  More than 16 vectors take
+// 16 or 32 lanes of two: four of each a lane spill.  GB/s over 512 MiB of y and
+// dy, 8 to 32 lanes with a bound on every vector -> this routine: bf16 16 B
+// 1845 -> 7092, 32 B 3492 -> 7053, 64 B 6195 -> 7105, 528 B 6833 -> 7054, longer
+// ones as before (7.0 to 7.1 TB/s); fp32 16 B 2523 -> 7077, 32 B 4680 -> 7050,
+// 48 B 6280 -> 7082.
 template <typename Tag, bool Checked, int T, int V>
-__device__ __forceinline__ int rows_bwd_registers(const unsigned char *sbuf, int half, const StageMeta &mt,
-                                                  unsigned char *ybase, int row_bytes, int nvec, int first,
-                                                  int lane, const Bounds &by, const Bounds &bdy)
+__device__ __forceinline__ int rows_bwd_in_lanes(const unsigned char *sbuf, int half, const StageMeta &mt,
+                                                 unsigned char *ybase, int row_bytes, int nvec, int first,
+                                                 int lane, const Bounds &by, const Bounds &bdy)
 {
     constexpr int G = 32 / T;
     const int g = lane / T, l = lane % T;
+    const bool in_last = (V - 1) * T + l < nvec;
     for (int rb = first * G; rb < mt.nrows; rb += G * kConsumerWarps) {
         const int r = rb + g;
-        row_bwd_registers<Tag, Checked, T, V>(sbuf + (size_t)r * row_bytes, sbuf + half + (size_t)r * row_bytes,
-                                              ybase + (size_t)r * row_bytes, nvec, l, r < mt.nrows, by, bdy);
+        const bool valid = r < mt.nrows;
+        const unsigned char *sy = sbuf + (size_t)(valid ? r : mt.nrows - 1) * row_bytes + 16 * l;
+        uint4 yv[V], dv[V];
+        Pair acc = pair(0.0f, 0.0f);
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            yv[j] = dv[j] = make_uint4(0u, 0u, 0u, 0u);
+            uint4 a, b;
+            if ((j < V - 1 || in_last) && load_vec<Checked>(sy + 16 * j * T, by, a) &&
+                load_vec<Checked>(sy + half + 16 * j * T, bdy, b)) {
+                yv[j] = a;
+                dv[j] = b;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+            acc = add_products<Tag>(acc, yv[j], dv[j]);
+        const float2 a2 = halves(acc);
+        const float dot = group_sum<T>(a2.x + a2.y);
+        const Pair nd = pair(-dot, -dot);
+        // (unpacked again for the write, as in row_team)
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            asm volatile("" : "+r"(yv[j].x), "+r"(yv[j].y), "+r"(yv[j].z), "+r"(yv[j].w));
+            asm volatile("" : "+r"(dv[j].x), "+r"(dv[j].y), "+r"(dv[j].z), "+r"(dv[j].w));
+        }
+        unsigned char *dx = ybase + (size_t)r * row_bytes + 16 * l;
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+            if (valid && (j < V - 1 || in_last))
+                store_vec<Checked>(dx + 16 * j * T, by, vec_dx<Tag>(yv[j], dv[j], nd));
     }
     return (mt.nrows + G - 1) / G;
 }
@@ -867,21 +871,20 @@ __device__ __forceinline__ int consume_stage_bwd(const unsigned char *sbuf, int 
     Bounds bdy = by;
     bdy.s_lo = sbuf + half;
     bdy.s_hi = sbuf + half + (size_t)mt.nrows * row_bytes;
-    constexpr int VMAX = 16 / E::kPerVec;   // y and dy: at most 32 floats per lane
+    auto rows = [&](auto t, auto v) {
+        return rows_bwd_in_lanes<Tag, Checked, decltype(t)::value, decltype(v)::value>(
+            sbuf, half, mt, ybase, row_bytes, nvec, first, lane, by, bdy);
+    };
     if (nvec <= 8)
-        return rows_bwd_registers<Tag, Checked, 8, 1>(sbuf, half, mt, ybase, row_bytes, nvec, first, lane, by,
-                                                      bdy);
-    if (nvec <= 16)
-        return rows_bwd_registers<Tag, Checked, 8, 2>(sbuf, half, mt, ybase, row_bytes, nvec, first, lane, by,
-                                                      bdy);
+        return nvec > 4    ? rows(Int<4>{}, Int<2>{})
+               : nvec > 2  ? rows(Int<2>{}, Int<2>{})
+               : nvec == 2 ? rows(Int<1>{}, Int<2>{})
+                           : rows(Int<1>{}, Int<1>{});
     if (nvec <= 32)
-        return rows_bwd_registers<Tag, Checked, 16, 2>(sbuf, half, mt, ybase, row_bytes, nvec, first, lane, by,
-                                                       bdy);
-    if (VMAX == 2 || nvec <= 64)
-        return rows_bwd_registers<Tag, Checked, 32, 2>(sbuf, half, mt, ybase, row_bytes, nvec, first, lane, by,
-                                                       bdy);
-    // fp32 (bf16 rows of more than 64 vectors go to teams)
-    return rows_bwd_registers<Tag, Checked, 32, VMAX>(sbuf, half, mt, ybase, row_bytes, nvec, first, lane, by, bdy);
+        return nvec > 16 ? rows(Int<16>{}, Int<2>{}) : rows(Int<8>{}, Int<2>{});
+    if (E::kSize == 2 || nvec <= 64)   // (bf16 rows of more than 64 vectors go to teams)
+        return rows(Int<32>{}, Int<2>{});
+    return nvec > 96 ? rows(Int<32>{}, Int<4>{}) : rows(Int<32>{}, Int<3>{});
 }
 
 // ------------------------------------------------------------ long rows
@@ -990,10 +993,6 @@ __device__ __forceinline__ void long_chunk_bwd(const unsigned char *sbuf, int ha
         }
     }
 }
-
-template <int N> struct Int {
-    static constexpr int value = N;
-};
 
 // Warps that share a row: the fewest whose registers hold it.
 __device__ __forceinline__ int team_warps(int nvec)

@@ -1,7 +1,7 @@
 """Rows that one lane group's registers hold (every class and its edges, 16
 bytes to 2 KiB), against the oracle and bit-identical across policies, whose
 patches end such rows at different places; causal, non-finite and lowest-value
-rows."""
+rows, and the backward pass."""
 import pytest
 
 from gpu_util import bits, check_all_against_oracle, run, to_device, to_host
@@ -67,3 +67,25 @@ def test_non_finite_and_lowest_value_rows(nvec, dtype):
     ref = torch.softmax(x[[0, 6]].double(), -1)
     err = (y[[0, 6]].double() - ref).abs()
     assert float(err.max()) <= 2e-6 if dtype == "f32" else bool((err <= ref * 2.0 ** -8 + 1e-30).all())
+
+
+@pytest.mark.parametrize("nvec", NVEC)
+@pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
+def test_backward_row_lengths_of_every_class(nvec, dtype):
+    import torch
+    from test_backward_gpu import _check, _inputs
+    C = nvec * (4 if dtype == workload.F32 else 8)
+    w = workload.uniform("lanes bwd", dtype, 7, 333, C, 2.0, 0x1B0 + nvec).materialize()
+    y, dy = _inputs(w)
+    yd, dyd = to_device(y), to_device(dy)
+    outs = []
+    for p in POLICIES:
+        dx = torch.full_like(yd, float("nan"))
+        bsm.bsm_softmax_backward(yd, dyd, dx, w.nslices, 333, C, dtype, p)
+        outs.append(dx)
+    bsm.bsm_softmax_backward(yd, dyd, dyd, w.nslices, 333, C, dtype, bsm.POLICY_DYNAMIC)   # in place
+    torch.cuda.synchronize()
+    assert bsm.bsm_device_status() == 0
+    for dx in outs[1:] + [dyd]:
+        assert torch.equal(bits(dx), bits(outs[0]))
+    _check(w, y, dy, to_host(outs[0]))
