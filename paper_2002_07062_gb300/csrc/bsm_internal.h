@@ -68,12 +68,12 @@ enum Op : int32_t {
 // warps, in a kernel instance of its own so that the routines of shorter rows
 // do not pay its registers.  One warp per row with three sweeps over shared
 // memory (before) against teams, GB/s over 256 MiB of rows: bf16 4 KiB 5885 ->
-// 6800, 16 KiB 4880 -> 6720, 64 KiB 1970 -> 6700, 113 KiB 1413 -> 6480; fp32
-// 16 KiB 6450 -> 6690, 64 KiB 3050 -> 6750, 113 KiB 2245 -> 6560.  What
+// 6820, 16 KiB 4880 -> 6745, 64 KiB 1970 -> 6430, 113 KiB 1413 -> 6450; fp32
+// 16 KiB 6450 -> 6820, 64 KiB 3050 -> 6770, 113 KiB 2245 -> 6575.  What
 // bounded the old routines: a stage of one 64 KiB row left 3 of 16 warps
 // busy, each on a serial chain of shared loads.
 constexpr int kLaneRowBytes = 2048;
-// The backward pass's (y and dy as at most 32 floats a lane).  One
+// The backward pass's (at most four vectors of each of y and dy a lane).  One
 // warp a row (two sweeps over shared memory) against teams, 512 MiB of y and
 // dy: bf16 16 KiB rows 6550 -> 7055 GB/s, 32 KiB 4640 -> 7050, 56 KiB 3380 ->
 // 6900; fp32 24 KiB 6680 -> 7050, 48 KiB 6370 -> 7000.
@@ -83,9 +83,9 @@ template <int ElemSize> constexpr int kLaneRowBytesBwd = ElemSize == 4 ? 2048 : 
 // [g*K, g*K + K); its rank-0 CTA claims rows and announces them in the
 // group's ring of kGroupRing claim words (row sequence number + 1 in the high
 // half, the row's position in the table in the low half); each member stages
-// its part of the row and publishes its (max, sum) in one of kGroupSlots
+// its part of the row and publishes its (offset, sum) in one of kGroupSlots
 // exchange slots as two words (the row sequence number + 1 in the high half
-// of each, max or sum in the low half).  Rings and exchange words are reset
+// of each, offset or sum in the low half).  Rings and exchange words are reset
 // by the last CTA of every launch.
 constexpr int kGroupRing = 16;
 constexpr int kGroupSlots = 4;
