@@ -829,19 +829,33 @@ def sweep(args, bsm, workload, stream):
     bmm_sweep(bsm, workload, stream)
 
 
-def _moved_factor(st, op="forward"):
-    """Bytes a plan moves per algorithmic byte: rows split over groups of CTAs
-    and rows staged whole read x once; rows streamed twice read it again
-    (forward: 1.5, backward: 5/3 of the algorithmic bytes at most)."""
-    if st["group_rows"] and st["group_rows"] == st["long_items"]:
+# Rows of up to this many bytes (16 parts of two stages; backward: of y and dy)
+# that fill the SMs run over clusters of CTAs.
+CLUSTER_ROW_BYTES = {"forward": 16 * 112 * 1024, "backward": 16 * 56 * 1024}
+
+
+def _long_kernel(st, row_bytes, op="forward"):
+    """The kernel a plan of rows longer than a stage runs on."""
+    if st["group_rows"]:
+        return "softmax_group"
+    if st["launches"] == 1 and row_bytes <= CLUSTER_ROW_BYTES[op]:
+        return "softmax_cluster"
+    return "softmax_persistent (long rows)"
+
+
+def _moved_factor(st, row_bytes, op="forward"):
+    """Bytes a plan moves per algorithmic byte: rows split over groups or
+    clusters of CTAs read x once; rows streamed twice read it again (forward:
+    1.5, backward: 5/3 of the algorithmic bytes at most)."""
+    if _long_kernel(st, row_bytes, op) != "softmax_persistent (long rows)":
         return 1.0
     return 1.5 if op == "forward" else 5 / 3
 
 
 def long_row_sweep(bsm, workload, stream):
     """Rows longer than a shared-memory stage: GB/s of algorithmic traffic,
-    forward (rows split over groups of CTAs, or streamed twice) and backward
-    (streamed twice)."""
+    forward and backward (over clusters or groups of CTAs, or streamed
+    twice)."""
     import torch
     for dtype, name in ((workload.F32, "fp32"), (workload.BF16, "bf16")):
         tdt = torch.float32 if dtype == workload.F32 else torch.bfloat16
@@ -866,9 +880,12 @@ def long_row_sweep(bsm, workload, stream):
                               "policy": "dynamic", "ms": round(med, 4),
                               "GBps": round(alg / (med * 1e-3) / 1e9, 2),
                               "group_k": st["group_k"], "launches": st["launches"],
-                              "moved_GBps": round(_moved_factor(st) * alg / (med * 1e-3) / 1e9, 2)}),
+                              "moved_GBps": round(_moved_factor(st, C * es) * alg / (med * 1e-3) / 1e9, 2)}),
                   flush=True)
             dy = torch.randn(R * C, device="cuda").to(tdt)
+            plan = bsm.bsm_plan_create(y, x, [R], [C], dtype, bsm.POLICY_DYNAMIC, op=bsm.OP_BACKWARD, x2=dy)
+            st = plan.stats()
+            plan.close()
 
             def bstep():
                 bsm.bsm_softmax_backward(y, dy, x, 1, R, C, dtype, bsm.POLICY_DYNAMIC, stream)
@@ -881,7 +898,8 @@ def long_row_sweep(bsm, workload, stream):
                               "%s %d rows x %d (%d KiB rows)" % (name, R, C, C * es >> 10),
                               "policy": "dynamic", "ms": round(med, 4),
                               "GBps": round(alg / (med * 1e-3) / 1e9, 2),
-                              "moved_GBps": round(5 / 3 * alg / (med * 1e-3) / 1e9, 2)}), flush=True)
+                              "moved_GBps": round(_moved_factor(st, C * es, "backward") * alg / (med * 1e-3) / 1e9,
+                                                  2)}), flush=True)
             del x, y, dy
             torch.cuda.empty_cache()
 
@@ -917,7 +935,7 @@ def time_long_rows(bsm, C, dtype, stream, dev, target_s=0.5):
     peak, peak_src = measured_peak()
     gbs = alg / (ms * 1e-3) / 1e9
     plan.close()
-    kernel = "softmax_group" if st["group_rows"] else "softmax_persistent (long rows)"
+    kernel = _long_kernel(st, C * es)
     return {"value": round(gbs, 2), "unit": "GB/s", "ms_per_step": round(ms, 5), "steps": steps,
             "dtype": "f32" if dtype == workload.F32 else "bf16",
             "config": {"workload": "%s %d rows x %d (%d KiB rows), 256 MiB, random normal"
@@ -934,7 +952,7 @@ def time_long_rows(bsm, C, dtype, stream, dev, target_s=0.5):
                          if st["launches"] == 1 else None,
                          "peak_source": peak_src,
                          "kernel": kernel, "launch_ms": round(ms / max(1, st["launches"]), 5),
-                         "moved_bytes_per_step": int(_moved_factor(st) * alg)},
+                         "moved_bytes_per_step": int(_moved_factor(st, C * es) * alg)},
             "clocks": clk.summary(), "device_status": bsm.bsm_device_status()}
 
 
@@ -1033,7 +1051,7 @@ def run_long_rows(args, bsm, ws, rank, dev):
            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
            "data": "synthetic", "config": {"workload": "fp32 %d rows x %d" % (R, C),
                                            "policy": "dynamic", "bytes_per_step": alg},
-           "moved_GBps": round(_moved_factor(st) * alg / (ms * 1e-3) / 1e9, 2),
+           "moved_GBps": round(_moved_factor(st, 4 * C) * alg / (ms * 1e-3) / 1e9, 2),
            "gpu_launches": int(st["launches"]) * args.steps,
            "plan": {k: st[k] for k in ("n_items", "long_items", "launches", "stage_bytes", "n_stages",
                                        "group_rows", "group_k", "n_groups")},

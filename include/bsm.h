@@ -56,21 +56,20 @@
  *     Batches of longer rows, at least two per SM, run over clusters of 2, 4, 8
  *     or 16 SMs: each takes a part of the row in one of its stages and every
  *     element is read once (rows of up to 1.7 MiB, 880 KiB backward).  Other
- *     longer rows go through the stages in chunks, in two passes -- a running maximum
- *     and rescaled sum (backward: the dot product), then the output -- and are
- *     read again, all but their last chunk (a row of two chunks whose halves
- *     fit three stages stays staged).  When a batch has fewer such rows than
- *     two per SM, each is cut into segments spread over the SMs and the execute
- *     takes two launches (segment partials, then combine and write); otherwise
- *     each row stays on one SM within one launch.  Forward rows of 5 to 32
- *     parts of at most 64 KiB, enough of them to fill two thirds of the groups'
- *     waves, are instead split over groups of K CTAs (K = ceil(row / 64
+ *     longer rows go through the stages in chunks, in two passes -- a running
+ *     maximum and rescaled sum (backward: the dot product), then the output --
+ *     and are read again, all but their last chunk (a row of two chunks whose
+ *     halves fit three stages stays staged).  When a batch has fewer such rows
+ *     than two per SM, each is cut into segments spread over the SMs and the
+ *     execute takes two launches (segment partials, then combine and write);
+ *     otherwise each row stays on one SM within one launch.  Forward rows of 5
+ *     to 32 parts of at most 64 KiB, enough of them to fill two thirds of the
+ *     groups' waves, are instead split over groups of K CTAs (K = ceil(row / 64
  *     KiB); n_sm / K groups) in one cooperative launch -- each CTA stages one
  *     part, the group exchanges (offset, sum) partials through global memory
  *     and every element is read once -- or over clusters where those are
- *     faster.  Which path a row takes depends on the
- *     rows of the batch and the device, never on the policy: every policy
- *     gives the same bits.
+ *     faster.  Which path a row takes depends on the rows of the batch and the
+ *     device, never on the policy: every policy gives the same bits.
  */
 #ifndef BSM_H
 #define BSM_H

@@ -325,7 +325,10 @@ int choose_groups(const std::vector<SliceView> &slices, int es, int n_sm, int64_
     // the vectors each of its threads holds (kGroupVecs at the cap), so the
     // fewest members with full parts move the most bytes per exchange, even
     // when n_sm / K groups leave SMs idle.  Measured on GB300 (256 MiB of
-    // rows, GB/s): fp32 1 MiB rows K = 16 (9 groups) 4746 against K = 19 (8
+    // rows, GB/s; with the consumer warps reading the exchange words
+    // themselves -- since a warp of its own does, 1 MiB rows take 5472 (fp32)
+    // and 5136 (bf16), and batches that clusters serve better go there, see
+    // choose_clusters): fp32 1 MiB rows K = 16 (9 groups) 4746 against K = 19 (8
     // groups) 4347, 17 and 18 lower still; bf16 1 MiB the same (3952 against
     // 3635); bf16 512 KiB K = 8 4139 against K = 16 2612 and K = 19 2316;
     // fp32 2 MiB K = 32 4336 against K = 38 3748.  Against the paths that

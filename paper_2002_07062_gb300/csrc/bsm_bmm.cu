@@ -22,9 +22,9 @@
 // The accumulators are double-buffered so the epilogue of a tile overlaps the
 // MMAs of the next.  Warps 0 and 1 run their loops as a whole, the copies and
 // MMAs under an election (see elect_one).  Products bound by the tensor cores
-// run on pairs of CTAs instead (bmm_pair, below).  Every wait is bounded (2 s of %globaltimer): on expiry
-// the CTA records BSM_DEV_TIMEOUT and leaves; the tensor memory is always
-// deallocated before the CTA exits.
+// run on pairs of CTAs instead (bmm_pair, below).  Every wait is bounded (2 s
+// of %globaltimer): on expiry the CTA records BSM_DEV_TIMEOUT and leaves; the
+// tensor memory is always deallocated before the CTA exits.
 
 #include <cuda.h>
 #include <cuda_runtime.h>
