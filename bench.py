@@ -835,9 +835,11 @@ CLUSTER_ROW_BYTES = {"forward": 16 * 112 * 1024, "backward": 16 * 56 * 1024}
 
 
 def _long_kernel(st, row_bytes, op="forward"):
-    """The kernel a plan of rows longer than a stage runs on."""
+    """The kernel a plan of rows longer than a stage runs on (rows that
+    qualify for groups go to clusters where those are faster; the statistics
+    count them as group rows all the same)."""
     if st["group_rows"]:
-        return "softmax_group"
+        return "softmax_group or softmax_cluster"
     if st["launches"] == 1 and row_bytes <= CLUSTER_ROW_BYTES[op]:
         return "softmax_cluster"
     return "softmax_persistent (long rows)"

@@ -342,7 +342,7 @@ typedef struct {
     int64_t map_chunk_bytes;    /* granularity of the address->die map used */
     double plan_ms;             /* host time spent in bsm_plan_create */
     int64_t long_items;         /* rows longer than a stage (group rows included) */
-    int64_t group_rows;         /* rows split over groups of CTAs (one cooperative launch) */
+    int64_t group_rows;         /* rows split over groups of CTAs (or clusters, where faster) */
     int32_t group_k;            /* CTAs per group */
     int32_t n_groups;           /* groups of that launch */
 } bsm_plan_stats;
