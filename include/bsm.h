@@ -453,12 +453,18 @@ int bsm_plan_device_table(const bsm_plan *plan, int phase, bsm_patch *out, int64
  *                             past the regular table's address the table of rows
  *                             split over groups of CTAs (every member of the
  *                             group skips such a row alike).
+ *   BSM_DEBUG_LAG_WARP        (arg 0) in later self-checking executes of rows split
+ *                             over groups of CTAs, one warp of each CTA waits 50 us
+ *                             per row before it reads the previous row's result;
+ *                             the outputs stay the same.
  *   BSM_DEBUG_NONE            restore the normal wait limit and switch the
- *                             withheld stage off (a corrupted entry stays).
+ *                             withheld stage and the late warp off (a corrupted
+ *                             entry stays).
  * Synchronous.  Returns BSM_ERR_INVALID_ARG for an unknown `what` or arg. */
 #define BSM_DEBUG_NONE 0
 #define BSM_DEBUG_WITHHOLD_STAGE 1
 #define BSM_DEBUG_CORRUPT_PATCH 2
+#define BSM_DEBUG_LAG_WARP 3
 int bsm_plan_debug(bsm_plan *plan, int what, int64_t arg);
 
 /* Drop every cached plan of bsm_softmax / bsm_softmax_ex / bsm_softmax_ragged. */

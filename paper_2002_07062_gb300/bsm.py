@@ -499,7 +499,7 @@ def bsm_addr_group_map(ptr, nbytes: int, chunk: int, sm_group, device: int = -1)
     return out
 
 
-DEBUG_NONE, DEBUG_WITHHOLD_STAGE, DEBUG_CORRUPT_PATCH = 0, 1, 2
+DEBUG_NONE, DEBUG_WITHHOLD_STAGE, DEBUG_CORRUPT_PATCH, DEBUG_LAG_WARP = 0, 1, 2, 3
 
 
 def bsm_plan_debug(plan, what: int, arg: int = 0):

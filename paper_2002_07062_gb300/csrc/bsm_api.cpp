@@ -1480,6 +1480,11 @@ int bsm_plan_debug(bsm_plan *plan, int what, int64_t arg)
         plan->argsg.debug |= KDEBUG_WITHHOLD_STAGE0;
         plan->argsg.wait_limit_ns = static_cast<uint64_t>(arg);
         return BSM_OK;
+    case BSM_DEBUG_LAG_WARP:
+        if (arg != 0)
+            return BSM_ERR_INVALID_ARG;
+        plan->argsg.debug |= KDEBUG_LAG_WARP;
+        return BSM_OK;
     case BSM_DEBUG_CORRUPT_PATCH: {
         // slots of the regular table first, then those of the group rows
         if (arg < 0 || arg >= int64_t(plan->args.n_items) + plan->n_group)

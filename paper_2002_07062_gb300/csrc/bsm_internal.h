@@ -146,6 +146,7 @@ struct KernelArgs {
 
 // Test-only fault injection (bsm_plan_debug).
 constexpr uint32_t KDEBUG_WITHHOLD_STAGE0 = 1u;   // producer never fills stage 0 of its first round
+constexpr uint32_t KDEBUG_LAG_WARP = 2u;          // rows over groups, self-checking: one warp reads results late
 
 // One output tile of the batched matrix product: rows [m0, m0 + 128) (256 on
 // pairs of CTAs) and columns [n0, n0 + BN) of slice `slice`.

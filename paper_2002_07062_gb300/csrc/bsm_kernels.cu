@@ -74,8 +74,8 @@ struct SmemHeader {
     union {
         uint64_t team[kTeamBars];   // rows shared by a team of warps: its partials are in
         struct {                    // rows over groups:
-            uint64_t xres;          // a row's result is in
-            float2 result[2];       // ... its (offset, sum), two rows deep
+            uint64_t xres[2];       // a row's result is in, by row parity
+            float2 result[2];       // ... its (offset, sum)
             uint32_t xarrive[2];    // warps whose partial is in, by row parity
             uint32_t xleft;         // consumer warps that have left
         };
@@ -2051,7 +2051,8 @@ __global__ void __launch_bounds__(kGroupThreads, 1) softmax_group(const KernelAr
             mbar_init(&h.full[s], 1);
             mbar_init(&h.empty[s], kConsumerWarps);
         }
-        mbar_init(&h.xres, 1);
+        mbar_init(&h.xres[0], 1);
+        mbar_init(&h.xres[1], 1);
         h.xarrive[0] = h.xarrive[1] = h.xleft = 0u;
         h.abort_flag = 0;
         mbar_init_fence();
@@ -2195,7 +2196,10 @@ __global__ void __launch_bounds__(kGroupThreads, 1) softmax_group(const KernelAr
         // For every row: the group's words read until all are in, combined,
         // and handed to the consumers through shared memory.  One warp a CTA
         // polls (16 polling the same few lines held the stores up), and the
-        // consumers never wait on global memory.
+        // consumers never wait on global memory.  Barrier and result alternate
+        // by row: row t + 1's result can be in before a consumer warp has
+        // tested row t's (all partials of t + 1 are out by then, that warp's
+        // too), row t + 2's cannot (that warp's partial follows its test).
         uint64_t t0 = 0;
         uint32_t xt = 0;
         for (uint32_t tries = 0; tries < (1u << 30); ++tries) {
@@ -2214,7 +2218,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1) softmax_group(const KernelAr
                 pw = combine_lanes(pw);
                 if (lane == 0) {
                     h.result[xt & 1] = pw;
-                    mbar_arrive(&h.xres);
+                    mbar_arrive(&h.xres[xt & 1]);
                 }
                 __syncwarp();
                 ++xt;
@@ -2251,7 +2255,8 @@ __global__ void __launch_bounds__(kGroupThreads, 1) softmax_group(const KernelAr
         // the row held in rr, once its group's result is in; false when that wait gave up
         auto finish = [&]() -> bool {
             const uint32_t par = (xt - 1) & 1u;
-            if (!__all_sync(0xFFFFFFFFu, mbar_spin_bounded(&h.xres, par, &h.abort_flag, wait_limit))) {
+            if (!__all_sync(0xFFFFFFFFu,
+                            mbar_spin_bounded(&h.xres[par], ((xt - 1) >> 1) & 1u, &h.abort_flag, wait_limit))) {
                 if (lane == 0) {
                     atomicOr(a.status, BSM_DEV_TIMEOUT);
                     h.abort_flag = 1;
@@ -2348,6 +2353,9 @@ __global__ void __launch_bounds__(kGroupThreads, 1) softmax_group(const KernelAr
                                  tag | __float_as_uint(pw.x), tag | __float_as_uint(pw.y));
                     }
                 }
+                if (Checked && (a.debug & KDEBUG_LAG_WARP) && warp == 5)
+                    for (int i = 0; i < 50; ++i)     // test hook: the row before's result is read late
+                        __nanosleep(1000);
                 if (held && !finish()) {
                     held = false;
                     break;

@@ -231,3 +231,27 @@ def test_corrupted_group_row_is_skipped_by_every_member():
     assert np.max(np.abs(yh[ok].astype(np.float64) - y64.reshape(-1, C)[ok])) <= 2e-6
     p.close()
     bsm.bsm_device_status_clear()
+
+
+def test_group_rows_with_one_warp_that_reads_results_late():
+    """Each CTA has the next row's partial out, and may have its result in,
+    before its last warp has read the previous row's: nothing is missed and
+    the bits stay the same."""
+    import torch
+    from gpu_util import bits
+    # 1 MiB bf16 rows, five for each of the 9 groups of 16 CTAs on 152 SMs
+    w = workload.uniform("late warp", workload.BF16, 1, 45, 524288, 2.0, 0xFA14).materialize()
+    x = to_device(w.x)
+    y, late = torch.zeros_like(x), torch.zeros_like(x)
+    bsm.bsm_device_status_clear()
+    bsm.bsm_softmax(x, y, 1, 45, 524288, w.dtype, bsm.POLICY_DYNAMIC)
+    p = bsm.bsm_plan_create(x, late, w.rows, w.cols, w.dtype, bsm.POLICY_DYNAMIC)
+    assert p.stats()["group_rows"] == 45
+    bsm.bsm_plan_debug(p, bsm.DEBUG_LAG_WARP)
+    bsm.bsm_set_device_checks(True)
+    p.execute()
+    torch.cuda.synchronize()
+    bsm.bsm_set_device_checks(False)
+    assert bsm.bsm_device_status() == 0
+    assert torch.equal(bits(late), bits(y))
+    p.close()
