@@ -2455,8 +2455,8 @@ __device__ __forceinline__ void cluster_barrier()
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// Wait (without sleeping, bounded) for a phase that other CTAs of the cluster
-// complete.
+// Wait (without sleeping, bounded; `abort` may be null) for a phase that other
+// CTAs of the cluster complete.
 __device__ __forceinline__ bool cluster_spin_bounded(uint64_t *bar, uint32_t parity, const volatile int32_t *abort,
                                                      uint64_t limit_ns)
 {
@@ -2475,7 +2475,7 @@ __device__ __forceinline__ bool cluster_spin_bounded(uint64_t *bar, uint32_t par
         if ((it & 1023u) == 1023u) {
             const uint64_t t = global_timer_ns();
             t0 = t0 ? t0 : t;
-            if (*abort || t - t0 > limit_ns)
+            if ((abort && *abort) || t - t0 > limit_ns)
                 return false;
         }
     }
@@ -2625,7 +2625,7 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_cluster(const KernelArgs 
             post(1);
             int s = 0;
             uint32_t ph = 0;
-            uint32_t n_issued = 0;              // copies: stages issued so far
+            uint32_t issued = 0, issued_phase = 0;      // by stage: a copy issued, its phase
             bool first = true;
             for (uint32_t t = 0; !aborted; ++t) {
                 uint32_t pos = 0;
@@ -2645,6 +2645,8 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_cluster(const KernelArgs 
                 ClusterMeta &mt = h.meta[s];
                 uint64_t *full = &h.full[s];
                 unsigned char *dst = stages + static_cast<size_t>(s) * a.stage_bytes;
+                const uint32_t bit = 1u << s, phase_bit = ph << s;
+                issued &= ~bit;
                 if (++s == S) {
                     s = 0;
                     ph ^= 1u;
@@ -2699,20 +2701,18 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_cluster(const KernelArgs 
                 bulk_load(dst, src, bytes, full);
                 if (Bwd)
                     bulk_load(dst + half, src2, bytes, full);
-                ++n_issued;
+                issued |= bit;
+                issued_phase = (issued_phase & ~bit) | phase_bit;
             }
             if (aborted) {
                 atomicOr(a.status, BSM_DEV_TIMEOUT);
                 h.abort_flag = 1;
-                // the copies in flight land before the CTA may leave (normally
-                // the consumers waited for them): at most the S newest stages
-                for (uint32_t j = 0; j < static_cast<uint32_t>(S) && j < n_issued; ++j) {
-                    s = s == 0 ? S - 1 : s - 1;
-                    if (s == S - 1)
-                        ph ^= 1u;
-                    mbar_wait_bounded(&h.full[s], ph, nullptr, wait_limit);
-                }
             }
+            // every copy issued has landed before the CTA leaves, whoever gave
+            // up (normally they have: the consumers waited for them)
+            for (int j = 0; j < S; ++j)
+                if (issued >> j & 1u)
+                    mbar_wait_bounded(&h.full[j], issued_phase >> j & 1u, nullptr, wait_limit);
             if (rank == 0 && a.mode == PULL_QUEUE) {
                 // the last cluster to finish pulling rewinds the queue heads
                 __threadfence();
@@ -2826,6 +2826,9 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_cluster(const KernelArgs 
         if (!ok && lane == 0) {
             atomicOr(a.status, BSM_DEV_TIMEOUT);
             h.abort_flag = 1;
+            // pairs of the row given up may still be on their way here: they
+            // are in, or a wait limit has passed, before this CTA leaves
+            cluster_spin_bounded(&h.xbar[x & 1u], (x >> 1) & 1u, nullptr, wait_limit);
         }
         __syncwarp();
     }

@@ -146,3 +146,32 @@ def test_backward_withheld_stage_and_corrupted_record():
     ref = yd * (gd - (yd * gd).sum(-1, keepdim=True))
     assert float((dx[keep].double() - ref).abs().max()) < 1e-7
     p.close()
+
+
+@pytest.mark.parametrize("rows,C", [(0, 40000), (64, 262144)])      # clusters of 2, of 16
+def test_forward_withheld_stage(rows, C):
+    """Every wait of every CTA ends, with copies and other CTAs' partials in
+    flight; the next execute is right."""
+    import time
+    import torch
+    R = rows or _rows()
+    w = workload.uniform("cluster fail", workload.F32, 1, R, C, 2.0, 0xC1F).materialize()
+    x = to_device(w.x)
+    y = torch.zeros_like(x)
+    p = bsm.bsm_plan_create(x, y, w.rows, w.cols, w.dtype, bsm.POLICY_DYNAMIC)
+    for _ in range(3):
+        bsm.bsm_plan_debug(p, bsm.DEBUG_WITHHOLD_STAGE, 20_000_000)      # 0.02 s waits
+        t0 = time.time()
+        p.execute()
+        torch.cuda.synchronize()
+        assert time.time() - t0 < 5.0
+        assert bsm.bsm_device_status() & bsm.DEV_TIMEOUT
+        bsm.bsm_plan_debug(p, bsm.DEBUG_NONE)
+        bsm.bsm_device_status_clear()
+        y.fill_(float("nan"))
+        p.execute()
+        torch.cuda.synchronize()
+        assert bsm.bsm_device_status() == 0
+        check_rows_against_oracle(w, to_host(y), sample_rows(w, 16, 1))
+        assert float((y.view(R, C).double().sum(1) - 1).abs().max()) < 1e-5
+    p.close()
