@@ -923,12 +923,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             if (!ok) {
                 atomicOr(a.status, BSM_DEV_TIMEOUT);
                 h.abort_flag = 1;
-                // copies in flight land before the CTA may leave (normally
-                // the MMAs consumed every stage)
-                if (rank == 0)
-                    for (uint32_t j = it > static_cast<uint32_t>(S) ? it - S : 0u; j < it; ++j)
-                        bar_wait(&h.full[j % S], (j / S) & 1u, nullptr);
             }
+            // both CTAs' copies in flight land before either may leave (a
+            // no-op on the normal path, where the MMAs consumed every stage),
+            // whichever role gave up
+            if (rank == 0)
+                for (uint32_t j = it > static_cast<uint32_t>(S) ? it - S : 0u; j < it; ++j)
+                    bar_wait(&h.full[j % S], (j / S) & 1u, nullptr);
             if (rank == 0 && a.mode == PULL_QUEUE) {
                 __threadfence();
                 const uint32_t prev = atomicAdd(&a.heads[BSM_MAX_DIES], 1u);
