@@ -169,3 +169,33 @@ def check_every_element_against_oracle(w: workload.Workload, y_host: np.ndarray,
         worst = max(worst, check_all_against_oracle(sub, ys))
         s0 = s1
     return worst
+
+
+FINITE_MASKS = [-1e9, -1e10, -1e30, None]       # None: the type's lowest value
+
+
+def check_finite_masks(mask, dtype, R, C):
+    """Rows of which all but a few places hold a finite mask value: a head, a
+    tail, a middle piece or alternate elements are left, so that whole warps
+    and whole parts of a row see the mask only.  Against float64."""
+    import torch
+    t = torch.float32 if dtype == workload.F32 else torch.bfloat16
+    mask = torch.finfo(t).min if mask is None else mask
+    g = torch.Generator(device="cuda").manual_seed(R + C)
+    x = torch.randn(R, C, generator=g, device="cuda").to(t)
+    x[1, 8:] = mask
+    x[2, C // 2:] = mask
+    x[3, :C - 5] = mask
+    x[4, C // 3: C // 2] = mask
+    x[5, ::2] = mask
+    x[6, :C // 2] = mask
+    x[6, C // 2 + 8:] = mask
+    y = torch.full_like(x, -1.0)
+    bsm.bsm_softmax(x, y, 1, R, C, dtype, bsm.POLICY_DYNAMIC)
+    torch.cuda.synchronize()
+    assert bsm.bsm_device_status() == 0
+    ref = torch.softmax(x.double(), -1)
+    err = (y.double() - ref).abs()
+    bound = FP32_TOL if dtype == workload.F32 else ref * 2.0 ** -8 + 1e-30
+    wrong = (~(err <= bound)).any(1).nonzero().flatten().tolist()
+    assert not wrong, wrong

@@ -6,7 +6,8 @@ the self-checking kernel, a withheld stage and a corrupted record."""
 import numpy as np
 import pytest
 
-from gpu_util import bits, check_rows_against_oracle, run, sample_rows, to_device, to_host
+from gpu_util import (FINITE_MASKS, bits, check_finite_masks, check_rows_against_oracle, run, sample_rows,
+                      to_device, to_host)
 from paper_2002_07062_gb300 import bsm, workload
 
 pytestmark = pytest.mark.gpu
@@ -115,6 +116,13 @@ def test_non_finite_and_lowest_value_rows(dtype, nvec):
     ref = torch.softmax(x[rest].double(), -1)
     err = (y[rest].double() - ref).abs()
     assert float(err.max()) <= 2e-6 if dtype == "f32" else bool((err <= ref * 2.0 ** -8 + 1e-30).all())
+
+
+@pytest.mark.parametrize("mask", FINITE_MASKS)
+@pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
+@pytest.mark.parametrize("nvec", [9000, 15000, 28845, 70003])       # clusters of 2 and 4, of 4 to 16 or groups
+def test_finite_masks(mask, dtype, nvec):
+    check_finite_masks(mask, dtype, _rows(nvec), nvec * (4 if dtype == workload.F32 else 8))
 
 
 def test_backward_withheld_stage_and_corrupted_record():

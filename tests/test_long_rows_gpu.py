@@ -7,7 +7,8 @@ the backward pass."""
 import numpy as np
 import pytest
 
-from gpu_util import bits, check_all_against_oracle, run, to_device, to_host
+from gpu_util import (FINITE_MASKS, bits, check_all_against_oracle, check_finite_masks, run, to_device,
+                      to_host)
 from paper_2002_07062_gb300 import bsm, workload
 
 pytestmark = pytest.mark.gpu
@@ -226,3 +227,10 @@ def test_non_finite_group_rows():
     assert np.isnan(yh[1]).all() and np.isnan(yh[2]).all() and np.isnan(yh[4]).all()
     assert yh[3, 99999] == 1.0 and np.count_nonzero(yh[3]) == 1
     check_all_against_oracle(w, to_host(y))
+
+
+@pytest.mark.parametrize("mask", FINITE_MASKS)
+@pytest.mark.parametrize("case", [1, 4])
+def test_finite_masks_in_group_rows(mask, case):
+    R, C, dtype, _ = GROUP_CASES[case]
+    check_finite_masks(mask, dtype, R, C)

@@ -6,7 +6,8 @@ stage changes; batches that mix team sizes (and long rows); rows with NaN,
 import numpy as np
 import pytest
 
-from gpu_util import bits, check_all_against_oracle, run, to_device, to_host
+from gpu_util import (FINITE_MASKS, bits, check_all_against_oracle, check_finite_masks, run, to_device,
+                      to_host)
 from paper_2002_07062_gb300 import bsm, workload
 
 pytestmark = pytest.mark.gpu
@@ -100,6 +101,13 @@ def test_non_finite_and_lowest_value_rows(nvec, dtype):
     ref = torch.softmax(x[[0, 6, 7, 8]].double(), -1)
     err = (y[[0, 6, 7, 8]].double() - ref).abs()
     assert float(err.max()) <= 2e-6 if dtype == "f32" else bool((err <= ref * 2.0 ** -8 + 1e-30).all())
+
+
+@pytest.mark.parametrize("mask", FINITE_MASKS)
+@pytest.mark.parametrize("nvec", [100, 300, 1000, 2000, 5000, 7000])
+@pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
+def test_finite_masks(mask, nvec, dtype):
+    check_finite_masks(mask, dtype, 9, nvec * (4 if dtype == workload.F32 else 8))
 
 
 def test_withheld_stage_times_out_on_team_rows():
