@@ -174,10 +174,11 @@ def check_every_element_against_oracle(w: workload.Workload, y_host: np.ndarray,
 FINITE_MASKS = [-1e9, -1e10, -1e30, None]       # None: the type's lowest value
 
 
-def check_finite_masks(mask, dtype, R, C):
+def check_finite_masks(mask, dtype, R, C, short_row=False):
     """Rows of which all but a few places hold a finite mask value: a head, a
     tail, a middle piece or alternate elements are left, so that whole warps
-    and whole parts of a row see the mask only.  Against float64."""
+    and whole parts of a row see the mask only.  Against float64.  short_row
+    adds a slice of one short row, beside which long rows go to one CTA each."""
     import torch
     t = torch.float32 if dtype == workload.F32 else torch.bfloat16
     mask = torch.finfo(t).min if mask is None else mask
@@ -190,8 +191,14 @@ def check_finite_masks(mask, dtype, R, C):
     x[5, ::2] = mask
     x[6, :C // 2] = mask
     x[6, C // 2 + 8:] = mask
-    y = torch.full_like(x, -1.0)
-    bsm.bsm_softmax(x, y, 1, R, C, dtype, bsm.POLICY_DYNAMIC)
+    if short_row:
+        x = torch.cat([x.view(-1), x[0, :64]])
+        y = torch.full_like(x, -1.0)
+        bsm.bsm_softmax_ragged(x, y, [0, R * C], [R, 1], [C, 64], dtype, bsm.POLICY_DYNAMIC)
+        x, y = x[:-64].view(R, C), y[:-64].view(R, C)
+    else:
+        y = torch.full_like(x, -1.0)
+        bsm.bsm_softmax(x, y, 1, R, C, dtype, bsm.POLICY_DYNAMIC)
     torch.cuda.synchronize()
     assert bsm.bsm_device_status() == 0
     ref = torch.softmax(x.double(), -1)

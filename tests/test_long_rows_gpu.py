@@ -234,3 +234,17 @@ def test_non_finite_group_rows():
 def test_finite_masks_in_group_rows(mask, case):
     R, C, dtype, _ = GROUP_CASES[case]
     check_finite_masks(mask, dtype, R, C)
+
+
+@pytest.mark.parametrize("mask", FINITE_MASKS)
+@pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
+@pytest.mark.parametrize("C", [40000, 600000])
+def test_finite_masks_in_rows_cut_into_segments(mask, dtype, C):
+    check_finite_masks(mask, dtype, 8, C * (1 if dtype == workload.F32 else 2))
+
+
+@pytest.mark.parametrize("mask", FINITE_MASKS)
+@pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
+@pytest.mark.parametrize("C", [30000, 60000])          # staged between the passes; streamed twice
+def test_finite_masks_in_rows_streamed_by_one_cta(mask, dtype, C):
+    check_finite_masks(mask, dtype, 310, C * (1 if dtype == workload.F32 else 2), short_row=True)
