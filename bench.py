@@ -829,27 +829,18 @@ def sweep(args, bsm, workload, stream):
     bmm_sweep(bsm, workload, stream)
 
 
-# Rows of up to this many bytes (16 parts of two stages; backward: of y and dy)
-# that fill the SMs run over clusters of CTAs.
-CLUSTER_ROW_BYTES = {"forward": 16 * 112 * 1024, "backward": 16 * 56 * 1024}
+def _long_kernel(bsm, plan):
+    """(kernel, CTAs that share a row) of a plan of rows longer than a stage."""
+    kernel, ctas = bsm.bsm_plan_kernel(plan, 2 if plan.stats()["group_rows"] else 0)
+    return {bsm.KERNEL_GROUP: "softmax_group", bsm.KERNEL_CLUSTER: "softmax_cluster"}.get(
+        kernel, "softmax_persistent (long rows)"), ctas
 
 
-def _long_kernel(st, row_bytes, op="forward"):
-    """The kernel a plan of rows longer than a stage runs on (rows that
-    qualify for groups go to clusters where those are faster; the statistics
-    count them as group rows all the same)."""
-    if st["group_rows"]:
-        return "softmax_group or softmax_cluster"
-    if st["launches"] == 1 and row_bytes <= CLUSTER_ROW_BYTES[op]:
-        return "softmax_cluster"
-    return "softmax_persistent (long rows)"
-
-
-def _moved_factor(st, row_bytes, op="forward"):
+def _moved_factor(ctas, op="forward"):
     """Bytes a plan moves per algorithmic byte: rows split over groups or
     clusters of CTAs read x once; rows streamed twice read it again (forward:
     1.5, backward: 5/3 of the algorithmic bytes at most)."""
-    if _long_kernel(st, row_bytes, op) != "softmax_persistent (long rows)":
+    if ctas > 1:
         return 1.0
     return 1.5 if op == "forward" else 5 / 3
 
@@ -868,6 +859,7 @@ def long_row_sweep(bsm, workload, stream):
             y = torch.empty_like(x)
             plan = bsm.bsm_plan_create(x, y, [R], [C], dtype, bsm.POLICY_DYNAMIC)
             st = plan.stats()
+            kernel, ctas = _long_kernel(bsm, plan)
             plan.close()
 
             def step():
@@ -881,12 +873,12 @@ def long_row_sweep(bsm, workload, stream):
                               "%s %d rows x %d (%d KiB rows)" % (name, R, C, C * es >> 10),
                               "policy": "dynamic", "ms": round(med, 4),
                               "GBps": round(alg / (med * 1e-3) / 1e9, 2),
-                              "group_k": st["group_k"], "launches": st["launches"],
-                              "moved_GBps": round(_moved_factor(st, C * es) * alg / (med * 1e-3) / 1e9, 2)}),
+                              "kernel": kernel, "ctas_per_row": ctas, "launches": st["launches"],
+                              "moved_GBps": round(_moved_factor(ctas) * alg / (med * 1e-3) / 1e9, 2)}),
                   flush=True)
             dy = torch.randn(R * C, device="cuda").to(tdt)
             plan = bsm.bsm_plan_create(y, x, [R], [C], dtype, bsm.POLICY_DYNAMIC, op=bsm.OP_BACKWARD, x2=dy)
-            st = plan.stats()
+            kernel, ctas = _long_kernel(bsm, plan)
             plan.close()
 
             def bstep():
@@ -899,9 +891,9 @@ def long_row_sweep(bsm, workload, stream):
             print(json.dumps({"sweep": True, "op": "backward long rows", "workload":
                               "%s %d rows x %d (%d KiB rows)" % (name, R, C, C * es >> 10),
                               "policy": "dynamic", "ms": round(med, 4),
-                              "GBps": round(alg / (med * 1e-3) / 1e9, 2),
-                              "moved_GBps": round(_moved_factor(st, C * es, "backward") * alg / (med * 1e-3) / 1e9,
-                                                  2)}), flush=True)
+                              "GBps": round(alg / (med * 1e-3) / 1e9, 2), "kernel": kernel, "ctas_per_row": ctas,
+                              "moved_GBps": round(_moved_factor(ctas, "backward") * alg / (med * 1e-3) / 1e9, 2)}),
+                  flush=True)
             del x, y, dy
             torch.cuda.empty_cache()
 
@@ -936,16 +928,15 @@ def time_long_rows(bsm, C, dtype, stream, dev, target_s=0.5):
     alg = 2 * R * C * es
     peak, peak_src = measured_peak()
     gbs = alg / (ms * 1e-3) / 1e9
+    kernel, ctas = _long_kernel(bsm, plan)
     plan.close()
-    kernel = _long_kernel(st, C * es)
     return {"value": round(gbs, 2), "unit": "GB/s", "ms_per_step": round(ms, 5), "steps": steps,
             "dtype": "f32" if dtype == workload.F32 else "bf16",
             "config": {"workload": "%s %d rows x %d (%d KiB rows), 256 MiB, random normal"
                                    % ("fp32" if dtype == workload.F32 else "bf16", R, C, C * es >> 10),
                        "policy": "dynamic", "bytes_per_step": alg,
                        "l2": "inputs larger than L2 (256 MiB vs 129 MB), no flush"},
-            "plan": {"group_k": st["group_k"], "n_groups": st["n_groups"], "launches": st["launches"],
-                     "stage_bytes": st["stage_bytes"]},
+            "plan": {"ctas_per_row": ctas, "launches": st["launches"]},
             "gpu_launches": int(st["launches"]) * steps,
             "roofline": {"bound": "hbm", "achieved": round(gbs, 2), "peak": peak, "unit": "GB/s",
                          "frac": round(gbs / peak, 4),
@@ -954,7 +945,7 @@ def time_long_rows(bsm, C, dtype, stream, dev, target_s=0.5):
                          if st["launches"] == 1 else None,
                          "peak_source": peak_src,
                          "kernel": kernel, "launch_ms": round(ms / max(1, st["launches"]), 5),
-                         "moved_bytes_per_step": int(_moved_factor(st, C * es) * alg)},
+                         "moved_bytes_per_step": int(_moved_factor(ctas) * alg)},
             "clocks": clk.summary(), "device_status": bsm.bsm_device_status()}
 
 
@@ -1053,7 +1044,8 @@ def run_long_rows(args, bsm, ws, rank, dev):
            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
            "data": "synthetic", "config": {"workload": "fp32 %d rows x %d" % (R, C),
                                            "policy": "dynamic", "bytes_per_step": alg},
-           "moved_GBps": round(_moved_factor(st, 4 * C) * alg / (ms * 1e-3) / 1e9, 2),
+           "kernel": _long_kernel(bsm, plan)[0],
+           "moved_GBps": round(_moved_factor(_long_kernel(bsm, plan)[1]) * alg / (ms * 1e-3) / 1e9, 2),
            "gpu_launches": int(st["launches"]) * args.steps,
            "plan": {k: st[k] for k in ("n_items", "long_items", "launches", "stage_bytes", "n_stages",
                                        "group_rows", "group_k", "n_groups")},

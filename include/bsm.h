@@ -430,12 +430,24 @@ int bsm_plan_layout_host(const bsm_plan_desc *d, int32_t n_sm, int64_t smem_opti
 
 /* The patch records as the kernel reads them from the plan's device table
  * (queue policies: in queue order, so that slot k holds patch queue[k]),
- * phase 0 or 1 (the second launch of rows cut into segments).  At most cap
- * records go to out (host, caller-owned); *n_out receives the count.
- * Synchronous (a device-to-host copy).  BSM_ERR_INVALID_ARG for a null plan
- * or n_out, a phase other than 0/1, or a capacity without an array. */
+ * phase 0, 1 (the second launch of rows cut into segments) or 2 (the rows that
+ * bsm_plan_stats counts as group_rows).  At most cap records go to out (host,
+ * caller-owned); *n_out receives the count.  Synchronous (a device-to-host
+ * copy).  BSM_ERR_INVALID_ARG for a null plan or n_out, another phase, or a
+ * capacity without an array. */
 int bsm_plan_device_table(const bsm_plan *plan, int phase, bsm_patch *out, int64_t cap,
                           int64_t *n_out);
+
+/* Which kernel an execute launches for the patches of a phase (as above) and how
+ * many CTAs share a row there.  ctas may be null.  Host-only.
+ * BSM_ERR_INVALID_ARG for a null plan or kernel, or another phase. */
+#define BSM_KERNEL_NONE 0      /* no patch in this phase */
+#define BSM_KERNEL_ROWS 1      /* every row in the registers of up to 32 lanes */
+#define BSM_KERNEL_TEAM 2      /* rows of up to a stage, the longer ones shared by warps */
+#define BSM_KERNEL_STREAM 3    /* the same, and longer rows in chunks */
+#define BSM_KERNEL_GROUP 4     /* each row over a group of CTAs */
+#define BSM_KERNEL_CLUSTER 5   /* each row over a cluster of CTAs */
+int bsm_plan_kernel(const bsm_plan *plan, int phase, int32_t *kernel, int32_t *ctas);
 
 /* Fault injection on one plan, for the library's failure-detection tests
  * (nothing here faults, traps or hangs the GPU).  plan = NULL applies

@@ -153,6 +153,7 @@ def lib():
         "bsm_plan_destroy": ([vp], None),
         "bsm_plan_debug": ([vp, ctypes.c_int, i64], ctypes.c_int),
         "bsm_plan_get_schedule": ([vp, ctypes.POINTER(PlanSchedule)], ctypes.c_int),
+        "bsm_plan_kernel": ([vp, ctypes.c_int, c_i32p, c_i32p], ctypes.c_int),
         "bsm_plan_device_table": ([vp, ctypes.c_int, ctypes.POINTER(Patch), i64, ctypes.POINTER(i64)],
                                   ctypes.c_int),
         "bsm_die_check_read": ([ctypes.c_int, vp, i64, i64, ctypes.POINTER(ctypes.c_int8),
@@ -464,6 +465,16 @@ def bsm_plan_device_table(plan: Plan, phase: int = 0) -> np.ndarray:
     _check(lib().bsm_plan_device_table(plan.handle, phase, buf, n.value, ctypes.byref(n)),
            "bsm_plan_device_table")
     return _patch_array(buf, n.value)
+
+
+KERNEL_NONE, KERNEL_ROWS, KERNEL_TEAM, KERNEL_STREAM, KERNEL_GROUP, KERNEL_CLUSTER = 0, 1, 2, 3, 4, 5
+
+
+def bsm_plan_kernel(plan: Plan, phase: int = 0):
+    """(kernel, CTAs that share a row) of the plan's patches of a phase."""
+    k, c = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib().bsm_plan_kernel(plan.handle, phase, ctypes.byref(k), ctypes.byref(c)), "bsm_plan_kernel")
+    return k.value, c.value
 
 
 def bsm_die_check_read(ptr, nbytes: int, chunk: int, die_of_chunk, invert: bool = False,

@@ -1441,6 +1441,25 @@ int bsm_plan_device_table(const bsm_plan *plan, int phase, bsm_patch *out, int64
     return BSM_OK;
 }
 
+int bsm_plan_kernel(const bsm_plan *plan, int phase, int32_t *kernel, int32_t *ctas)
+{
+    if (!plan || !kernel || phase < 0 || phase > 2)
+        return BSM_ERR_INVALID_ARG;
+    const int64_t n = phase == 0 ? plan->args.n_items : phase == 1 ? plan->n_phase1 : plan->n_group;
+    const int op = phase == 2 ? plan->op_g : plan->kernel_op;
+    int k = BSM_KERNEL_NONE;
+    if (n > 0)
+        k = op == OP_FORWARD_GROUP                                      ? BSM_KERNEL_GROUP
+            : op == OP_FORWARD_CLUSTER || op == OP_BACKWARD_CLUSTER     ? BSM_KERNEL_CLUSTER
+            : op == OP_FORWARD_LONG || op == OP_BACKWARD_LONG           ? BSM_KERNEL_STREAM
+            : op == OP_FORWARD_TEAM || op == OP_BACKWARD_TEAM           ? BSM_KERNEL_TEAM
+                                                                        : BSM_KERNEL_ROWS;
+    *kernel = k;
+    if (ctas)
+        *ctas = k == BSM_KERNEL_NONE ? 0 : k >= BSM_KERNEL_GROUP ? (phase == 2 ? plan->argsg : plan->args).group_k : 1;
+    return BSM_OK;
+}
+
 int bsm_die_check_read(int device, const void *ptr, int64_t bytes, int64_t chunk, const int8_t *die_of_chunk,
                        const int8_t *sm_group, int invert, uint32_t *xor_out, float *ms_out)
 {

@@ -247,3 +247,8 @@ def test_ragged_extent_host_helper():
     assert ext([-8], [1], [4]) == -1
     assert ext([0], [1], [-4]) == -1
     assert ext([(1 << 63) - 8], [1], [16]) == -1               # past INT64_MAX
+
+
+def test_plan_kernel_rejects_null_arguments():
+    k = ctypes.c_int32()
+    assert bsm.lib().bsm_plan_kernel(None, 0, ctypes.byref(k), None) == bsm.ERR_INVALID_ARG

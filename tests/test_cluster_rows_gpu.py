@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 POLICIES = [bsm.POLICY_DYNAMIC, bsm.POLICY_RR, bsm.POLICY_CBMF, bsm.POLICY_CBMF_LB, bsm.POLICY_WHOLE_GPU]
 # 16-byte vectors per row: just past a stage, odd parts, either side of the
 # largest row of two CTAs, then rows of 4, 8 and 16 (forward rows of more than
-# 16384 vectors are those that groups take otherwise)
+# 16384 vectors are those that groups take otherwise: some of these do)
 FWD = [7233, 8195, 14463, 14465, 16383, 28845, 40001, 70003]
 BWD = [3617, 4099, 7231, 7233, 14401, 20003, 29001]
 
@@ -58,6 +58,34 @@ def test_forward_row_lengths(nvec, dtype, flags):
     assert float((s - 1).abs().max()) < (1e-5 if dtype == workload.F32 else 0.02)     # every row written
 
 
+# (vectors a row, rows, CTAs a cluster): rows that fill the clusters' waves
+# better than the groups'
+LARGER = [(28845, 144, 4), (28863, 36, 4), (40002, 30, 8), (57001, 15, 8), (70003, 7, 16), (113001, 7, 16)]
+
+
+@pytest.mark.parametrize("nvec,R,K", LARGER)
+@pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
+@pytest.mark.parametrize("flags", [0, workload.CAUSAL])
+def test_forward_rows_on_larger_clusters(nvec, R, K, dtype, flags):
+    import torch
+    C = nvec * (4 if dtype == workload.F32 else 8)
+    w = workload.uniform("larger", dtype, 1, R, C, 3.0, 0xC20 + nvec + flags, flags).materialize()
+    x = to_device(w.x)
+    p = bsm.bsm_plan_create(x, x, w.rows, w.cols, dtype, bsm.POLICY_DYNAMIC, flags=flags)
+    kernel = bsm.bsm_plan_kernel(p, 2)
+    p.close()
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152 and not (dtype == workload.BF16 and nvec == 40002):
+        assert kernel == (bsm.KERNEL_CLUSTER, K)
+    ys = [run(w, x, p) for p in POLICIES]
+    torch.cuda.synchronize()
+    assert bsm.bsm_device_status() == 0, bsm.bsm_device_debug()
+    for y in ys[1:]:
+        assert torch.equal(bits(y), bits(ys[0]))
+    check_rows_against_oracle(w, to_host(ys[0]), sample_rows(w, 7, nvec))
+    s = ys[0].view(-1, C).double().sum(1)
+    assert float((s - 1).abs().max()) < (1e-5 if dtype == workload.F32 else 0.02)     # every row written
+
+
 @pytest.mark.parametrize("nvec", BWD)
 @pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
 def test_backward_row_lengths(nvec, dtype):
@@ -69,6 +97,9 @@ def test_backward_row_lengths(nvec, dtype):
     g = torch.Generator(device="cuda").manual_seed(nvec)
     y = torch.softmax(torch.randn(R, C, generator=g, device="cuda") * 3, -1).to(t)
     dy = torch.randn(R, C, generator=g, device="cuda").to(t)
+    p = bsm.bsm_plan_create(y, dy, [R], [C], dtype, bsm.POLICY_DYNAMIC, op=bsm.OP_BACKWARD, x2=dy)
+    assert bsm.bsm_plan_kernel(p)[0] == bsm.KERNEL_CLUSTER
+    p.close()
     outs = []
     for p in POLICIES:
         dx = torch.full_like(y, float("nan"))
@@ -156,8 +187,8 @@ def test_backward_withheld_stage_and_corrupted_record():
     p.close()
 
 
-@pytest.mark.parametrize("rows,C", [(0, 40000), (64, 262144)])      # clusters of 2, of 16
-def test_forward_withheld_stage(rows, C):
+@pytest.mark.parametrize("rows,C,K", [(0, 40000, 2), (64, 262144, 16)])
+def test_forward_withheld_stage(rows, C, K):
     """Every wait of every CTA ends, with copies and other CTAs' partials in
     flight; the next execute is right."""
     import time
@@ -167,6 +198,7 @@ def test_forward_withheld_stage(rows, C):
     x = to_device(w.x)
     y = torch.zeros_like(x)
     p = bsm.bsm_plan_create(x, y, w.rows, w.cols, w.dtype, bsm.POLICY_DYNAMIC)
+    assert bsm.bsm_plan_kernel(p, 2 if rows else 0) == (bsm.KERNEL_CLUSTER, K)
     for _ in range(3):
         bsm.bsm_plan_debug(p, bsm.DEBUG_WITHHOLD_STAGE, 20_000_000)      # 0.02 s waits
         t0 = time.time()

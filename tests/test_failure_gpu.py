@@ -85,8 +85,8 @@ def test_corrupted_patch_is_skipped_with_bounds_status():
 
 
 def _w_long():
-    """Two waves of rows just over a stage: the one-launch long-row path
-    (rows staged whole between their passes)."""
+    """Two waves of rows just over a stage: whole rows in one launch (over
+    clusters of two CTAs)."""
     import torch
     n_sm = torch.cuda.get_device_properties(0).multi_processor_count
     C = bsm.bsm_max_row_bytes() // 4 + 64
@@ -186,6 +186,7 @@ def test_withheld_stage_in_a_group_launch_times_out_and_context_survives():
     bsm.bsm_device_status_clear()
     p = bsm.bsm_plan_create(x, y, w.rows, w.cols, w.dtype, bsm.POLICY_DYNAMIC)
     assert p.stats()["group_rows"] == 19          # 19 of the 25 groups of 6 CTAs on 152 SMs
+    assert bsm.bsm_plan_kernel(p, 2)[0] == bsm.KERNEL_GROUP
     bsm.bsm_plan_debug(p, bsm.DEBUG_WITHHOLD_STAGE, 100_000_000)      # 0.1 s waits
     t0 = time.time()
     p.execute()
@@ -246,7 +247,7 @@ def test_group_rows_with_one_warp_that_reads_results_late():
     bsm.bsm_device_status_clear()
     bsm.bsm_softmax(x, y, 1, 45, 524288, w.dtype, bsm.POLICY_DYNAMIC)
     p = bsm.bsm_plan_create(x, late, w.rows, w.cols, w.dtype, bsm.POLICY_DYNAMIC)
-    assert p.stats()["group_rows"] == 45
+    assert p.stats()["group_rows"] == 45 and bsm.bsm_plan_kernel(p, 2)[0] == bsm.KERNEL_GROUP
     bsm.bsm_plan_debug(p, bsm.DEBUG_LAG_WARP)
     bsm.bsm_set_device_checks(True)
     p.execute()

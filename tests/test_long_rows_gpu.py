@@ -1,9 +1,10 @@
 """Rows longer than one shared-memory stage against the oracle, under every
 policy, bit-identical across policies: forward rows split over groups of CTAs
-(each CTA stages one part; the group exchanges (max, sum) partials), and the
+(each CTA stages one part; the group exchanges (offset, sum) partials) and the
 paths that stream a row twice in chunks (a running max and rescaled sum,
-then the output): few long rows cut into segments over two launches, and
-the backward pass."""
+then the output): few long rows cut into segments over two launches, rows
+beside short ones.  Batches that go to clusters of CTAs instead have their own
+tests; those here that do say so."""
 import numpy as np
 import pytest
 
@@ -90,11 +91,11 @@ def test_non_finite_long_rows():
 
 @pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
 def test_many_long_rows_stream_whole_rows_in_one_launch(dtype):
-    """With at least two waves of rows too short for a group each row is one
-    segment that one CTA streams in a single launch (fewer rows are cut into
-    segments over two launches).  Rows just over the cap get three stages of
-    half a row: a row (two chunks) stays staged for its second pass.  Against
-    the oracle, all policies bit-identical."""
+    """With at least two waves of rows too short for a group each row is whole,
+    in a single launch (fewer rows are cut into segments over two launches), on
+    a cluster of two CTAs; beside a short row, on one CTA.  Rows just over the
+    cap get three stages of half a row: there a row (two chunks) stays staged
+    for its second pass.  Against the oracle, all policies bit-identical."""
     import torch
     es = 4 if dtype == workload.F32 else 2
     limit = bsm.bsm_max_row_bytes() // es
@@ -107,9 +108,18 @@ def test_many_long_rows_stream_whole_rows_in_one_launch(dtype):
     assert st["long_items"] == R and st["launches"] == 1 and st["n_items"] == R
     assert st["group_rows"] == 0
     assert st["n_stages"] == 3 and 2 * st["stage_bytes"] >= C * es
+    assert bsm.bsm_plan_kernel(p) == (bsm.KERNEL_CLUSTER, 2)
     p.close()
     y = _all(w, x)
     check_all_against_oracle(w, to_host(y))
+    rows, cols = np.array([R, 1], np.int32), np.array([C, 64], np.int32)
+    w = workload.Workload("many long, one short", dtype, rows, cols, np.array([0, R * C], np.int64), 0,
+                          0x10A8 + dtype, 3.0).materialize()
+    x = to_device(w.x)
+    p = bsm.bsm_plan_create(x, x, w.rows, w.cols, dtype, bsm.POLICY_DYNAMIC)
+    assert p.stats()["n_stages"] == 3 and bsm.bsm_plan_kernel(p) == (bsm.KERNEL_STREAM, 1)
+    p.close()
+    check_all_against_oracle(w, to_host(_all(w, x)))
     assert bsm.bsm_device_status() == 0
 
 
@@ -122,6 +132,7 @@ def test_few_long_rows_are_segmented_over_two_launches():
     p = bsm.bsm_plan_create(x, torch.empty_like(x), w.rows, w.cols, workload.F32, bsm.POLICY_DYNAMIC)
     st = p.stats()
     assert st["long_items"] == 3 and st["launches"] == 2 and st["n_items"] > 3
+    assert bsm.bsm_plan_kernel(p) == bsm.bsm_plan_kernel(p, 1) == (bsm.KERNEL_STREAM, 1)
     p.close()
     y = _all(w, x)
     check_all_against_oracle(w, to_host(y))
@@ -130,12 +141,12 @@ def test_few_long_rows_are_segmented_over_two_launches():
 @pytest.mark.parametrize("dtype", [workload.F32, workload.BF16])
 @pytest.mark.parametrize("chunks,flags", [(3, workload.CAUSAL), (4, 0)])
 def test_many_long_rows_of_several_chunks(dtype, chunks, flags):
-    """Two waves of rows of three and four stages' length: the three-chunk
-    rows (four parts of 64 KiB at most: too few for a group) are streamed
-    whole by one CTA each, starting the second pass on the chunk still
-    staged and running backwards; the four-chunk rows go to groups of eight
-    CTAs.  Under the causal mask most of every row is masked (the row index is
-    below the column count)."""
+    """Two waves of rows of three and four stages' length, on clusters of four
+    CTAs (the four-chunk rows would fill groups of CTAs too).  The three-chunk
+    rows beside a short one are streamed whole by one CTA each, starting the
+    second pass on the chunk still staged and running backwards.  Under the
+    causal mask most of every row is masked (the row index is below the column
+    count)."""
     import torch
     es = 4 if dtype == workload.F32 else 2
     limit = bsm.bsm_max_row_bytes() // es
@@ -148,9 +159,20 @@ def test_many_long_rows_of_several_chunks(dtype, chunks, flags):
     st = p.stats()
     assert st["long_items"] == R and st["launches"] == 1
     assert st["group_rows"] == (0 if chunks == 3 else R)
+    if n_sm == 152:
+        assert bsm.bsm_plan_kernel(p, 0 if chunks == 3 else 2) == (bsm.KERNEL_CLUSTER, 4)
     p.close()
     y = _all(w, x)
     check_all_against_oracle(w, to_host(y))
+    if chunks == 3:
+        rows, cols = np.array([R, 1], np.int32), np.array([C, 64], np.int32)
+        w = workload.Workload("three chunks, one short", dtype, rows, cols, np.array([0, R * C], np.int64), flags,
+                              0x10B8 + dtype, 3.0).materialize()
+        x = to_device(w.x)
+        p = bsm.bsm_plan_create(x, x, w.rows, w.cols, dtype, bsm.POLICY_DYNAMIC, flags=flags)
+        assert bsm.bsm_plan_kernel(p) == (bsm.KERNEL_STREAM, 1)
+        p.close()
+        check_all_against_oracle(w, to_host(_all(w, x)))
     assert bsm.bsm_device_status() == 0
 
 
@@ -172,9 +194,10 @@ def test_group_rows_every_group_size(case, flags):
     p = bsm.bsm_plan_create(x, torch.empty_like(x), w.rows, w.cols, dtype, bsm.POLICY_DYNAMIC,
                             flags=flags)
     st = p.stats()
+    kernel = bsm.bsm_plan_kernel(p, 2)
     p.close()
     if n_sm == 152:
-        assert st["group_k"] == k
+        assert st["group_k"] == k and kernel == (bsm.KERNEL_GROUP, k)
     assert st["group_rows"] == R and st["launches"] == 1
     y = _all(w, x)
     check_all_against_oracle(w, to_host(y))
@@ -182,10 +205,17 @@ def test_group_rows_every_group_size(case, flags):
 
 
 def test_group_rows_beside_short_rows_two_launches():
-    """A ragged batch: short rows (one launch of the regular kernel) and a
-    wave of rows split over groups (a second, cooperative launch), slices
-    interleaved and not contiguous."""
-    rows = np.array([3, 20, 5, 19, 1, 0, 7], np.int32)
+    """A ragged batch: short rows (one launch of the regular kernel) and rows
+    that qualify for groups (a second launch), slices interleaved and not
+    contiguous: 39 of them on clusters of 8, 22 (two waves of 11 groups, which
+    clusters would take three for) on groups, that launch cooperative."""
+    import torch
+    for k, kernel in ((19, bsm.KERNEL_CLUSTER), (2, bsm.KERNEL_GROUP)):
+        _short_and_group_rows(k, kernel, torch.cuda.get_device_properties(0).multi_processor_count)
+
+
+def _short_and_group_rows(k, kernel, n_sm):
+    rows = np.array([3, 20, 5, k, 1, 0, 7], np.int32)
     cols = np.array([512, 200000, 64, 180000, 4096, 64, 2048], np.int32)
     sizes = rows.astype(np.int64) * cols
     off = np.concatenate([[0], np.cumsum(sizes + 64)[:-1]]).astype(np.int64)
@@ -196,8 +226,11 @@ def test_group_rows_beside_short_rows_two_launches():
     p = bsm.bsm_plan_create(x, torch.empty_like(x), w.rows, w.cols, workload.F32,
                             bsm.POLICY_DYNAMIC, offsets=w.offsets)
     st = p.stats()
+    kernels = bsm.bsm_plan_kernel(p)[0], bsm.bsm_plan_kernel(p, 2)[0]
     p.close()
-    assert st["group_rows"] == 39 and st["launches"] == 2
+    if n_sm == 152:
+        assert kernels == (bsm.KERNEL_TEAM, kernel)
+    assert st["group_rows"] == 20 + k and st["launches"] == 2
     y = _all(w, x)
     check_all_against_oracle(w, to_host(y))
     assert bsm.bsm_device_status() == 0
@@ -221,6 +254,8 @@ def test_non_finite_group_rows():
     p = bsm.bsm_plan_create(xd, torch.empty_like(xd), w.rows, w.cols, workload.F32,
                             bsm.POLICY_DYNAMIC)
     assert p.stats()["group_rows"] == R
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert bsm.bsm_plan_kernel(p, 2) == (bsm.KERNEL_GROUP, 7)
     p.close()
     y = _all(w, xd)
     yh = to_host(y).reshape(R, C)
