@@ -384,9 +384,11 @@ ClusterChoice choose_clusters(const std::vector<Item> &items, int dtype, bool bw
 {
     const ClusterChoice none;
     ClusterChoice c;
-    int64_t lmax = 0;
-    for (const Item &it : items)
+    int64_t lmax = 0, total = 0;
+    for (const Item &it : items) {
         lmax = std::max<int64_t>(lmax, it.C);
+        total += it.C;
+    }
     const int64_t arrays = bwd ? 2 : 1, nv = (lmax * esize(dtype) + 15) / 16;
     for (int K : {2, 4, 8, 16}) {
         c.K = K;
@@ -396,6 +398,16 @@ ClusterChoice choose_clusters(const std::vector<Item> &items, int dtype, bool bw
             break;
     }
     if (lmax == 0 || c.n_stages < 2)
+        return none;
+    // A batch of unequal rows: the longest sets K, and a row on a cluster takes
+    // about 1.7 us however short, so the mean part must be a third of what a
+    // stage holds, backward half of it.  One row of the longest among others, one
+    // CTA a row against clusters, us: backward fp32, longest 800 KiB (K = 16),
+    // others 58 KiB 83 / 552, 400 KiB 105 / 101, 448 KiB 113 / 99; 200 KiB (4),
+    // 58 KiB 79 / 113, 112 KiB 79 / 74; forward fp32 250 KiB (4), 115 KiB 62 / 68,
+    // 152 KiB 68 / 58; bf16 146 KiB 74 / 68.  (Groups lose more to unequal rows.)
+    const int64_t mean_part = total / static_cast<int64_t>(items.size()) * esize(dtype) / c.K;
+    if (group_k == 0 && mean_part < (bwd ? 28 : 36) * 1024)
         return none;
     if (cluster_units(dtype, bwd, c.K, n_sm, static_cast<int>(cluster_header(c.K) + c.n_stages * c.stage), &c.units)) {
         cudaGetLastError();

@@ -215,3 +215,30 @@ def test_forward_withheld_stage(rows, C, K):
         check_rows_against_oracle(w, to_host(y), sample_rows(w, 16, 1))
         assert float((y.view(R, C).double().sum(1) - 1).abs().max()) < 1e-5
     p.close()
+
+
+@pytest.mark.parametrize("others,kernel", [(58, bsm.KERNEL_STREAM), (500, bsm.KERNEL_CLUSTER)])
+def test_backward_rows_beside_one_much_longer(others, kernel):
+    """One row of 800 KiB sets the size of the clusters: rows that leave them
+    nearly empty stay with one CTA each."""
+    import torch
+    n = 2 * torch.cuda.get_device_properties(0).multi_processor_count + 6
+    cols = np.full(n, others * 256, np.int32)
+    cols[n // 3] = 800 * 256
+    rows = np.ones(n, np.int32)
+    off = np.concatenate([[0], np.cumsum(cols.astype(np.int64))[:-1]])
+    total = int(cols.astype(np.int64).sum())
+    dy = torch.randn(total, device="cuda")
+    y = torch.rand(total, device="cuda") / 1000
+    dx = torch.full_like(y, float("nan"))
+    p = bsm.bsm_plan_create(y, dx, rows, cols, bsm.F32, bsm.POLICY_DYNAMIC, op=bsm.OP_BACKWARD, x2=dy)
+    assert bsm.bsm_plan_kernel(p)[0] == kernel
+    p.execute()
+    torch.cuda.synchronize()
+    assert bsm.bsm_device_status() == 0
+    for o, c in zip(off.tolist(), cols.tolist()):
+        yd, gd = y[o:o + c].double(), dy[o:o + c].double()
+        ref = yd * (gd - (yd * gd).sum())
+        # (two roundings of 2^-24 and the dot product's error, a few 2^-24 of it)
+        assert float((dx[o:o + c].double() - ref).norm()) <= 4e-7 * float(ref.norm())
+    p.close()
