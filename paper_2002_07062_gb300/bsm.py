@@ -267,7 +267,7 @@ def _stream(s) -> Optional[int]:
 
 
 def _np(a, dt):
-    if type(a) is np.ndarray and a.dtype == dt and a.flags.c_contiguous:
+    if type(a) is np.ndarray and a.ndim and a.dtype == dt and a.flags.c_contiguous:
         return a
     return np.ascontiguousarray(np.asarray(a), dtype=dt)
 

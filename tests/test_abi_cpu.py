@@ -252,3 +252,9 @@ def test_ragged_extent_host_helper():
 def test_plan_kernel_rejects_null_arguments():
     k = ctypes.c_int32()
     assert bsm.lib().bsm_plan_kernel(None, 0, ctypes.byref(k), None) == bsm.ERR_INVALID_ARG
+
+
+def test_array_of_no_dimension_is_one_slice():
+    for one in (np.array(8, np.int32), np.int32(8), 8, [8]):
+        lay = bsm.bsm_plan_layout_host(one, one, bsm.F32, bsm.POLICY_DYNAMIC, 152, 232448)
+        assert [(int(p["cols"]), int(p["nrows"])) for p in lay["phase0"]] == [(8, 1)] * 8
