@@ -55,7 +55,8 @@
  *     shared-memory stage, by one warp or, past 2 KiB, by a team of up to 16.
  *     Batches of longer rows, at least two per SM, run over clusters of 2, 4, 8
  *     or 16 SMs: each takes a part of the row in one of its stages and every
- *     element is read once (rows of up to 1.7 MiB, 880 KiB backward).  Other
+ *     element is read once (rows of up to 1.7 MiB, 880 KiB backward; not where
+ *     the batch's mean row would leave the parts nearly empty).  Other
  *     longer rows go through the stages in chunks, in two passes -- a running
  *     maximum and rescaled sum (backward: the dot product), then the output --
  *     and are read again, all but their last chunk (a row of two chunks whose

@@ -326,8 +326,8 @@ int choose_groups(const std::vector<SliceView> &slices, int es, int n_sm, int64_
     // fewest members with full parts move the most bytes per exchange, even
     // when n_sm / K groups leave SMs idle.  Measured on GB300 (256 MiB of
     // rows, GB/s; with the consumer warps reading the exchange words
-    // themselves -- since a warp of its own does, 1 MiB rows take 5472 (fp32)
-    // and 5136 (bf16), and batches that clusters serve better go there, see
+    // themselves -- since a warp of its own does, 1 MiB rows run at 5496 (fp32)
+    // and 5212 (bf16), and batches that clusters serve better go there, see
     // choose_clusters): fp32 1 MiB rows K = 16 (9 groups) 4746 against K = 19 (8
     // groups) 4347, 17 and 18 lower still; bf16 1 MiB the same (3952 against
     // 3635); bf16 512 KiB K = 8 4139 against K = 16 2612 and K = 19 2316;
@@ -367,10 +367,10 @@ int choose_groups(const std::vector<SliceView> &slices, int es, int n_sm, int64_
 // Why the smallest: the larger the cluster, the fewer SMs take part (clusters
 // share a GPC: 76 of 2, 36 of 4, 15 of 8, 7 of 16 are resident at once, 152,
 // 144, 120 and 112 SMs), and a part of 57 to 113 KiB runs like a row of that
-// length.  Against groups, GB/s over 256 MiB: fp32 320 KiB rows (K = 4) 6512 /
-// 5680, 512 KiB (8) 6291 / 5668, 768 KiB (8) 6372 / 5775, 1 MiB (16) 5671 /
-// 5472, 1.5 MiB (16) 5885 / 5185; bf16 384 KiB (4) 6410 / 5360, 512 KiB (8) 5234
-// / 5343, 1 MiB (16) 4710 / 5136 (a bf16 part costs as many exponentials as an
+// length.  Against groups, GB/s over 256 MiB: fp32 384 KiB rows (K = 4) 6465 /
+// 5626, 512 KiB (8) 6247 / 5695, 768 KiB (8) 6352 / 5555, 1 MiB (16) 5648 /
+// 5496, 1.5 MiB (16) 5874 / 5614; bf16 384 KiB (4) 6393 / 5452, 512 KiB (8) 5234
+// / 5512, 1 MiB (16) 4710 / 5212 (a bf16 part costs as many exponentials as an
 // fp32 part twice as long: on 112 SMs they bound it).  Against one CTA a row,
 // backward: 256 KiB (8) 5900 / 5344, 384 KiB (8) 6660 / 4700, 768 KiB (16) 6100 /
 // 4150.
@@ -417,7 +417,11 @@ ClusterChoice choose_clusters(const std::vector<Item> &items, int dtype, bool bw
     if (c.units * c.K * 8 < n_sm * 5)          // three eighths of the SMs would idle: another device's clusters
         return none;
     if (group_k > 0) {
-        // the two measured rates (TB/s, all units busy) and the rows' waves
+        // the rows' waves, and the time of one: the bytes that `at` clusters (the
+        // measured device's) or its groups hold over the rate measured with all
+        // of them busy (TB/s).  Past 12 members the groups' rates fall with their
+        // number (fp32 5.5 and 5.6 for 16 and 24, 5.15 for 32; bf16 5.2, 5.3, 4.8):
+        // 5.2 and 5.0 lie between
         const double n = static_cast<double>(items.size()), f32 = dtype == BSM_F32;
         const double rate = c.K <= 4 ? 6.4 : c.K == 8 ? (f32 ? 6.3 : 5.3) : (f32 ? 5.7 : 4.75);
         const double at = c.K == 2 ? 76 : c.K == 4 ? 36 : c.K == 8 ? 15 : 7;

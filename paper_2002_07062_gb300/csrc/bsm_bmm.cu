@@ -17,8 +17,8 @@
 //                   one output row per thread), round, write 32 rows x 128
 //                   bytes at a time into a 128-byte-swizzled shared buffer
 //                   (conflict-free), and one lane stores it with a 2-D TMA
-//                   tensor store; two buffers per warp, so the next unit is
-//                   converted while the last one drains.
+//                   tensor store; usually two to four buffers per warp, so the
+//                   next unit is converted while the last one drains.
 // The accumulators are double-buffered so the epilogue of a tile overlaps the
 // MMAs of the next.  Warps 0 and 1 run their loops as a whole, the copies and
 // MMAs under an election (see elect_one).  Products bound by the tensor cores
@@ -679,8 +679,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 // then takes 32 KiB per CTA (BN = 256), so six of them fit beside the store
 // buffers where a 128 x 256 tile has three of 48 KiB, and an SM takes 64
 // bytes a cycle from L2 at the full tensor rate instead of 96.  8 x 2048^3,
-// bf16: 122.9 us (1.12 PFLOP/s) before, 104 with the warp-wide issue alone
-// (elect_one), 80.2 (1.71 PFLOP/s) on pairs; the tensor cores' own time is 60.
+// bf16, launches back to back: 122.9 us (1.12 PFLOP/s) before, 104 with the
+// warp-wide issue alone (elect_one), 81.0 (1.70 PFLOP/s) on pairs; 72.3 at the
+// card's measured bf16 rate.  One call on cold operands takes 90 to 93 us.
 //
 // Roles as in bmm_persistent, in both CTAs; what differs:
 //   - the first CTA claims the pair's tiles and posts each to both CTAs' rings

@@ -399,16 +399,16 @@ int run_plan(GemmPlan *p, bsm_stream_t stream)
 
 // Whether the product runs on tiles of 256 x bn over pairs of CTAs: where the
 // tensor cores rather than HBM bound it, and a CTA has enough of them.  Pairs
-// against single CTAs (us, bf16 out, same box): 8 x 2048^3 80.2 / 104, 64 x
-// 1024^3 115 / 132, 64 x (1024 x 512)(512 x 1024) 56.7 / 73.0, 32 x (1024 x
-// 2048)(2048 x 384) 53.6 / 71.2, 1 x 2048^3 17.2 / 19.0.
+// against single CTAs (us back to back, bf16 out, same box): 8 x 2048^3 81.0 /
+// 104.2, 64 x 1024^3 93.1 / 120.4, 64 x (1024 x 512)(512 x 1024) 56.8 / 73.1, 32 x
+// (1024 x 2048)(2048 x 384) 53.3 / 71.4, 1 x 2048^3 16.3 / 16.0.
 // - Fewer than 120 operations a byte (about 0.4 of the ratio of the two
 //   peaks) are bound by HBM, where a pair only adds its fixed cost: 300 x (256 x
 //   512)(512 x 128) 26.8 / 25.3, 64 x (1024 x 128)(128 x 1024) 45 / 36.7.
 // - Under 1280 of K per SM (tiles x K / SMs) a pair's start, about 1.5 us
 //   longer, is not made up: 19 x (512 x 1024)(1024 x 512) 12.3 / 11.4, 2048 x
 //   2048 x 1024 12.7 / 11.0 -- but a single long tile is: 1024 x 1024 x 4096
-//   24.8 / 28.9.
+//   23.6 / 25.0.
 // Results do not depend on it (the same order of the K blocks in one
 // accumulator).
 bool use_pair(int n_sm, int64_t B, int64_t M, int64_t N, int64_t K, int bn, bool out_bf16)

@@ -141,7 +141,7 @@ struct KernelArgs {
     int32_t group_k;            // CTAs per group (2..kMaxGroup; per cluster, OP_*_CLUSTER); the grid is n_groups * group_k
     int32_t n_groups;
     unsigned long long *ring;   // n_groups x kGroupRing claim words
-    unsigned long long *xch;    // n_groups x kGroupSlots x group_k x 2 tagged words: max, sum
+    unsigned long long *xch;    // n_groups x kGroupSlots x group_k x 2 tagged words: offset, sum
 };
 
 // Test-only fault injection (bsm_plan_debug).
@@ -170,7 +170,7 @@ struct GemmArgs {
     uint32_t *heads;
     const int8_t *sm_die;
     int32_t n_stages;
-    int32_t epi_bufs;               // 2..4 store buffers per epilogue warp
+    int32_t epi_bufs;               // 1..4 store buffers per epilogue warp
     int32_t kbs;                    // K blocks of 64 per stage (1, 2 or 4)
     int32_t identity;               // items in natural order: computed, not read
     int32_t tiles_m, tiles_n;       // row / column blocks per slice

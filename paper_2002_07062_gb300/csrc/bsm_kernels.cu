@@ -1797,8 +1797,8 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
                 // the row's partials, left by phase 0: dot products added in slot
                 // order, (maximum, sum) pairs over the lanes and a fixed tree
                 // (every segment of the row, on any SM, gets the same result).
-                // One pair after another by every thread (152 a row here) was
-                // a fifth of the time of 8 rows of 16 MiB: 91.9 us against 71.8
+                // One pair after another by every thread took 20 of 92 us on 8
+                // fp32 rows of 16 MiB (109 segments each)
                 const float *pp = a.partials + 2 * static_cast<int64_t>(mt.part_first);
                 if constexpr (kBwd) {
                     float dot = 0.0f;
@@ -1986,11 +1986,10 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
 // writing the previous row (held in registers), so the exchange overlaps
 // work.  fp32 1 MiB rows (K = 16) ran at 4811 GB/s when every consumer warp
 // polled for itself, with a running maximum rescaled per chunk and the
-// producer's chain of round trips (see there), and run at 5472; bf16 4137 and
-// 5136; without the row between, 4180; with the exchange warp publishing as
-// well (so behind its polling), 4830.  What is left is the stage held through
-// a partial and a write (5400 without any exchange).  The group's
-// rank-0 CTA claims the rows (any policy's puller, with the group as the
+// producer's chain of round trips (see there), and run at 5496; bf16 4137 and
+// 5212.  On the way, without the row between, 4180; with the exchange warp
+// publishing as well (so behind its polling), 4830.  The group's rank-0 CTA
+// claims the rows (any policy's puller, with the group as the
 // unit) and announces them to its members through a ring of claim words.
 // The launch is cooperative, so every member of a group is resident and each
 // wait ends; every wait is bounded all the same.

@@ -1,7 +1,7 @@
 """Batches of rows longer than a stage that clusters of 2 to 16 CTAs share,
 against the oracle (sampled rows) and bit-identical across policies: the
 lengths at which the cluster grows and parts of unequal length, the causal
-mask across parts, NaN, +inf, all -inf and masks of the type's lowest value,
+mask across parts, NaN, +inf, all -inf and finite masks, unequal rows,
 the self-checking kernel, a withheld stage and a corrupted record."""
 import numpy as np
 import pytest

@@ -1,8 +1,8 @@
-"""Rows that teams of 1, 2, 4, 8 or 16 warps share (past 4 KiB fp32, 2 KiB
-bf16, up to one stage) against the oracle, bit-identical across policies: the
+"""Rows that teams of 1, 2, 4, 8 or 16 warps share (past 2 KiB, up to one
+stage) against the oracle, bit-identical across policies: the
 lengths at which the team, the vectors a lane holds, or the part left in the
 stage changes; batches that mix team sizes (and long rows); rows with NaN,
-+inf, all -inf, and masks of the type's lowest value; and the bounded wait."""
++inf, all -inf, and finite masks; and the bounded wait."""
 import numpy as np
 import pytest
 
