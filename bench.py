@@ -465,7 +465,8 @@ def main():
     status = bsm.bsm_device_status()
     # context on this very box: a plain device-to-device copy of the same
     # bytes (x into y: one read and one write of every element), timed the
-    # same way; the roofline's peak stays the measured copy bandwidth
+    # same way; the roofline's peak stays the copy bandwidth of the measured
+    # peaks file
     copy_reps = 50
 
     def copy_step():

@@ -405,7 +405,9 @@ ClusterChoice choose_clusters(const std::vector<Item> &items, int dtype, bool bw
     // CTA a row against clusters, us: backward fp32, longest 800 KiB (K = 16),
     // others 58 KiB 83 / 552, 400 KiB 105 / 101, 448 KiB 113 / 99; 200 KiB (4),
     // 58 KiB 79 / 113, 112 KiB 79 / 74; forward fp32 250 KiB (4), 115 KiB 62 / 68,
-    // 152 KiB 68 / 58; bf16 146 KiB 74 / 68.  (Groups lose more to unequal rows.)
+    // 152 KiB 68 / 58; bf16 146 KiB 74 / 68.  (Batches that qualify for groups are
+    // not held to it: there too unequal rows cost clusters less, fp32 800 KiB among
+    // 115 KiB 267 / 396, but for rows of about 1 MiB, on 16 CTAs either way, 592 / 476.)
     const int64_t mean_part = total / static_cast<int64_t>(items.size()) * esize(dtype) / c.K;
     if (group_k == 0 && mean_part < (bwd ? 28 : 36) * 1024)
         return none;

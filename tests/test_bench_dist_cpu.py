@@ -42,7 +42,7 @@ def test_two_rank_max_time_and_job_throughput():
 
 
 def test_reference_arm_under_torchrun_prints_one_line():
-    """`bench.py --impl reference` launched like the driver's N = 2 run: rank 0
+    """`bench.py --impl reference` launched with two ranks: rank 0
     times the oracle and prints the one JSON line, rank 1 exits 0 without work."""
     import json
     import subprocess
