@@ -913,10 +913,14 @@ __device__ __forceinline__ int consume_stage_bwd(const unsigned char *sbuf, int 
 // one launch, pass 1 starts on the last chunk, still in its stage, and takes
 // the others in reverse order.
 
+// The exponents' offset of the streamed rows: m * log2 e itself, no lower than the
+// lowest float (see exp_offset; for a mask of the type's lowest value it would be
+// -inf, and a -inf beside it NaN).
+__device__ __forceinline__ float long_offset(float m) { return fmaxf(m * kLog2e, kLowest); }
+
 // A sum s of 2^((v - m) log2 e) once a value above m is the maximum: one that
 // overflowed counts nothing.  It does where m is a finite mask such as -1e10 (see
-// half_share; below -2.3e38 m log2 e itself is infinite), and inf * 2^(far below
-// 0) would be NaN.
+// half_share), and inf * 2^(far below 0) would be NaN.
 __device__ __forceinline__ float finite_or_none(float s) { return s == INFINITY ? 0.0f : s; }
 
 // A sum s of maximum m as part of one of maximum M >= m.
@@ -963,14 +967,14 @@ __device__ __forceinline__ void long_chunk(const unsigned char *sbuf, const Stag
                     m_l = vm;
                 }
             }
+            // the exponentials in fp32 pairs (the same bits as one at a time);
             // while the running max is still -inf every value seen is -inf (or
-            // NaN): it adds 0 (NaN), as a masked vector does; otherwise the
-            // exponentials in fp32 pairs (the same bits as one at a time)
-            if (masked || m_l == -INFINITY) {
-                vec_exp<EPV>(v, m_l * kLog2e, true);
+            // NaN) and adds 0 (NaN), as a masked vector does
+            if (masked) {
+                vec_exp<EPV>(v, 0.0f, true);
                 s_l += tree_sum<EPV>(v);
             } else {
-                s_l += vec_exp_sum_pairs<EPV>(v, m_l * kLog2e);
+                s_l += vec_exp_sum_pairs<EPV>(v, long_offset(m_l));
             }
         } else {
             vec_exp<EPV>(v, mL, masked);
@@ -1812,7 +1816,7 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
                     m = warp_max(m);
                     for (int k = lane; k < mt.part_count; k += 32)
                         sum += ms_share(pp[2 * k], pp[2 * k + 1], m);
-                    long_mL = m * kLog2e;
+                    long_mL = long_offset(m);
                     long_inv = __frcp_rn(group_sum<32>(sum));
                 }
             }
@@ -1880,7 +1884,7 @@ __global__ void __launch_bounds__(kThreads, 1) softmax_persistent(const KernelAr
                     if constexpr (kBwd) {
                         long_mL = m;
                     } else {
-                        long_mL = m * kLog2e;
+                        long_mL = long_offset(m);
                         long_inv = __frcp_rn(sum);
                     }
                     if (!mt.resident) {

@@ -177,7 +177,7 @@ FINITE_MASKS = [-1e9, -1e10, -1e30, None]       # None: the type's lowest value
 def check_finite_masks(mask, dtype, R, C, short_row=False):
     """Rows of which all but a few places hold a finite mask value: a head, a
     tail, a middle piece or alternate elements are left, so that whole warps
-    and whole parts of a row see the mask only.  Against float64.  short_row
+    and whole parts of a row see the mask only; one has -inf between the masks.  Against float64.  short_row
     adds a slice of one short row, beside which long rows go to one CTA each."""
     import torch
     t = torch.float32 if dtype == workload.F32 else torch.bfloat16
@@ -191,6 +191,8 @@ def check_finite_masks(mask, dtype, R, C, short_row=False):
     x[5, ::2] = mask
     x[6, :C // 2] = mask
     x[6, C // 2 + 8:] = mask
+    x[7, :C // 2] = mask
+    x[7, 3:C // 2:7] = -float("inf")
     if short_row:
         x = torch.cat([x.view(-1), x[0, :64]])
         y = torch.full_like(x, -1.0)
